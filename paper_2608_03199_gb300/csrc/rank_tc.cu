@@ -133,8 +133,8 @@ struct RankModeT {
     __device__ static const float *b_row(const Args &a, const Tile &T, int64_t r) {
         return r < T.nb ? a.C + (T.c0 + r) * a.d : nullptr;
     }
-    __device__ static const unsigned char *b_block(const Args &a, const Tile &T, int ch) {
-        return a.tc_cent + (T.c0 / kTcRows + ch) * (int64_t)((a.d + 63) / 64) * kTcBlockBytes;
+    __device__ static const unsigned char *b_block(const Args &a, const Tile &T) {
+        return a.tc_cent + (T.c0 / kTcRows) * (int64_t)((a.d + 63) / 64) * kTcBlockBytes;
     }
     struct Epi {
         bool valid;

@@ -231,8 +231,8 @@ struct RotMode {
     __device__ static const float *a_row(const Args &a, const Tile &T, int i) {
         return i < T.ni ? a.Q + (T.q0 + i) * a.d : nullptr;
     }
-    __device__ static const unsigned char *b_block(const Args &a, const Tile &, int ch) {
-        return a.rot + (int64_t)ch * ((a.d + 63) / 64) * kTcBlockBytes;
+    __device__ static const unsigned char *b_block(const Args &a, const Tile &) {
+        return a.rot;
     }
     struct Epi {
         float *row;

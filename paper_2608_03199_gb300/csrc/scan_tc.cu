@@ -63,9 +63,9 @@ struct ScanModeT {
     __device__ static const float *b_row(const Args &a, const Tile &T, int64_t r) {
         return r < T.nb ? a.X + (T.r_begin + r) * a.d : nullptr;
     }
-    __device__ static const unsigned char *b_block(const Args &a, const Tile &T, int ch) {
-        if (kRQ) return a.rq_rows + (T.blk0 + ch) * (int64_t)tc_nkb_dev(a.d) * tcb::kKbBytesHi;
-        return a.tc_rows + (T.blk0 + ch) * (int64_t)tc_nkb_dev(a.d) * kTcBlockBytes;
+    __device__ static const unsigned char *b_block(const Args &a, const Tile &T) {
+        if (kRQ) return a.rq_rows + T.blk0 * (int64_t)tc_nkb_dev(a.d) * tcb::kKbBytesHi;
+        return a.tc_rows + T.blk0 * (int64_t)tc_nkb_dev(a.d) * kTcBlockBytes;
     }
 
     struct Epi {

@@ -27,13 +27,13 @@
 //               the previous tile's last MMAs on that K-block are done
 //               ("a_empty[kb]"), split the values, store them with tcgen05.st
 //               and publish the K-block ("a_full[kb]")
-//   warp 8      lane 0 takes the block's next tile (an atomic work counter,
+//   warp 8      (in step, lane 0 acting) takes the block's next tile (an atomic work counter,
 //               or a static stride when the mode has none) and hands it to the
 //               other roles through a small ring in shared memory; it then
 //               issues the tile's bulk copies of B stages ("b_full" with the
 //               transfer byte count; waits on "b_empty")
-//   warp 9      allocates the tensor memory; lane 0 issues the mode's one to
-//               three kind::f16 MMAs per K step (A from tensor memory, B from
+//   warp 9      allocates the tensor memory; the whole warp runs the issue loop
+//               and lane 0 issues the mode's one to three kind::f16 MMAs per K step (A from tensor memory, B from
 //               shared memory)
 //   warps 10-13 epilogue: thread i owns tensor-memory lane i = A row i; it
 //               hands its row of a chunk (scores x 2^16) to Mode::Epi
@@ -174,6 +174,27 @@ __device__ __forceinline__ uint32_t epi_wait_polls(const typename Mode::Args &a)
     }
 }
 
+// A value every lane of the warp holds, as one the compiler knows to be
+// uniform: role branches, loop bounds and the operands of MMAs and bulk copies.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ const unsigned char *uniform_ptr(const unsigned char *p) {
+    return reinterpret_cast<const unsigned char *>(
+        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(p), 0));
+}
+
+// A position in a ring of n slots and the parity of the phase it is in: the
+// producer, the MMA issuer and the epilogue step through their rings with it
+// (slot = i % n and phase = i / n with a run-time n are two divisions a step).
+struct RingPos {
+    uint32_t slot = 0, phase = 0;
+    __device__ __forceinline__ void step(uint32_t n) {
+        if (++slot == n) {
+            slot = 0;
+            phase ^= 1u;
+        }
+    }
+};
+
 // one 32-column group of an accumulator row to the mode's epilogue
 template <class Epi, class Args, class Tile>
 __device__ __forceinline__ void hand(Epi &epi, const Args &a, const Tile &T, int64_t col0,
@@ -185,6 +206,14 @@ __device__ __forceinline__ void hand(Epi &epi, const Args &a, const Tile &T, int
     epi.chunk(a, T, col0, v, left < 32 ? (int)left : 32);
 }
 
+// What bounds the issuing warp: each chunk's waits, commits and MMAs are one
+// serial chain, so every instruction between two MMAs costs.  Running the
+// producer and issuer loops as whole warps in uniform flow (lane 0 predicated,
+// uniform() on every loaded value) and without divisions took, on 1M x 256 at
+// W = 64, the scan from 7.07 to 6.38 ms, at W = 8 from 1.86 to 1.68 ms, the
+// scan over codes from 1.47 to 1.23 ms, and the ranking contractions of 100K
+// queries x 65,536 x 96 from 4.4 to 3.95 ms.
+//
 // The MMAs of one B stage for one sub-tile, fully unrolled: K1 K steps of 16
 // in the stage's first K-block and K2 in its second (0: none).  a0 = the
 // sub-tile's A columns of that first K-block (hi; lo 32 columns on), b0 = the
@@ -195,7 +224,7 @@ __device__ __forceinline__ void hand(Epi &epi, const Args &a, const Tile &T, int
 // One straight run of MMAs with their operands a constant off two bases: the
 // single issuing thread keeps up with the tensor pipe.
 template <int kProd, int K1, int K2, uint32_t kKbStageBytes>
-__device__ __forceinline__ void issue_stage(uint32_t dt, uint32_t a0, uint64_t b0, uint32_t acc_first,
+__device__ __forceinline__ void issue_stage(uint32_t lead, uint32_t dt, uint32_t a0, uint64_t b0, uint32_t acc_first,
                                             uint32_t idesc) {
     constexpr uint32_t kAKbT = kProd == 1 ? 32 : 64;                       // A columns per K-block
     constexpr uint64_t kKbDesc = kKbStageBytes >> 4;                         // B K-block in 16-byte units
@@ -207,14 +236,14 @@ __device__ __forceinline__ void issue_stage(uint32_t dt, uint32_t a0, uint64_t b
         const uint64_t bh = b0 + (uint64_t)kb * kKbDesc + 2u * (uint64_t)ks;
         const uint32_t acc = j == 0 ? acc_first : 1u;
         if constexpr (kProd == 3) {        // lo_a hi_b + hi_a lo_b + hi_a hi_b
-            tc::mma_f16_ta(dt, a + 32u, bh, idesc, acc);
-            tc::mma_f16_ta(dt, a, bh + kLoDesc, idesc, 1u);
-            tc::mma_f16_ta(dt, a, bh, idesc, 1u);
+            tc::mma_f16_ta(lead, dt, a + 32u, bh, idesc, acc);
+            tc::mma_f16_ta(lead, dt, a, bh + kLoDesc, idesc, 1u);
+            tc::mma_f16_ta(lead, dt, a, bh, idesc, 1u);
         } else if constexpr (kProd == 2) { // B exact in fp16: lo_a b + hi_a b
-            tc::mma_f16_ta(dt, a + 32u, bh, idesc, acc);
-            tc::mma_f16_ta(dt, a, bh, idesc, 1u);
+            tc::mma_f16_ta(lead, dt, a + 32u, bh, idesc, acc);
+            tc::mma_f16_ta(lead, dt, a, bh, idesc, 1u);
         } else {                           // a screen: hi_a hi_b
-            tc::mma_f16_ta(dt, a, bh, idesc, acc);
+            tc::mma_f16_ta(lead, dt, a, bh, idesc, acc);
         }
     }
 }
@@ -222,25 +251,26 @@ __device__ __forceinline__ void issue_stage(uint32_t dt, uint32_t a0, uint64_t b
 // issue_stage for a run-time K-step pattern: a stage's first K-block has k1
 // steps (1..4) and its second k2 (0..4, only after a full first block)
 template <int kProd, uint32_t kKbStageBytes>
-__device__ __forceinline__ void issue_stage_rt(int k1, int k2, uint32_t dt, uint32_t a0, uint64_t b0,
+__device__ __forceinline__ void issue_stage_rt(uint32_t lead, int k1, int k2, uint32_t dt, uint32_t a0, uint64_t b0,
                                                uint32_t acc_first, uint32_t idesc) {
     constexpr uint32_t B = kKbStageBytes;
     switch (k1 * 8 + k2) {
-        case 4 * 8 + 4: issue_stage<kProd, 4, 4, B>(dt, a0, b0, acc_first, idesc); break;
-        case 4 * 8 + 3: issue_stage<kProd, 4, 3, B>(dt, a0, b0, acc_first, idesc); break;
-        case 4 * 8 + 2: issue_stage<kProd, 4, 2, B>(dt, a0, b0, acc_first, idesc); break;
-        case 4 * 8 + 1: issue_stage<kProd, 4, 1, B>(dt, a0, b0, acc_first, idesc); break;
-        case 4 * 8 + 0: issue_stage<kProd, 4, 0, B>(dt, a0, b0, acc_first, idesc); break;
-        case 3 * 8 + 0: issue_stage<kProd, 3, 0, B>(dt, a0, b0, acc_first, idesc); break;
-        case 2 * 8 + 0: issue_stage<kProd, 2, 0, B>(dt, a0, b0, acc_first, idesc); break;
-        default: issue_stage<kProd, 1, 0, B>(dt, a0, b0, acc_first, idesc); break;
+        case 4 * 8 + 4: issue_stage<kProd, 4, 4, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 4 * 8 + 3: issue_stage<kProd, 4, 3, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 4 * 8 + 2: issue_stage<kProd, 4, 2, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 4 * 8 + 1: issue_stage<kProd, 4, 1, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 4 * 8 + 0: issue_stage<kProd, 4, 0, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 3 * 8 + 0: issue_stage<kProd, 3, 0, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        case 2 * 8 + 0: issue_stage<kProd, 2, 0, B>(lead, dt, a0, b0, acc_first, idesc); break;
+        default: issue_stage<kProd, 1, 0, B>(lead, dt, a0, b0, acc_first, idesc); break;
     }
 }
 
 // Mode provides (in addition to what tc_pipeline.cuh asks): Epi::prefetch(a,
 // T, ch) and Epi::start(a, T, ch), called by every epilogue lane of a warp
-// before and after the wait for chunk ch's accumulator; b_block(a, T, ch)
-// = pointer to the tensor-layout bytes of the tile's ch-th block of B rows;
+// before and after the wait for chunk ch's accumulator; b_block(a, T) =
+// pointer to the tensor-layout bytes of the tile's first block of B rows
+// (the others follow it);
 // tile_counter(a) = a zeroed global int the blocks draw tiles from (nullptr:
 // block b takes tiles b, b + gridDim.x, ...).
 template <class Mode>
@@ -279,7 +309,7 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
 
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const int n_tiles = Mode::num_tiles(a);
     const int d = Mode::d(a);
     const int nkb = (int)ceil_div(d, 64);
@@ -292,6 +322,7 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
         return;
     }
     const uint32_t nacc = acc_slots(nkb, kProd, kSub);
+    const uint32_t blk_bytes = (uint32_t)nkb * kSrcKb;         // one block of B in global memory
     const uint32_t aTile = a_cols(nkb, kProd);                 // A columns of one sub-tile
     unsigned char *Bst = base;                                 // stages x kStage
     unsigned char *epi_smem = Bst + (size_t)stages * kStage;
@@ -322,7 +353,7 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = (uint32_t)uniform((int)tmem_slot);
     const uint32_t tA = tmem + nacc * kNB;                     // A after the accumulators
 
     auto wait_n = [&](uint64_t *bar, uint32_t parity, uint32_t polls) -> bool {
@@ -342,6 +373,11 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
         return false;
     };
     auto wait = [&](uint64_t *bar, uint32_t parity) -> bool { return wait_n(bar, parity, kWaitPolls); };
+    // a whole warp's wait: every lane polls, and all take the same way on
+    auto warp_wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+        return __all_sync(0xffffffffu, wait(bar, parity));
+    };
+    const uint32_t lead = lane == 0;
     const uint32_t epi_wait = epi_wait_polls<Mode>(a);
     // the i-th tile of this block from the ring, read by a whole warp (one
     // arrival per warp); false when the wait gave up.  t < 0 ends the loop.
@@ -405,16 +441,21 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
         }
     } else if (warp == kProdW) {
         // ---------------- tile scheduler + B producer ----------------
-        if (lane == 0) {
-            uint32_t s = 0;
+        // (the whole warp, in step; lane 0 publishes the tiles and issues the copies)
+        {
+            uint32_t s = 0;   // stages filled
+            RingPos bp;       // the stage to fill next
             // the block's i-th tile into ring slot i % kRing (t < 0: no more)
             auto publish = [&](uint32_t i, int &t) -> bool {
                 const uint32_t slot = i % kRing, ph = (i / kRing) & 1u;
-                if (!wait(&ring_empty[slot], ph ^ 1u)) return false;
-                t = tile_counter ? atomicAdd(tile_counter, 1) : (int)(blockIdx.x + i * gridDim.x);
-                if (t >= n_tiles) t = -1;
-                ring_tile[slot] = t;
-                tc::mbar_arrive(&ring_full[slot]);   // release: the tile id is visible with the phase
+                if (!warp_wait(&ring_empty[slot], ph ^ 1u)) return false;
+                if (lane == 0) {
+                    t = tile_counter ? atomicAdd(tile_counter, 1) : (int)(blockIdx.x + i * gridDim.x);
+                    if (t >= n_tiles) t = -1;
+                    ring_tile[slot] = t;
+                    tc::mbar_arrive(&ring_full[slot]);   // release: the tile id is visible with the phase
+                }
+                t = uniform(t);
                 return true;
             };
             int cur = -1;
@@ -427,8 +468,9 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 if (!(ok = publish(i + 1, nxt))) break;
                 const typename Mode::Tile T = Mode::tile(a, cur);
                 cur = nxt;
-                const int nch = (int)ceil_div(T.nb, kNB);
-                const int nblk = (int)ceil_div(T.nb, kN);             // layout blocks of the tile's B
+                const int nch = uniform((int)ceil_div(T.nb, kNB));
+                const int nblk = uniform((int)ceil_div(T.nb, kN));   // layout blocks of the tile's B
+                const unsigned char *src0 = uniform_ptr(Mode::b_block(a, T));
                 for (int ch = 0; ok && ch < nch; ++ch) {
                     if constexpr (kNB != kN) {
                         // a 192-row chunk: rows r0 .. r0 + 191 of the tile's B, from
@@ -439,41 +481,43 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                         const int r0 = ch * kNB, b0 = r0 / kN, o0 = r0 % kN;
                         const uint32_t n0 = (uint32_t)(kN - o0);
                         const uint32_t n1 = b0 + 1 < nblk ? (uint32_t)kNB - n0 : 0u;
-                        const unsigned char *p0 = Mode::b_block(a, T, b0);
-                        const unsigned char *p1 = n1 ? Mode::b_block(a, T, b0 + 1) : nullptr;
+                        const unsigned char *p0 = src0 + (size_t)b0 * blk_bytes;
+                        const unsigned char *p1 = p0 + blk_bytes;
                         for (int kb = 0; kb < nkb; kb += kKs) {
-                            const uint32_t st = s % stages, sph = (s / stages) & 1u;
+                            const uint32_t st = bp.slot;
                             const int nk = nkb - kb < kKs ? nkb - kb : kKs;
-                            if (!(ok = wait(&b_empty[st], sph ^ 1u))) break;
-                            tc::mbar_arrive_expect_tx(&b_full[st], (uint32_t)nk * (n0 + n1) * 128u);
+                            if (!(ok = warp_wait(&b_empty[st], bp.phase ^ 1u))) break;
+                            tc::mbar_arrive_expect_tx(lead, &b_full[st], (uint32_t)nk * (n0 + n1) * 128u);
                             for (int j = 0; j < nk; ++j) {
                                 unsigned char *dst = Bst + (size_t)st * kStage + (size_t)j * kKbB;
-                                tc::bulk_g2s(dst, p0 + (size_t)(kb + j) * kSrcKb + (size_t)o0 * 128u, n0 * 128u,
+                                tc::bulk_g2s(lead, dst, p0 + (size_t)(kb + j) * kSrcKb + (size_t)o0 * 128u, n0 * 128u,
                                              &b_full[st]);
                                 if (n1)
-                                    tc::bulk_g2s(dst + (size_t)n0 * 128u, p1 + (size_t)(kb + j) * kSrcKb, n1 * 128u,
+                                    tc::bulk_g2s(lead, dst + (size_t)n0 * 128u, p1 + (size_t)(kb + j) * kSrcKb, n1 * 128u,
                                                  &b_full[st]);
                             }
                             ++s;
+                            bp.step(stages);
                         }
                         continue;
                     }
                     // a block's K-blocks are contiguous: a stage is one copy
-                    const unsigned char *src = Mode::b_block(a, T, ch);
+                    const unsigned char *src = src0 + (size_t)ch * blk_bytes;
                     for (int kb = 0; kb < nkb; kb += kKs) {
-                        const uint32_t st = s % stages, sph = (s / stages) & 1u;
+                        const uint32_t st = bp.slot;
                         const uint32_t bytes = (uint32_t)(nkb - kb < kKs ? nkb - kb : kKs) * kKbB;
-                        if (!(ok = wait(&b_empty[st], sph ^ 1u))) break;
-                        tc::mbar_arrive_expect_tx(&b_full[st], bytes);
+                        if (!(ok = warp_wait(&b_empty[st], bp.phase ^ 1u))) break;
+                        tc::mbar_arrive_expect_tx(lead, &b_full[st], bytes);
                         if constexpr (kSrcKb == kKbB) {
-                            tc::bulk_g2s(Bst + (size_t)st * kStage, src + (size_t)kb * kKbB, bytes,
+                            tc::bulk_g2s(lead, Bst + (size_t)st * kStage, src + (size_t)kb * kKbB, bytes,
                                          &b_full[st]);
                         } else {   // the hi halves of this stage's K-blocks
                             for (uint32_t j = 0; j * kKbB < bytes; ++j)
-                                tc::bulk_g2s(Bst + (size_t)st * kStage + j * kKbB,
+                                tc::bulk_g2s(lead, Bst + (size_t)st * kStage + j * kKbB,
                                              src + ((size_t)kb + j) * kSrcKb, kKbB, &b_full[st]);
                         }
                         ++s;
+                        bp.step(stages);
                     }
                 }
             }
@@ -486,8 +530,10 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
         __syncwarp();
     } else if (warp == kMmaW) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            uint32_t s = 0, c = 0, u = 0;   // c: accumulator uses, kSub per chunk
+        // (the whole warp, in step; lane 0 issues the MMAs and commits)
+        {
+            uint32_t u = 0;
+            RingPos bp, dp;   // the B stage and the accumulator (kSub of them per chunk) in use
             bool ok = true;
             // the descriptor of stage 0's first K-block; stage st is st * kStage
             // bytes on (the start-address field does not carry: shared
@@ -495,25 +541,25 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
             const uint64_t b_desc0 = tc::desc_k_sw128(tc::smem_u32(Bst));
             for (uint32_t i = 0; ok; ++i) {
                 const uint32_t slot = i % kRing, rph = (i / kRing) & 1u;
-                if (!(ok = wait(&ring_full[slot], rph))) break;
-                const int t = *(volatile int *)&ring_tile[slot];
-                tc::mbar_arrive(&ring_empty[slot]);
+                if (!(ok = warp_wait(&ring_full[slot], rph))) break;
+                const int t = uniform(*(volatile int *)&ring_tile[slot]);
+                if (lane == 0) tc::mbar_arrive(&ring_empty[slot]);
                 if (t < 0) break;
                 const typename Mode::Tile T = Mode::tile(a, t);
-                const int nch = (int)ceil_div(T.nb, kNB);
+                const int nch = uniform((int)ceil_div(T.nb, kNB));
                 if (nch == 0) continue;
-                for (int ch = 0; ok && ch < nch; ++ch, c += kSub) {
+                for (int ch = 0; ok && ch < nch; ++ch) {
                     if constexpr (kSub == 1) {   // the chunk's accumulator
-                        if (!(ok = wait(&dempty_bar[c % nacc], ((c / nacc) & 1u) ^ 1u))) break;
+                        if (!(ok = warp_wait(&dempty_bar[dp.slot], dp.phase ^ 1u))) break;
                         tc::fence_after_sync();
                     }
-                    for (int kb0 = 0; kb0 < nkb; kb0 += kKs, ++s) {
-                        const uint32_t st = s % stages, ph = (s / stages) & 1u;
+                    for (int kb0 = 0; kb0 < nkb; kb0 += kKs, bp.step(stages)) {
+                        const uint32_t st = bp.slot, ph = bp.phase;
                         const int kb1 = nkb - kb0 < kKs ? nkb : kb0 + kKs;   // this stage's K-blocks
                         const bool last = kb1 == nkb;                       // the chunk's last stage
                         if (ch == 0)
-                            for (int kb = kb0; ok && kb < kb1; ++kb) ok = wait(&a_full[kb], u & 1u);
-                        if (!ok || !(ok = wait(&b_full[st], ph))) break;
+                            for (int kb = kb0; ok && kb < kb1; ++kb) ok = warp_wait(&a_full[kb], u & 1u);
+                        if (!ok || !(ok = warp_wait(&b_full[st], ph))) break;
                         tc::fence_after_sync();
                         // K steps of 16 that hold any of the d elements (the rest of
                         // the last K-block is zero padding), per K-block of the stage
@@ -522,29 +568,32 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                         const uint64_t b_stage = b_desc0 + (uint64_t)st * (kStage >> 4);
 #pragma unroll 1
                         for (int h = 0; ok && h < kSub; ++h) {
-                            if (kSub > 1 && kb0 == 0) {   // sub-tile h's accumulator, just before its MMAs
-                                if (!(ok = wait(&dempty_bar[(c + h) % nacc], (((c + h) / nacc) & 1u) ^ 1u))) break;
+                            // two sub-tiles: accumulator h is sub-tile h's, one phase per chunk
+                            const uint32_t buf = kSub > 1 ? (uint32_t)h : dp.slot;
+                            if (kSub > 1 && kb0 == 0) {   // waited for just before its MMAs
+                                if (!(ok = warp_wait(&dempty_bar[buf], dp.phase ^ 1u))) break;
                                 tc::fence_after_sync();
                             }
-                            const uint32_t dt = tmem + ((c + h) % nacc) * kNB;
-                            issue_stage_rt<kProd, kKbB>(k1, k2, dt, tA + (uint32_t)h * aTile + (uint32_t)kb0 * kAKb,
+                            const uint32_t dt = tmem + buf * kNB;
+                            issue_stage_rt<kProd, kKbB>(lead, k1, k2, dt, tA + (uint32_t)h * aTile + (uint32_t)kb0 * kAKb,
                                                         b_stage, kb0 > 0 ? 1u : 0u, kIdesc);
                             // with two sub-tiles, the first sub-tile's accumulator is
                             // handed over before the second's MMAs are issued
-                            if (kSub > 1 && last && h + 1 < kSub) tc::mma_commit(&dfull_bar[(c + h) % nacc]);
+                            if (kSub > 1 && last && h + 1 < kSub) tc::mma_commit(lead, &dfull_bar[h]);
                         }
                         if (!ok) break;
-                        tc::mma_commit(&b_empty[st]);
+                        tc::mma_commit(lead, &b_empty[st]);
                         // the tile's last reads of these K-blocks of A: they may be
                         // overwritten by the next tile once they are done
                         if (ch == nch - 1)
-                            for (int kb = kb0; kb < kb1; ++kb) tc::mma_commit(&a_empty[kb]);
+                            for (int kb = kb0; kb < kb1; ++kb) tc::mma_commit(lead, &a_empty[kb]);
                     }
-                    if (ok) tc::mma_commit(&dfull_bar[(c + kSub - 1) % nacc]);
+                    if (ok) tc::mma_commit(lead, &dfull_bar[kSub > 1 ? (uint32_t)(kSub - 1) : dp.slot]);
+                    dp.step(kSub > 1 ? 1u : nacc);
                 }
                 ++u;
             }
-            tc::mma_commit(&drain_bar);
+            tc::mma_commit(lead, &drain_bar);
             for (uint32_t it = 0; it < kWaitPolls; ++it)
                 if (tc::mbar_try_wait(&drain_bar, 0u)) break;
         }
@@ -554,7 +603,7 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
         const int quarter = warp & 3;                      // the lanes this warp may read
         const int h = (warp - kEpiW0) >> 2;                // its sub-tile
         const int slot = h * tcp::kM + quarter * 32 + lane;
-        uint32_t c = h;
+        RingPos dp;                                        // two sub-tiles: accumulator h, one phase per chunk
         bool ok = true;
         typename Mode::Epi epi;
         for (uint32_t i = 0; ok; ++i) {
@@ -563,8 +612,8 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
             const typename Mode::Tile T = Mode::tile(a, t);
             const int nch = (int)ceil_div(T.nb, kNB);
             epi.begin(a, T, slot, epi_smem);
-            for (int ch = 0; ch < nch; ++ch, c += kSub) {
-                const uint32_t buf = c % nacc, dph = (c / nacc) & 1u;
+            for (int ch = 0; ch < nch; ++ch, dp.step(kSub > 1 ? 1u : nacc)) {
+                const uint32_t buf = kSub > 1 ? (uint32_t)h : dp.slot, dph = dp.phase;
                 epi.prefetch(a, T, ch);   // per-chunk loads, in flight during the wait
                 ok = __all_sync(0xffffffffu, wait_n(&dfull_bar[buf], dph, epi_wait));
                 if (!ok) break;

@@ -118,7 +118,7 @@ __device__ __forceinline__ void run_pipeline(const typename Mode::Args &a, unsig
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     unsigned char *epi_smem = base + kStages * G::STAGE_BYTES;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int n_tiles = Mode::num_tiles(a);
     const int d = Mode::d(a);
     const int nkb = (int)ceil_div(d, kKB);
@@ -141,7 +141,7 @@ __device__ __forceinline__ void run_pipeline(const typename Mode::Args &a, unsig
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
 
     // bounded wait; gives up early once another role has aborted
     auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
@@ -195,20 +195,22 @@ __device__ __forceinline__ void run_pipeline(const typename Mode::Args &a, unsig
     conv_done:;
     } else if (warp == kMmaWarp) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        // (the whole warp, in step; lane 0 issues the MMAs and commits)
+        {
+            const uint32_t lead = lane == 0;
             uint32_t s = 0, c = 0;
             bool ok = true;
             for (int t = blockIdx.x; ok && t < n_tiles; t += gridDim.x) {
                 const typename Mode::Tile T = Mode::tile(a, t);
-                const int nch = (int)ceil_div(T.nb, kN);
+                const int nch = __shfl_sync(0xffffffffu, (int)ceil_div(T.nb, kN), 0);
                 for (int ch = 0; ok && ch < nch; ++ch, ++c) {
                     const uint32_t buf = c & 1u, dph = (c >> 1) & 1u;
-                    if (!(ok = wait(&dempty_bar[buf], dph ^ 1u))) break;
+                    if (!(ok = __all_sync(0xffffffffu, wait(&dempty_bar[buf], dph ^ 1u)))) break;
                     tc::fence_after_sync();
                     const uint32_t dt = tmem + buf * kN;
                     for (int kb = 0; kb < nkb; ++kb, ++s) {
                         const uint32_t st = s & 1u, ph = (s >> 1) & 1u;
-                        if (!(ok = wait(&full_bar[st], ph))) break;
+                        if (!(ok = __all_sync(0xffffffffu, wait(&full_bar[st], ph)))) break;
                         tc::fence_after_sync();
                         const uint32_t sa = tc::smem_u32(base + st * G::STAGE_BYTES);
                         const uint32_t a_hi = sa, a_lo = sa + A_BYTES;
@@ -219,21 +221,21 @@ __device__ __forceinline__ void run_pipeline(const typename Mode::Args &a, unsig
                         for (int ks = 0; ks < kKB / 16; ++ks) {   // K = 16 fp16 = 32 bytes per MMA
                             if (ks >= kst) break;
                             const uint32_t o = ks * 32;
-                            tc::mma_f16(dt, tc::desc_k_sw128(a_lo + o), tc::desc_k_sw128(b_hi + o),
+                            tc::mma_f16(lead, dt, tc::desc_k_sw128(a_lo + o), tc::desc_k_sw128(b_hi + o),
                                         kIdesc, (kb > 0 || ks > 0) ? 1u : 0u);
-                            tc::mma_f16(dt, tc::desc_k_sw128(a_hi + o), tc::desc_k_sw128(b_lo + o),
+                            tc::mma_f16(lead, dt, tc::desc_k_sw128(a_hi + o), tc::desc_k_sw128(b_lo + o),
                                         kIdesc, 1u);
-                            tc::mma_f16(dt, tc::desc_k_sw128(a_hi + o), tc::desc_k_sw128(b_hi + o),
+                            tc::mma_f16(lead, dt, tc::desc_k_sw128(a_hi + o), tc::desc_k_sw128(b_hi + o),
                                         kIdesc, 1u);
                         }
-                        tc::mma_commit(&empty_bar[st]);
+                        tc::mma_commit(lead, &empty_bar[st]);
                     }
-                    if (ok) tc::mma_commit(&dfull_bar[buf]);
+                    if (ok) tc::mma_commit(lead, &dfull_bar[buf]);
                 }
             }
             // every MMA issued by this thread has finished once drain_bar
             // flips (waited for even after an abort, within the poll limit)
-            tc::mma_commit(&drain_bar);
+            tc::mma_commit(lead, &drain_bar);
             for (uint32_t it = 0; it < kWaitPolls; ++it)
                 if (tc::mbar_try_wait(&drain_bar, 0u)) break;
         }

@@ -49,15 +49,22 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
                  : "memory");
 }
 
+// The MMAs, commits, arrivals and copies below are issued by the calling
+// threads for which `lead` is non-zero (one lane of a warp).  The whole warp
+// runs the surrounding loop and only the instruction is predicated: MMAs and
+// bulk copies take their operands from uniform registers, which the compiler
+// computes in place only in warp-uniform control flow; under a branch on the
+// lane every operand of every instruction is moved there first.
+
 // kind::f16 MMA with A in tensor memory: lane i holds row i of A, each 32-bit
 // column two consecutive K elements (the even one in the low half); one
 // K = 16 step reads 8 columns from a_tmem
-__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                           uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16_ta(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem,
+                                           uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
 
@@ -74,20 +81,21 @@ __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                        uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16(uint32_t lead, uint32_t d_tmem, uint64_t a_desc,
+                                        uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
 
 // arrive once on an mbarrier when every MMA this thread issued so far is done
-__device__ __forceinline__ void mma_commit(uint64_t *mbar) {
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint64_t *mbar) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(mbar))
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+            smem_u32(mbar)), "r"(lead)
         : "memory");
 }
 
@@ -179,22 +187,24 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, uint32_t parit
 
 // arrive on an mbarrier and announce `bytes` of asynchronous transfer that
 // will complete on it
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *mbar, uint32_t bytes) {
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t lead, uint64_t *mbar, uint32_t bytes) {
     asm volatile(
-        "{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.release.cta.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
+        "{\n\t.reg .b64 st;\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+        "@q mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
             smem_u32(mbar)),
-        "r"(bytes)
+        "r"(bytes), "r"(lead)
         : "memory");
 }
 
 // bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned)
 // from global to this CTA's shared memory, completing on an mbarrier
-__device__ __forceinline__ void bulk_g2s(void *smem_dst, const void *gmem_src, uint32_t bytes,
-                                         uint64_t *mbar) {
+__device__ __forceinline__ void bulk_g2s(uint32_t lead, void *smem_dst, const void *gmem_src,
+                                         uint32_t bytes, uint64_t *mbar) {
     asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+        "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}" ::"r"(
             smem_u32(smem_dst)),
-        "l"(gmem_src), "r"(bytes), "r"(smem_u32(mbar))
+        "l"(gmem_src), "r"(bytes), "r"(smem_u32(mbar)), "r"(lead)
         : "memory");
 }
 
