@@ -619,24 +619,27 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 if (!ok) break;
                 epi.start(a, T, ch);
                 tc::fence_after_sync();
-                // pairs of 32-column loads, each pair in flight together; the
-                // accumulator is released as soon as the last pair has landed,
-                // before its columns are handed to the mode
+                // one copy of the mode's code per load, in a loop that is not
+                // unrolled: each role runs straight code of its own, and with
+                // the loop unrolled the epilogue waits for instructions (join
+                // of 100K queries with 1M x 256, W = 8: scan 1.70 -> 1.23 ms).  The accumulator is released as soon as the
+                // last load has landed, before its columns go to the mode.
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kNB;
                 const int64_t col0 = (int64_t)ch * kNB;
-                uint32_t ra[32], rb[32];
+                constexpr int kLd = kSub;   // 32-column loads per step
+                uint32_t r[kLd][32];
+#pragma unroll 1
+                for (int g = 0; g < kNB / 32; g += kLd) {
 #pragma unroll
-                for (int pr = 0; pr < kNB / 64; ++pr) {
-                    tc::tmem_ld32_issue(taddr + pr * 64, ra);
-                    tc::tmem_ld32_issue(taddr + pr * 64 + 32, rb);
-                    tc::tmem_ld_wait(ra);
-                    tc::tmem_ld_wait(rb);
-                    if (pr == kNB / 64 - 1) {
+                    for (int u = 0; u < kLd; ++u) tc::tmem_ld32_issue(taddr + (g + u) * 32, r[u]);
+#pragma unroll
+                    for (int u = 0; u < kLd; ++u) tc::tmem_ld_wait(r[u]);
+                    if (g == kNB / 32 - kLd) {
                         tc::fence_before_sync();
                         tc::mbar_arrive(&dempty_bar[buf]);
                     }
-                    hand(epi, a, T, col0 + pr * 64, ra);
-                    hand(epi, a, T, col0 + pr * 64 + 32, rb);
+#pragma unroll
+                    for (int u = 0; u < kLd; ++u) hand(epi, a, T, col0 + (g + u) * 32, r[u]);
                 }
             }
             if (!ok) break;
