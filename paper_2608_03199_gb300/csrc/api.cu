@@ -73,6 +73,12 @@ constexpr int kScreenMinWindow = 16;   // automatic scan path: the screen from t
 constexpr int kScreenMinD = 192;       // ... or at any window from this d up ...
 constexpr float kScreenMinTau = 0.85f; // ... and this threshold up (below it nearly every row
                                        // of a probed partition needs its fp32 rescore)
+// Up to 2,048 centroids the full ranking is two short launches, and a small
+// batch pays the latency of filling the prefix's lists instead of bandwidth
+// (1,003 queries x 149 x 100: ranking 42 us whole, 58 us as a prefix; 10,007 x
+// 1,024 x 256: 60 us less as a prefix)
+constexpr int64_t kPrefixAlwaysNlist = 2048;
+constexpr int64_t kPrefixMinQueries = 4096;
 constexpr int64_t kAutoCapMax = int64_t(1) << 24;
 constexpr int64_t kCapMax = int64_t(1) << 30;
 
@@ -132,7 +138,8 @@ Layout make_layout(const sieve_index_view *ix, int64_t nq, const sieve_params *p
     L.res_s = take((size_t)cap * p->k * 4);
     L.res_id = take((size_t)cap * p->k * 8);
     L.rank_scratch = (p->scan_path != 1 && rank_tc_supported(ix->nlist, p->nprobe))
-                         ? take(rank_tc_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d))
+                         ? take(std::max(rank_tc_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d),
+                                         rank_prefix_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d)))
                          : 0;
     if (host_io) {
         L.h_Q = take((size_t)nq * ix->d * 4);
@@ -183,10 +190,19 @@ constexpr size_t kGraphCacheMax = 8;
 cudaError_t launch_search_rank(const SearchArgs &a, int rank_tc, cudaStream_t st,
                                float *mma_ms = nullptr) {
     int32_t *order = const_cast<int32_t *>(a.order);
+    if (a.limit)
+        return enqueue_rank_prefix(a.Q, 0, a.nq, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, order, a.cscores,
+                                   a.rank_scratch, &a.ctl->status, a.tc_cent, st, mma_ms);
     if (rank_tc)
         return enqueue_rank_tc(a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, order, a.cscores,
                                a.rank_scratch, &a.ctl->status, st, a.tc_cent, mma_ms);
     return enqueue_rank(a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, order, a.cscores, st);
+}
+
+// the end of a round that met queries whose stop line passes their prefix
+cudaError_t launch_search_ext(const SearchArgs &a, cudaStream_t st) {
+    return enqueue_rank_ext(a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, const_cast<int32_t *>(a.order),
+                            a.cscores, a.rank_scratch, &a.ctl->ext_n, &a.ctl->status, a.tc_cent, st);
 }
 
 // quantized search: q' = P^T q for the batch, after init (which clears the
@@ -195,52 +211,67 @@ cudaError_t launch_search_rotate(const SearchArgs &a, cudaStream_t st) {
     return launch_rq_rotate(a.Q, a.nq, a.d, a.rq_rot, const_cast<float *>(a.Qrot), &a.ctl->status, st);
 }
 
+// A conditional node at the end of what cs has captured so far; *handle is
+// created unless it is given, *body_out is the graph the node runs.
+cudaError_t add_conditional(cudaStream_t cs, cudaGraphConditionalNodeType type, unsigned initial,
+                            cudaGraphConditionalHandle *handle, cudaGraph_t *body_out) {
+    cudaStreamCaptureStatus cst;
+    cudaGraph_t cg = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t ndeps = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps);
+    if (e == cudaSuccess && !*handle)
+        e = cudaGraphConditionalHandleCreate(handle, cg, initial, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams np{};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = *handle;
+    np.conditional.type = type;
+    np.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    if ((e = cudaGraphAddNode(&node, cg, deps, nullptr, ndeps, &np)) != cudaSuccess) return e;
+    *body_out = np.conditional.phGraph_out[0];
+    return cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+}
+
 sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_t *exec_out) {
     const SearchArgs &a = key.a;
     cudaStream_t cs = nullptr;
     SIEVE_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaSuccess;
-    cudaGraphConditionalHandle cond = 0;
-    cudaGraphNodeParams np{};
-    cudaGraphNode_t wnode = nullptr;
+    cudaGraphConditionalHandle cond = 0, ext_cond = 0;
+    cudaGraph_t body = nullptr, ext_body = nullptr;
     do {
-        // outer graph: [rank] -> init -> WHILE(rounds) -> finalize
+        // outer graph: init -> [rank] -> WHILE(rounds) -> finalize
         if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
         e = launch_init(a, cs);
         if (e == cudaSuccess && a.rq) e = launch_search_rotate(a, cs);
         if (e == cudaSuccess && key.with_rank) e = launch_search_rank(a, key.rank_tc, cs);
-        cudaStreamCaptureStatus cst;
-        cudaGraph_t cg = nullptr;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t ndeps = 0;
-        if (e == cudaSuccess)
-            e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps);
-        if (e == cudaSuccess)
-            e = cudaGraphConditionalHandleCreate(&cond, cg, 1, cudaGraphCondAssignDefault);
-        if (e == cudaSuccess) {
-            np.type = cudaGraphNodeTypeConditional;
-            np.conditional.handle = cond;
-            np.conditional.type = cudaGraphCondTypeWhile;
-            np.conditional.size = 1;
-            e = cudaGraphAddNode(&wnode, cg, deps, nullptr, ndeps, &np);
-        }
-        if (e == cudaSuccess)
-            e = cudaStreamUpdateCaptureDependencies(cs, &wnode, nullptr, 1,
-                                                    cudaStreamSetCaptureDependencies);
+        if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeWhile, 1, &cond, &body);
         if (e == cudaSuccess) e = launch_finalize(a, cs);
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess) break;
-        // loop body: one round
-        cudaGraph_t body = np.conditional.phGraph_out[0];
+        // loop body: one round, and the extension of the ranking when it asks for it
         if ((e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0,
                                                cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             break;
-        e = launch_round(a, key.scan_smem, key.scan_blocks, cond, 1, cs);
+        if (a.limit) e = cudaGraphConditionalHandleCreate(&ext_cond, body, 0, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) e = launch_round(a, key.scan_smem, key.scan_blocks, cond, ext_cond, 1, cs);
+        if (e == cudaSuccess && a.limit) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &ext_cond, &ext_body);
         e2 = cudaStreamEndCapture(cs, &body);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess) break;
+        if (a.limit) {
+            if ((e = cudaStreamBeginCaptureToGraph(cs, ext_body, nullptr, nullptr, 0,
+                                                   cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+                break;
+            e = launch_search_ext(a, cs);
+            e2 = cudaStreamEndCapture(cs, &ext_body);
+            if (e == cudaSuccess) e = e2;
+            if (e != cudaSuccess) break;
+        }
         e = cudaGraphInstantiate(exec_out, g, 0);
     } while (0);
     cudaStreamDestroy(cs);
@@ -344,12 +375,19 @@ struct RqInputs {
     const float *cscores;
 };
 
+// whether a search ranks a prefix of each order first: the bulk pipeline's
+// centroid layout, and a window that visits few of the nprobe ranks
+bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p) {
+    return ix->tc_centroids && (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
+           rank_prefix_len(ix->nlist, p->nprobe, p->W, ix->d) > 0;
+}
+
 sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t nq,
                            const int64_t *qids, const int32_t *order, const sieve_params *p,
                            int64_t *out_ids, float *out_scores, int32_t *out_count,
                            int32_t *out_probes, sieve_stats *stats, unsigned char *ws,
                            const Layout &L, cudaStream_t st, const SearchExtras *ex = nullptr,
-                           const RqInputs *rq = nullptr) {
+                           const RqInputs *rq = nullptr, bool prefix_given = false) {
     SearchArgs a;
     std::memset(&a, 0, sizeof(a));   // padding takes part in the graph-cache key
     a.X = ix->vectors;
@@ -449,6 +487,15 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
 
     const bool with_rank = order == nullptr;
     const int rank_tc = with_rank && a.rank_scratch != nullptr;
+    // the ranking writes a prefix of each query's order (or, prefix_given, wrote
+    // it already), and rounds extend the orders that turn out too short; not
+    // for codes, whose estimates carry the full ranking's centroid scores (a
+    // given order with its scores must give the same bits)
+    const bool prefix = prefix_given || (rank_tc && !rq && use_prefix(ix, nq, p));
+    if (prefix) {
+        a.limit = rank_prefix_limit(a.rank_scratch, nq, ix->nlist, p->nprobe, p->W, ix->d, &a.ext);
+        a.max_rounds = (int)std::min<int64_t>(INT32_MAX, (int64_t)a.max_rounds + p->nprobe);
+    }
     const size_t smem = scan_smem_bytes(ix->d, p->k);
     SIEVE_CUDA(prepare_scan_kernel(smem));
     if (a.rq) {
@@ -459,7 +506,9 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                    : a.tc_screen ? prepare_scan_screen(ix->d, p->k, a.tc_stages)
                                  : prepare_scan_bulk(ix->d, p->k, a.tc_stages));
     }
-    if (with_rank) SIEVE_CUDA(rank_tc ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
+    if (with_rank || prefix)
+        SIEVE_CUDA(rank_tc || prefix ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
+    if (prefix) SIEVE_CUDA(prepare_rank_prefix(ix->nlist, p->nprobe, p->W, ix->d));
     const int blocks = scan_blocks_for(smem);
 
     float ms[SIEVE_NKERNELS] = {0};
@@ -499,10 +548,12 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                 return launch_search_rank(a, rank_tc, st, p->profile ? &ms[SIEVE_K_RANK_MMA] : nullptr);
             }));
         for (;;) {
-            SIEVE_CUDA(launch_round(a, smem, blocks, 0, 0, st, p->profile ? ev.e : nullptr));
-            // the status word and the loop flag are adjacent in the control block
-            static_assert(offsetof(Ctl, more) == offsetof(Ctl, status) + sizeof(int), "");
-            int word[2] = {0, 0};
+            SIEVE_CUDA(launch_round(a, smem, blocks, 0, 0, 0, st, p->profile ? ev.e : nullptr));
+            // the status word, the loop flag and the extension's count are
+            // adjacent in the control block
+            static_assert(offsetof(Ctl, more) == offsetof(Ctl, status) + sizeof(int) &&
+                              offsetof(Ctl, ext_n) == offsetof(Ctl, more) + sizeof(int), "");
+            int word[3] = {0, 0, 0};
             SIEVE_CUDA(cudaMemcpyAsync(word, &a.ctl->status, sizeof(word), cudaMemcpyDeviceToHost, st));
             SIEVE_CUDA(cudaStreamSynchronize(st));
             host_status = word[0];
@@ -518,6 +569,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                 }
             }
             if (!more) break;
+            if (prefix && word[2] > 0) SIEVE_CUDA(timed(SIEVE_K_RANK, [&] { return launch_search_ext(a, st); }));
         }
         SIEVE_CUDA(timed(SIEVE_K_FINALIZE, [&] { return launch_finalize(a, st); }));
     }
@@ -538,8 +590,13 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         for (int i = 0; i < SIEVE_NKERNELS; ++i) stats->kernel_ms[i] = ms[i];
         const int per_round[] = {SIEVE_K_ISSUE, SIEVE_K_BUCKET, SIEVE_K_SCATTER, SIEVE_K_SCAN,
                                  SIEVE_K_MERGE, SIEVE_K_ROUND_END};
+        int prefix_mma = 0;
+        const int prefix_launches =
+            prefix && with_rank
+                ? rank_prefix_launches(a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma) : 0;
         stats->kernel_launches[SIEVE_K_RANK] =
             !with_rank ? 0
+            : prefix   ? prefix_launches
             : rank_tc ? rank_tc_launches(a.nq, a.nlist, a.nprobe, a.d, 0,
                                          a.tc_cent && rank_bulk_stages(a.d) > 0)
                       : 1;
@@ -549,7 +606,8 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         stats->kernel_launches[SIEVE_K_SCAN_TC] = a.tc_min > 0 ? c.round : 0;
         stats->kernel_launches[SIEVE_K_RQ_ROTATE] = a.rq ? 1 : 0;
         stats->kernel_launches[SIEVE_K_RANK_MMA] =
-            with_rank && rank_tc ? rank_tc_mma_launches(a.nq, a.nlist, a.nprobe, a.d, 0,
+            prefix && with_rank ? prefix_mma
+            : with_rank && rank_tc ? rank_tc_mma_launches(a.nq, a.nlist, a.nprobe, a.d, 0,
                                                          a.tc_cent && rank_bulk_stages(a.d) > 0)
                                   : 0;
         if (a.tc_min == 1) stats->kernel_launches[SIEVE_K_SCAN] = 0;
@@ -882,7 +940,9 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
     const int64_t chunk = round_up(ceil_div(nq, kHostChunks), wave);
     const int nchunks = p->profile ? 0 : (int)std::min<int64_t>(kHostChunks, ceil_div(nq, chunk));
     const bool rank_tc = p->scan_path != 1 && L.rank_scratch != 0;
+    const bool prefix = rank_tc && nchunks > 0 && use_prefix(ix, nq, p);
     SIEVE_CUDA(rank_tc ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
+    if (prefix) SIEVE_CUDA(prepare_rank_prefix(ix->nlist, p->nprobe, p->W, ix->d));
     SIEVE_CUDA(cudaMemsetAsync(dstatus, 0, sizeof(int), st));
     SIEVE_CUDA(cudaEventRecord(cl.start, st));             // earlier work on the staging
     SIEVE_CUDA(cudaStreamWaitEvent(cl.stream, cl.start, 0));
@@ -905,6 +965,15 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
     for (int c = 0; c < nchunks; ++c) {
         const int64_t q0 = c * chunk, n = std::min<int64_t>(chunk, nq - q0);
         SIEVE_CUDA(cudaStreamWaitEvent(st, cl.landed[c], 0));
+        if (prefix) {
+            SIEVE_CUDA(enqueue_rank_prefix(dQ, q0, n, nq, ix->centroids, ix->nlist, ix->d, p->nprobe, p->W,
+                                           dorder, nullptr, w + L.rank_scratch, dstatus,
+                                           static_cast<const unsigned char *>(ix->tc_centroids), st));
+            int mma = 0;
+            rank_launches += rank_prefix_launches(n, nq, ix->nlist, p->nprobe, p->W, ix->d, &mma);
+            mma_launches += mma;
+            continue;
+        }
         if (rank_tc)
             SIEVE_CUDA(enqueue_rank_tc(dQ + q0 * ix->d, n, ix->centroids, ix->nlist, ix->d, p->nprobe,
                                        dorder + q0 * p->nprobe, nullptr,
@@ -919,7 +988,7 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
         mma_launches += rank_tc ? rank_tc_mma_launches(n, ix->nlist, p->nprobe, ix->d, nq, bulk) : 0;
     }
     rc = search_device(ix, dQ, nq, dqids, nchunks ? dorder : nullptr, p, dids, dsc, dcnt, dpr, stats,
-                       w, L, st);
+                       w, L, st, nullptr, nullptr, prefix);
     if (rc != SIEVE_OK) return rc;
     SIEVE_CUDA(cudaMemcpyAsync(out_ids_host, dids, (size_t)nq * p->k * 8, cudaMemcpyDeviceToHost, st));
     SIEVE_CUDA(cudaMemcpyAsync(out_scores_host, dsc, (size_t)nq * p->k * 4, cudaMemcpyDeviceToHost, st));

@@ -32,9 +32,11 @@ struct Ctl {
     int round;         // rounds finished
     int status;        // 0 or a SIEVE_E* code
     int more;          // 1 while another round is needed
+    int ext_n;         // queries whose ranking the end of this round extends
+    int n_ext;         // the same, counted while the round issues
     int n_tc_tiles;    // tensor-core scan tiles this round
     int tc_tile_next;  // tensor-core scan work counter
-    int pad[5];
+    int pad[3];
     unsigned long long tot_items, tot_groups, tot_tiles, tot_rows, tot_pairs;
     unsigned long long tot_rows_tc, tot_pairs_tc;   // the tensor-core share of the two above
 };

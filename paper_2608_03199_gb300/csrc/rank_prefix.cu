@@ -1,0 +1,631 @@
+// rank_prefix.cu -- the first ranks of the centroid order alone (Sec. 2.3,
+// Sec. 4.1), for a search whose stopping rule visits few of its nprobe ranks.
+//
+// A search with a window of W visits min(W, nprobe) partitions plus what its
+// hits add: about 8 of 256 ranks at W = 8.  So the search ranks a prefix
+// first, and only the queries whose stop line passes their prefix get the
+// whole ranking (the extension at the end of a round, below).
+//
+//   k_prefix_scan   one contraction pass on the screen (one fp16 product of
+//              the hi halves per score, tiles of two 128-query sub-tiles).
+//              Each epilogue thread owns one query and keeps its kL largest
+//              screened scores with their centroid ids, unordered, in shared
+//              memory.  An entry costs about 500 cycles of its warp and holds
+//              the accumulator meanwhile, so the tile first passes over an
+//              eighth of its chunks and keeps only the kL largest group
+//              maxima, in registers and without a branch: kL centroids reach
+//              the kL-th, and starting from there a list takes about
+//              kL (1 + ln 8) entries instead of kL (1 + ln(nlist / kL)) in a
+//              random order (1M queries x 8,192 x 256, kL = 16: 6.1 -> 5.7 ms).
+//   k_prefix_final  one warp per query: the kept centroids scored again in
+//              fp32 and sorted by (score desc, id asc).  A centroid that was
+//              not kept screens at most u, the largest of the lists'
+//              thresholds, so its fp32 score is below u plus the error
+//              bounds of both scores; the kept centroids above that are
+//              exactly the first ranks of the order, and their number is the
+//              query's limit.
+//   k_ext_gather / k_ext_merge  the extension: the listed queries gathered
+//              for the full ranking, whose order follows the prefix with the
+//              prefix's centroids left out, so that no partition is visited
+//              twice should the two disagree on a near-tie.
+//
+// Bound by the epilogue's entries (about half of the 32-score groups have one,
+// in some lane) and the single accumulator per sub-tile they hold meanwhile.
+// Against the full ranking (two contraction passes, ~310 candidates a query
+// sorted): 1M queries x 65,536 x 96, nprobe 256, 52.1 -> 25.0 ms; 1M x 8,192 x
+// 256, nprobe 128, 17.6 -> 7.7 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.35 ms.
+#include <cmath>
+#include <vector>
+
+#include "rank_select.cuh"
+#include "tc_bulk.cuh"
+
+namespace sieve {
+
+struct PrefixArgs {
+    const float *Q;
+    int64_t nq, nlist;
+    int d;
+    int *status;
+    const unsigned char *tc_cent;
+    int nranges;         // centroid ranges per query tile
+    int64_t range_len;   // centroids per range, a multiple of 128
+    float *list_s;       // [nq][nranges][kL] kept screened scores ...
+    int32_t *list_i;     // ... and their centroids (-1: an unused entry)
+    float *list_t;       // [nq][nranges] what a score left out can be at most (-inf: none was)
+};
+
+__device__ int g_prefix_status_sink;
+
+template <int kL, int kNBT>
+struct PrefixMode {
+    using Args = PrefixArgs;
+    static constexpr int kProducts = 1;
+    static constexpr int kNB = kNBT;
+    static constexpr int kSub = 2;
+    static constexpr int kRows = kSub * tcp::kM;
+    static constexpr bool kSampled = true;
+    struct Tile {
+        int64_t q0;
+        int ni;
+        int64_t c0, nb;
+        int ns, sstep;   // sample chunks first: chunks 0, sstep, 2 sstep, ...
+    };
+    __device__ static int num_tiles(const Args &a) { return (int)ceil_div(a.nq, kRows) * a.nranges; }
+    __device__ static int *tile_counter(const Args &) { return nullptr; }
+    __device__ static int d(const Args &a) { return a.d; }
+    __device__ static int *status(const Args &a) { return a.status ? a.status : &g_prefix_status_sink; }
+    __device__ static Tile tile(const Args &a, int t) {
+        Tile T;
+        T.q0 = (int64_t)(t / a.nranges) * kRows;
+        T.ni = (int)(a.nq - T.q0 < kRows ? a.nq - T.q0 : kRows);
+        T.c0 = (int64_t)(t % a.nranges) * a.range_len;
+        T.nb = a.nlist - T.c0 < a.range_len ? a.nlist - T.c0 : a.range_len;
+        // an eighth of the whole chunks where there are 16 or more
+        const int whole = (int)(T.nb / kNBT);
+        T.ns = whole >= 16 ? whole / 8 : 0;
+        T.sstep = 8;
+        return T;
+    }
+    __device__ static const float *a_row(const Args &a, const Tile &T, int i) {
+        return i < T.ni ? a.Q + (T.q0 + i) * a.d : nullptr;
+    }
+    __device__ static const unsigned char *b_block(const Args &a, const Tile &T) {
+        return a.tc_cent + (T.c0 / kTcRows) * (int64_t)((a.d + 63) / 64) * kTcBlockBytes;
+    }
+    struct Epi {
+        float *ks;      // entry j of this query's list at [j * kRows]
+        int32_t *ki;
+        int64_t at;
+        int n, pos;     // entries in the list; the smallest one's place once it is full
+        float thr;      // raw units: scores up to it are out (-inf: none yet; +inf: no query)
+        bool valid;
+        float top[kL];  // the sample's kL largest group maxima, largest first
+        __device__ void begin(const Args &a, const Tile &T, int slot, unsigned char *smem) {
+            ks = reinterpret_cast<float *>(smem) + slot;
+            ki = reinterpret_cast<int32_t *>(smem + (size_t)kRows * kL * 4) + slot;
+            valid = slot < T.ni;
+            at = (T.q0 + slot) * a.nranges + T.c0 / a.range_len;
+            n = 0;
+            pos = 0;
+            thr = valid ? -__int_as_float(0x7f800000) : __int_as_float(0x7f800000);
+#pragma unroll
+            for (int j = 0; j < kL; ++j) top[j] = -__int_as_float(0x7f800000);
+        }
+        // a sample chunk's scores: the maximum of each 16 into the sorted
+        // registers, without a branch (whole chunks only: no column is past
+        // the range)
+        __device__ __forceinline__ void sample(const float (&v)[32]) {
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                float x = fmax3f(fmax3f(v[16 * g], v[16 * g + 1], v[16 * g + 2]),
+                                 fmax3f(v[16 * g + 3], v[16 * g + 4], v[16 * g + 5]),
+                                 fmax3f(v[16 * g + 6], v[16 * g + 7], v[16 * g + 8]));
+                x = fmax3f(x, fmax3f(v[16 * g + 9], v[16 * g + 10], v[16 * g + 11]),
+                           fmax3f(fmaxf(v[16 * g + 12], v[16 * g + 13]), v[16 * g + 14], v[16 * g + 15]));
+#pragma unroll
+                for (int j = 0; j < kL; ++j) {
+                    const float hi = fmaxf(top[j], x);
+                    x = fminf(top[j], x);
+                    top[j] = hi;
+                }
+            }
+        }
+        // the sample is through: kL different centroids reach top[kL - 1], so
+        // only scores from there up are listed (the threshold is the value
+        // just below it; the list then fills)
+        __device__ __forceinline__ void seed() {
+            const float t = top[kL - 1];
+            if (valid && t > -3.402823466e38f && t < 3.402823466e38f)
+                thr = t - fmaxf(fabsf(t), 1.f) * 0x1p-22f;
+        }
+        __device__ __forceinline__ void find_smallest() {
+            float w[kL];
+#pragma unroll
+            for (int j = 0; j < kL; ++j) w[j] = ks[j * kRows];
+            float t = w[0];
+#pragma unroll
+            for (int j = 1; j < kL; ++j) t = fminf(t, w[j]);
+            int p = 0;
+#pragma unroll
+            for (int j = 1; j < kL; ++j) p = w[j] == t ? j : p;
+            thr = t;
+            pos = p;
+        }
+        // v: the chunk's raw accumulator values (scores x 2^16) of centroids
+        // T.c0 + col0 + j, j < ncol (warp-uniform)
+        __device__ __forceinline__ void chunk(const Args &, const Tile &T, int64_t col0,
+                                              const float (&v)[32], int ncol) {
+            if (ncol <= 0) return;
+            float mx = v[0];
+            if (ncol == 32) {
+                mx = max_of_32(v);
+            } else {
+#pragma unroll
+                for (int j = 1; j < 32; ++j) mx = j < ncol ? fmaxf(mx, v[j]) : mx;
+            }
+            const bool any = mx > thr;
+            if (!__any_sync(0xffffffffu, any)) return;
+            unsigned m = 0;
+            if (any) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) m |= v[j] > thr ? (1u << j) : 0u;
+                if (ncol < 32) m &= (1u << ncol) - 1u;
+            }
+            const int32_t id0 = (int32_t)(T.c0 + col0);
+            while (m) {
+                const int j = __ffs(m) - 1;
+                m &= m - 1u;
+                const float x = pick32(v, j);
+                if (!(x > thr)) continue;   // the threshold rose within this group
+                const int p = n < kL ? n : pos;
+                ks[p * kRows] = x;
+                ki[p * kRows] = id0 + j;
+                if (n < kL) ++n;
+                if (n == kL) find_smallest();
+            }
+            __syncwarp();
+        }
+        __device__ void end(const Args &a, const Tile &) {
+            if (!valid) return;
+            a.list_t[at] = thr * (1.f / 65536.f);
+            float4 *os = reinterpret_cast<float4 *>(a.list_s + at * kL);
+            int4 *oi = reinterpret_cast<int4 *>(a.list_i + at * kL);
+#pragma unroll
+            for (int j = 0; j < kL; j += 4) {
+                float s[4];
+                int32_t c[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    s[u] = j + u < n ? ks[(j + u) * kRows] * (1.f / 65536.f) : 0.f;
+                    c[u] = j + u < n ? ki[(j + u) * kRows] : -1;
+                }
+                os[j / 4] = make_float4(s[0], s[1], s[2], s[3]);
+                oi[j / 4] = make_int4(c[0], c[1], c[2], c[3]);
+            }
+        }
+        __device__ void prefetch(const Args &, const Tile &, int) {}
+        __device__ void start(const Args &, const Tile &, int) {}
+    };
+};
+
+template <int kL, int kNBT>
+__global__ void __launch_bounds__(tcb::kThreads, 1) k_prefix_scan(PrefixArgs a, int stages) {
+    extern __shared__ unsigned char smem_raw[];
+    tcb::run_bulk<PrefixMode<kL, kNBT>>(a, smem_raw, stages);
+}
+
+// One warp per query.  NT: float4 of a row per lane of a group of eight (d <=
+// 32 NT); KPL: list entries per lane (nranges * kL <= 32 KPL).
+constexpr int kFinalWarps = 8;
+template <int kL, int KPL, int NT>
+__global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
+    const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int d,
+    const float *__restrict__ list_s, const int32_t *__restrict__ list_i,
+    const float *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits, int32_t *__restrict__ order, float *__restrict__ cscores,
+    int *__restrict__ limit) {
+    __shared__ int s_id[kFinalWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t q = (int64_t)blockIdx.x * kFinalWarps + warp;
+    if (q >= nq) return;
+    const int M = nranges * kL;
+    const float *ls = list_s + q * M;
+    const int32_t *li = list_i + q * M;
+    uint32_t key[KPL];
+    uint32_t un = 0;   // the largest screened score a centroid outside the candidates can have
+#pragma unroll
+    for (int j = 0; j < KPL; ++j) {
+        const int c = j * 32 + lane;
+        key[j] = (c < M && li[c] >= 0) ? order_key(ls[c]) : 0u;
+    }
+    for (int r = lane; r < nranges; r += 32) {
+        const float t = list_t[q * nranges + r];
+        if (t > -__int_as_float(0x7f800000)) un = max(un, order_key(t));
+    }
+    // the candidates, one per lane: every entry, or the kL largest of several lists
+    int id = -1, n = 0;
+    bool fits = true;
+    if constexpr (KPL == 1) {
+        id = key[0] ? li[lane] : -1;
+        n = M < 32 ? M : 32;
+    } else {
+        uint32_t T;
+        int C32;
+        warp_threshold(key, kL, 32, T, C32);
+        T = max(T, 1u);
+        const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) {
+            const bool sel = key[j] >= T;
+            const unsigned b = __ballot_sync(0xffffffffu, sel);
+            const int p = n + __popc(b & below);
+            if (sel && p < 32) s_id[warp][p] = li[j * 32 + lane];
+            if (!sel) un = max(un, key[j]);
+            n += __popc(b);
+        }
+        fits = n <= 32;   // more: equal scores at the threshold
+        n = n < 32 ? n : 32;
+        __syncwarp();
+        if (lane < n) id = s_id[warp][lane];
+    }
+    un = __reduce_max_sync(0xffffffffu, un);
+    // fp32 scores: eight lanes per candidate, four candidates at a time
+    const int g = lane >> 3, sub = lane & 7;
+    float4 x[NT];
+    float qq = 0.f;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        const int c = 4 * sub + 32 * t;
+        x[t] = c < d ? __ldg(reinterpret_cast<const float4 *>(Q + q * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        qq = fmaf(x[t].x, x[t].x, fmaf(x[t].y, x[t].y, fmaf(x[t].z, x[t].z, fmaf(x[t].w, x[t].w, qq))));
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) qq += __shfl_xor_sync(0xffffffffu, qq, o);
+    float s[1] = {-__int_as_float(0x7f800000)};
+    int cid[1] = {id >= 0 ? id : INT32_MAX};
+#pragma unroll 2
+    for (int it = 0; it < (n + 3) / 4; ++it) {
+        const int ci = __shfl_sync(0xffffffffu, id, it * 4 + g);
+        float acc = 0.f;
+        if (ci >= 0) {
+            const float *row = C + (int64_t)ci * d;
+            float4 y[NT];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const int c = 4 * sub + 32 * t;
+                y[t] = c < d ? __ldg(reinterpret_cast<const float4 *>(row + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                acc = fmaf(x[t].x, y[t].x, acc);
+                acc = fmaf(x[t].y, y[t].y, acc);
+                acc = fmaf(x[t].z, y[t].z, acc);
+                acc = fmaf(x[t].w, y[t].w, acc);
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        const float mine = __shfl_sync(0xffffffffu, acc, (lane & 3) * 8);
+        if ((lane >> 2) == it && id >= 0) s[0] = mine;
+    }
+    warp_sort_regs<1>(s, cid);
+    // the norms and the margin rounded upward (the bounds of k_rank_threshold:
+    // the screen's, and one that covers fp32 sums with room)
+    const float qn = __fsqrt_ru(qq) * (1.f + 0x1p-20f);
+    const float cn = __uint_as_float(*cmax_bits) * (1.f + 0x1p-20f);
+    const float rd = __fsqrt_ru((float)d);
+    const float fp32 = (0x1p-20f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
+    const float scr = (0x1p-10f + 0x1p-12f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
+    const float margin = (scr + fp32) * (1.f + 0x1p-16f);
+    // scores past fp16's range (|256 x| above 65,504) are not screened soundly
+    const bool sound = fits && qn < 200.f && cn < 200.f;
+    const bool first = sound && cid[0] != INT32_MAX &&
+                       (un == 0u || s[0] > __fadd_ru(key_score(un), margin));
+    const unsigned b = __ballot_sync(0xffffffffu, first);
+    int R = b == 0xffffffffu ? 32 : __ffs(~b) - 1;   // the sorted entries up to the first that may not be
+    R = R < nprobe ? R : nprobe;
+    if (lane < R) {
+        order[q * nprobe + lane] = cid[0];
+        if (cscores) cscores[q * nprobe + lane] = s[0];
+    }
+    if (lane == 0) limit[q] = R;
+}
+
+// row i of Qx = query ext[q0 + i] (a warp per row), for the listed queries of this chunk
+__global__ void k_ext_gather(const float *__restrict__ Q, int d, const int *__restrict__ ext,
+                             const int *__restrict__ ext_n, int64_t q0, int64_t chunk,
+                             float *__restrict__ Qx) {
+    const int64_t left = (int64_t)*ext_n - q0, n = left < chunk ? left : chunk;
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+        const float *src = Q + (int64_t)ext[q0 + i] * d;
+        for (int c = 4 * lane; c < d; c += 128)
+            *reinterpret_cast<float4 *>(Qx + i * d + c) = *reinterpret_cast<const float4 *>(src + c);
+    }
+}
+
+// A warp per listed query: ranks limit + 1 .. nprobe of its order become the
+// full ranking's centroids, in order, without the limit[q] <= 32 of its prefix.
+__global__ void k_ext_merge(const int *__restrict__ ext, const int *__restrict__ ext_n, int64_t q0,
+                            int64_t chunk, int nprobe, const int32_t *__restrict__ full,
+                            const float *__restrict__ full_s, int32_t *__restrict__ order,
+                            float *__restrict__ cscores, int *__restrict__ limit) {
+    const int64_t left = (int64_t)*ext_n - q0, n = left < chunk ? left : chunk;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+        const int64_t q = ext[q0 + i];
+        const int R = limit[q];
+        const int32_t mine = lane < R ? order[q * nprobe + lane] : -1;
+        int at = R;
+        for (int p0 = 0; p0 < nprobe && at < nprobe; p0 += 32) {
+            const int p = p0 + lane;
+            const int32_t c = p < nprobe ? full[i * nprobe + p] : -2;
+            bool keep = p < nprobe;
+            for (int r = 0; r < R; ++r) {   // every lane takes part in each shuffle
+                const int32_t pr = __shfl_sync(0xffffffffu, mine, r);
+                keep = keep && c != pr;
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, keep);
+            const int o = at + __popc(b & below);
+            if (keep && o < nprobe) {
+                order[q * nprobe + o] = c;
+                if (cscores) cscores[q * nprobe + o] = full_s[i * nprobe + p];
+            }
+            at += __popc(b);
+        }
+        __syncwarp();
+        if (lane == 0) limit[q] = nprobe;
+    }
+}
+
+// ---------------------------------------------------------------------------
+static bool prefix_wide(int d) { return ceil_div(d, 64) <= 2; }   // 192-centroid chunks, as the screen
+static uint32_t prefix_stage_bytes(int d) {
+    return prefix_wide(d) ? tcb::kStageBytesHi / tcb::kN * 192 : tcb::kStageBytesHi;
+}
+static size_t prefix_epi_bytes(int L) { return (size_t)2 * tcp::kM * L * 8; }
+
+static int prefix_stages(int d, int L) {
+    const int nkb = (int)ceil_div(d, 64);
+    return tcb::sub_fits(nkb, 1, 2)
+               ? tcb::stages_for(nkb, prefix_epi_bytes(L), 232448 - 128, prefix_stage_bytes(d))
+               : 0;
+}
+
+// Entries kept per list: min(W, nprobe) ranks are visited for certain, a hit at
+// rank j adds up to rank j + W, and one or two entries are lost to the margin.
+// 16 entries serve windows up to 10 and 32 up to 24; 0: rank all of nprobe (a
+// wider window reads most of the order anyway, and a list of fewer than 64
+// centroids is ranked whole as cheaply).
+static bool prefix_fits(int64_t nlist, int nprobe, int d, int L) {
+    return nlist >= 4 * (int64_t)L && nprobe >= 4 && prefix_stages(d, L) > 0;
+}
+
+int rank_prefix_len(int64_t nlist, int nprobe, int W, int d) {
+    const int need = W < nprobe ? W : nprobe;
+    const int L = need <= 10 ? 16 : need <= 24 ? 32 : 0;
+    return L && prefix_fits(nlist, nprobe, d, L) ? L : 0;
+}
+
+struct PrefixPlan {
+    int nranges;
+    int64_t range_len;
+};
+
+// Ranges: enough tiles to fill the SMs in whole waves.  A tile costs its chunks
+// plus about six chunks' time for writing A and filling the lists.
+static PrefixPlan prefix_plan(int64_t nq, int64_t nlist, int d, int L) {
+    const int64_t tiles = std::max<int64_t>(1, ceil_div(nq, 2 * tcp::kM)), sms = num_sms();
+    const int64_t nb = prefix_wide(d) ? 192 : 128;
+    const int64_t most = std::min<int64_t>(ceil_div(nlist, kTcRows), std::min<int64_t>(1024 / L, 32));
+    PrefixPlan best{1, round_up(nlist, (int64_t)kTcRows)};
+    int64_t best_cost = INT64_MAX;
+    for (int64_t r = 1; r <= most; ++r) {
+        const int64_t len = round_up(ceil_div(nlist, r), (int64_t)kTcRows), nr = ceil_div(nlist, len);
+        const int64_t cost = ceil_div(tiles * nr, sms) * (ceil_div(len, nb) + 6);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = PrefixPlan{(int)nr, len};
+        }
+        if (tiles * r >= 16 * sms) break;
+    }
+    return best;
+}
+
+// Layout of the ranking scratch of a search with a prefix: the limits and the
+// extension list (kept for the whole search), then the lists of a chunk of
+// queries (the prefix) or the extension's buffers, which are never live at once.
+struct PrefixScratch {
+    int64_t limit, ext, rest;      // byte offsets
+    int64_t chunk;                 // queries per prefix pass
+    int64_t ext_chunk;             // queries per extension pass
+    int64_t ext_q, ext_order, ext_s;   // byte offsets of the extension's buffers (after its ranking scratch)
+    int64_t total;
+};
+
+static int64_t ext_bytes(int64_t x, int64_t nlist, int nprobe, int d, PrefixScratch *S) {
+    int64_t off = S->rest + round_up((int64_t)rank_tc_scratch_bytes(x, nlist, nprobe, d), 256);
+    S->ext_q = off;
+    off += round_up(x * d * 4, 256);
+    S->ext_order = off;
+    off += round_up(x * nprobe * 4, 256);
+    S->ext_s = off;
+    off += round_up(x * nprobe * 4, 256);
+    return off;
+}
+
+// The scratch stays within what the full ranking takes (plain) wherever a
+// chunk of queries fits it; a smaller chunk only means more passes.
+static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d, int L) {
+    PrefixScratch S{};
+    const int64_t plain = (int64_t)rank_tc_scratch_bytes(nq, nlist, nprobe, d);
+    S.limit = 0;
+    S.ext = round_up(nq * 4, 256);
+    S.rest = S.ext + round_up(nq * 4, 256);
+    S.ext_chunk = nq;
+    int64_t end = ext_bytes(nq, nlist, nprobe, d, &S);
+    while (end > plain && S.ext_chunk > 128) {
+        S.ext_chunk = std::max<int64_t>(128, round_up(ceil_div(S.ext_chunk, 2), 128));
+        end = ext_bytes(S.ext_chunk, nlist, nprobe, d, &S);
+    }
+    S.total = std::max(end, plain);
+    const PrefixPlan P = prefix_plan(nq, nlist, d, L);
+    const int64_t per = (int64_t)P.nranges * (L * 8 + 4);
+    S.total = std::max(S.total, S.rest + std::min<int64_t>(nq, 2 * tcp::kM) * per + 512);
+    S.chunk = std::min(nq, std::max<int64_t>(2 * tcp::kM, (S.total - S.rest - 512) / per / (2 * tcp::kM) * (2 * tcp::kM)));
+    return S;
+}
+
+// for any window: a calibrated search sizes its workspace before it picks one
+size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int d) {
+    int64_t b = 0;
+    for (int L : {16, 32})
+        if (nq > 0 && prefix_fits(nlist, nprobe, d, L))
+            b = std::max(b, prefix_scratch(nq, nlist, nprobe, d, L).total);
+    return (size_t)b;
+}
+
+int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext) {
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    unsigned char *w = static_cast<unsigned char *>(scratch);
+    *ext = reinterpret_cast<int *>(w + S.ext);
+    return reinterpret_cast<int *>(w + S.limit);
+}
+
+template <int kL, int kNBT>
+static cudaError_t set_scan_attr(int d) {
+    return cudaFuncSetAttribute(
+        k_prefix_scan<kL, kNBT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)tcb::smem_bytes(prefix_stages(d, kL), prefix_epi_bytes(kL), prefix_stage_bytes(d)));
+}
+
+cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d) {
+    const int L = rank_prefix_len(nlist, nprobe, W, d);
+    if (prefix_wide(d)) return L == 16 ? set_scan_attr<16, 192>(d) : set_scan_attr<32, 192>(d);
+    return L == 16 ? set_scan_attr<16, 128>(d) : set_scan_attr<32, 128>(d);
+}
+
+template <int kL, int KPL>
+static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, const unsigned *cmax,
+                                int32_t *order, float *cscores, int *limit, cudaStream_t st) {
+    const unsigned blocks = (unsigned)ceil_div(a.nq, kFinalWarps);
+    if (a.d <= 128)
+        k_prefix_final<kL, KPL, 4><<<blocks, kFinalWarps * 32, 0, st>>>(
+            a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe, cmax, order, cscores, limit);
+    else
+        k_prefix_final<kL, KPL, 8><<<blocks, kFinalWarps * 32, 0, st>>>(
+            a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe, cmax, order, cscores, limit);
+}
+
+// kernel launches of one prefix ranking of nq queries (and its contraction
+// launches), for scratch sized for plan_nq
+int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma) {
+    const int L = rank_prefix_len(nlist, nprobe, W, d);
+    const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
+    const int chunks = (int)ceil_div(nq, S.chunk);
+    *mma = chunks;
+    return 2 * chunks + 1;
+}
+
+// The prefix of nq queries q0 .. q0 + nq - 1 of a batch of plan_nq (whose
+// scratch this is): order, cscores (nullable) and the scratch's limits.
+cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
+                                int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
+                                void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
+                                float *mma_ms) {
+    if (nq <= 0) return cudaSuccess;
+    const int L = rank_prefix_len(nlist, nprobe, W, d);
+    const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
+    const PrefixPlan P = prefix_plan(plan_nq, nlist, d, L);
+    unsigned char *w = static_cast<unsigned char *>(scratch);
+    int *limit = reinterpret_cast<int *>(w + S.limit);
+    unsigned *cmax = reinterpret_cast<unsigned *>(w + S.rest);
+    float *list_s = reinterpret_cast<float *>(w + S.rest + 256);
+    const int64_t slots = S.chunk * P.nranges * L;
+    int32_t *list_i = reinterpret_cast<int32_t *>(list_s + slots);
+    float *list_t = reinterpret_cast<float *>(list_i + slots);
+    const int stages = prefix_stages(d, L);
+    const size_t smem = tcb::smem_bytes(stages, prefix_epi_bytes(L), prefix_stage_bytes(d));
+    struct Events {
+        std::vector<cudaEvent_t> v;
+        ~Events() {
+            for (cudaEvent_t e : v) cudaEventDestroy(e);
+        }
+    } ev;
+    cudaError_t e = launch_cnorm_max(C, nlist, d, cmax, st);
+    if (e != cudaSuccess) return e;
+    for (int64_t b = 0; b < nq; b += S.chunk) {
+        const int64_t n = std::min(S.chunk, nq - b);
+        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, tc_cent, P.nranges, P.range_len, list_s, list_i, list_t};
+        const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 2 * tcp::kM) * P.nranges, num_sms());
+        if (mma_ms) {
+            ev.v.resize(ev.v.size() + 2);
+            cudaEventCreate(&ev.v[ev.v.size() - 2]);
+            cudaEventCreate(&ev.v.back());
+            cudaEventRecord(ev.v[ev.v.size() - 2], st);
+        }
+        if (prefix_wide(d)) {
+            if (L == 16) k_prefix_scan<16, 192><<<grid, tcb::kThreads, smem, st>>>(a, stages);
+            else k_prefix_scan<32, 192><<<grid, tcb::kThreads, smem, st>>>(a, stages);
+        } else {
+            if (L == 16) k_prefix_scan<16, 128><<<grid, tcb::kThreads, smem, st>>>(a, stages);
+            else k_prefix_scan<32, 128><<<grid, tcb::kThreads, smem, st>>>(a, stages);
+        }
+        if (mma_ms) cudaEventRecord(ev.v.back(), st);
+        int32_t *o = order + (q0 + b) * nprobe;
+        float *cs = cscores ? cscores + (q0 + b) * nprobe : nullptr;
+        int *lim = limit + q0 + b;
+        const int kpl = (int)ceil_div(P.nranges * L, 32);
+#define SIEVE_PREFIX(K)                                                                       \
+    if (L == 16) launch_prefix_final<16, K>(a, C, nprobe, cmax, o, cs, lim, st);               \
+    else launch_prefix_final<32, K>(a, C, nprobe, cmax, o, cs, lim, st)
+        if (kpl <= 1) { SIEVE_PREFIX(1); }
+        else if (kpl <= 2) { SIEVE_PREFIX(2); }
+        else if (kpl <= 4) { SIEVE_PREFIX(4); }
+        else if (kpl <= 8) { SIEVE_PREFIX(8); }
+        else if (kpl <= 16) { SIEVE_PREFIX(16); }
+        else { SIEVE_PREFIX(32); }
+#undef SIEVE_PREFIX
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (mma_ms) {
+        e = cudaStreamSynchronize(st);
+        for (size_t i = 0; i + 1 < ev.v.size(); i += 2) {
+            float t = 0.f;
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&t, ev.v[i], ev.v[i + 1]);
+            *mma_ms += t;
+        }
+    }
+    return e;
+}
+
+// The extension: the full ranking of the queries ext[0 .. *ext_n - 1], behind
+// their prefixes.  Every pass is launched; passes past *ext_n find no work.
+cudaError_t enqueue_rank_ext(const float *Q, int64_t nq, const float *C, int64_t nlist, int d, int nprobe,
+                             int W, int32_t *order, float *cscores, void *scratch, const int *ext_n,
+                             int *status, const unsigned char *tc_cent, cudaStream_t st) {
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    unsigned char *w = static_cast<unsigned char *>(scratch);
+    int *limit = reinterpret_cast<int *>(w + S.limit);
+    const int *ext = reinterpret_cast<const int *>(w + S.ext);
+    float *Qx = reinterpret_cast<float *>(w + S.ext_q);
+    int32_t *full = reinterpret_cast<int32_t *>(w + S.ext_order);
+    float *full_s = cscores ? reinterpret_cast<float *>(w + S.ext_s) : nullptr;
+    const int blocks = 4 * num_sms();
+    for (int64_t b = 0; b < nq; b += S.ext_chunk) {
+        const int64_t n = std::min(S.ext_chunk, nq - b);
+        k_ext_gather<<<blocks, 256, 0, st>>>(Q, d, ext, ext_n, b, n, Qx);
+        cudaError_t e = enqueue_rank_tc(Qx, n, C, nlist, d, nprobe, full, full_s,
+                                        reinterpret_cast<float *>(w + S.rest), status, st, tc_cent, nullptr,
+                                        S.ext_chunk, ext_n, b);
+        if (e != cudaSuccess) return e;
+        k_ext_merge<<<blocks, 256, 0, st>>>(ext, ext_n, b, n, nprobe, full, full_s, order, cscores, limit);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace sieve

@@ -33,22 +33,11 @@
 #include <cmath>
 #include <vector>
 
+#include "rank_select.cuh"
 #include "tc_bulk.cuh"
 #include "tc_pipeline.cuh"
 
 namespace sieve {
-
-// selection: monotone map of fp32 to uint32 (larger float -> larger key); -0
-// is mapped as +0 so that equal scores have equal keys
-__device__ __forceinline__ uint32_t order_key(float s) {
-    const uint32_t u = __float_as_uint(s + 0.f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// the inverse of order_key
-__device__ __forceinline__ float key_score(uint32_t k) {
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
 
 // Running-threshold histogram: 256 bins of width 1/128 over scores in
 // [-1, 1); scores outside fall into the end bins.  In raw accumulator units
@@ -94,7 +83,16 @@ struct RankArgs {
     float *gmax;     // kRankGroupMax: [nq][gld] group maxima (score units)
     int64_t gld;
     int group;       // kRankGroupMax: centroids per group, 32 or 64
+    const int *n_dev;   // nullable: only the first *n_dev - n_off of the nq queries exist
+    int64_t n_off;
 };
+
+// the queries of a launch sized for nq whose count is known on the device
+__device__ __forceinline__ int64_t queries_of(int64_t nq, const int *n_dev, int64_t n_off) {
+    if (!n_dev) return nq;
+    const int64_t n = (int64_t)*n_dev - n_off;
+    return n < 0 ? 0 : (n < nq ? n : nq);
+}
 
 __device__ int g_rank_status_sink;
 
@@ -114,7 +112,9 @@ struct RankModeT {
         int64_t c0;    // first centroid of the tile's range
         int64_t nb;    // centroids in the range
     };
-    __device__ static int num_tiles(const Args &a) { return (int)ceil_div(a.nq, kRows) * a.nranges; }
+    __device__ static int num_tiles(const Args &a) {
+        return (int)ceil_div(queries_of(a.nq, a.n_dev, a.n_off), kRows) * a.nranges;
+    }
     // every tile costs about the same: a static stride over the blocks
     __device__ static int *tile_counter(const Args &) { return nullptr; }
     __device__ static int d(const Args &a) { return a.d; }
@@ -122,7 +122,8 @@ struct RankModeT {
     __device__ static Tile tile(const Args &a, int t) {
         Tile T;
         T.q0 = (int64_t)(t / a.nranges) * kRows;
-        T.ni = (int)(a.nq - T.q0 < kRows ? a.nq - T.q0 : kRows);
+        const int64_t left = queries_of(a.nq, a.n_dev, a.n_off) - T.q0;
+        T.ni = (int)(left < kRows ? left : kRows);
         T.c0 = (int64_t)(t % a.nranges) * a.range_len;
         T.nb = a.nlist - T.c0 < a.range_len ? a.nlist - T.c0 : a.range_len;
         return T;
@@ -343,144 +344,6 @@ __global__ void __launch_bounds__(tcb::kThreads, 1) k_rank_screen192(RankArgs a,
 }
 
 constexpr int kSelectWarps = 4;  // warps (queries) per block of the final selection
-constexpr int kSelectMaxR = 8;   // lane order statistics used for the lower bracket
-
-// warp-wide reductions in one instruction (redux.sync), not a chain of shuffles
-__device__ __forceinline__ int warp_sum(int x) { return __reduce_add_sync(0xffffffffu, x); }
-
-template <int KPL>
-__device__ __forceinline__ int count_ge(const uint32_t (&key)[KPL], uint32_t t) {
-    int c = 0;
-#pragma unroll
-    for (int j = 0; j < KPL; ++j) c += key[j] >= t;
-    return warp_sum(c);
-}
-
-// A bracket L <= T* <= U of the want-th largest of the warp's keys (keys of
-// padding are 0, below every score): U = the largest key, L = the smallest over
-// lanes of each lane's ceil(want / 32)-th largest key, so at least want keys
-// are >= L.  L = 0 when that rank is past kSelectMaxR.
-template <int KPL>
-__device__ __forceinline__ void warp_bracket(const uint32_t (&key)[KPL], int want, uint32_t &L,
-                                             uint32_t &U) {
-    const int r = (want + 31) / 32;
-    uint32_t m[kSelectMaxR] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    if (r <= 2) {
-#pragma unroll
-        for (int j = 0; j < KPL; ++j) {
-            m[1] = max(m[1], min(m[0], key[j]));
-            m[0] = max(m[0], key[j]);
-        }
-    } else if (r <= 4) {
-#pragma unroll
-        for (int j = 0; j < KPL; ++j) {
-            uint32_t x = key[j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t hi = max(m[i], x);
-                x = min(m[i], x);
-                m[i] = hi;
-            }
-        }
-    } else if (r <= kSelectMaxR) {
-#pragma unroll
-        for (int j = 0; j < KPL; ++j) {
-            uint32_t x = key[j];
-#pragma unroll
-            for (int i = 0; i < kSelectMaxR; ++i) {
-                const uint32_t hi = max(m[i], x);
-                x = min(m[i], x);
-                m[i] = hi;
-            }
-        }
-    } else {   // no lower bracket, but U is still the largest key
-#pragma unroll
-        for (int j = 0; j < KPL; ++j) m[0] = max(m[0], key[j]);
-    }
-    L = 0u;
-#pragma unroll
-    for (int i = 0; i < kSelectMaxR; ++i) L = r == i + 1 ? m[i] : L;
-    U = __reduce_max_sync(0xffffffffu, m[0]);
-    L = __reduce_min_sync(0xffffffffu, L);
-}
-
-// A threshold T <= T* (T* = the want-th largest of the warp's keys) with C =
-// #{keys >= T} >= want, refined bit by bit (the largest T with at least want
-// keys >= T) until C <= cap or T == T*.  The search starts from the common
-// high bits of the bracket L, U.
-template <int KPL>
-__device__ __forceinline__ void warp_threshold(const uint32_t (&key)[KPL], int want, int cap,
-                                               uint32_t &T, int &C) {
-    uint32_t L, U;
-    warp_bracket(key, want, L, U);
-    int b;
-    if (L == U) {
-        b = -1;
-        T = L;
-    } else {
-        b = 31 - __clz(L ^ U);                                // highest bit where they differ
-        T = b == 31 ? 0u : (L & ~((2u << b) - 1u));           // their common high bits
-    }
-    C = count_ge(key, T);
-    for (; b >= 0 && C > cap; --b) {
-        const uint32_t t = T | (1u << b);
-        const int c = count_ge(key, t);
-        if (c >= want) {
-            T = t;
-            C = c;
-        }
-    }
-}
-
-// Bitonic sort of the warp's R * 32 entries (entry i = r * 32 + lane in
-// register r), first-ranked first by (score desc, id asc).  Partners within a
-// register are exchanged by shuffles, partners across registers in place.
-// Entries are distinct except identical padding, so both sides of a pair
-// take the same decision.
-template <int R>
-__device__ __forceinline__ void warp_sort_regs(float (&s)[R], int (&c)[R]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 2; k <= 32 * R; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-                const int jr = j >> 5;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if (r & jr) continue;
-                    const int r2 = r | jr;
-                    const bool up = ((r * 32) & k) == 0;   // this block sorts first-ranked first
-                    // the lower entry keeps the better one when up, else the worse
-                    const bool swap = up ? ranks_before(s[r2], c[r2], s[r], c[r])
-                                         : ranks_before(s[r], c[r], s[r2], c[r2]);
-                    if (swap) {
-                        const float ts = s[r];
-                        const int tc = c[r];
-                        s[r] = s[r2];
-                        c[r] = c[r2];
-                        s[r2] = ts;
-                        c[r2] = tc;
-                    }
-                }
-            } else {
-                const bool lower = (lane & j) == 0;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float ps = __shfl_xor_sync(0xffffffffu, s[r], j);
-                    const int pc = __shfl_xor_sync(0xffffffffu, c[r], j);
-                    const bool up = (((r * 32) + lane) & k) == 0;
-                    const bool take = (lower == up) ? ranks_before(ps, pc, s[r], c[r])
-                                                    : ranks_before(s[r], c[r], ps, pc);
-                    if (take) {
-                        s[r] = ps;
-                        c[r] = pc;
-                    }
-                }
-            }
-        }
-    }
-}
 
 // Sort bs/bc[0 .. want-1] in place (R * 32 >= want entries; the rest become
 // padding (-inf, INT32_MAX))
@@ -623,7 +486,8 @@ constexpr int kDenseK2Max = 16;   // second-step keys per lane of the dense sele
 template <int KPL, int R>
 __global__ void __launch_bounds__(kSelectWarps * 32, (KPL >= 64 || R >= 8) ? 4 : 8) k_rank_dense_final(
     const float *__restrict__ list_s, const int *__restrict__ list_n, int64_t nq, int cap,
-    int nprobe, int32_t *__restrict__ order, float *__restrict__ cscores) {
+    int nprobe, int32_t *__restrict__ order, float *__restrict__ cscores, const int *n_dev,
+    int64_t n_off) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     constexpr int kK2 = R <= 2 ? 4 : R == 4 ? 8 : kDenseK2Max;   // about twice nprobe / 32
     constexpr int kSort = 32 * R;
@@ -634,7 +498,7 @@ __global__ void __launch_bounds__(kSelectWarps * 32, (KPL >= 64 || R >= 8) ? 4 :
     uint32_t *ck = reinterpret_cast<uint32_t *>(bc + kSort);
     int *ci = reinterpret_cast<int *>(ck + kS2);
     const int64_t q = (int64_t)blockIdx.x * kSelectWarps + warp;
-    if (q >= nq) return;
+    if (q >= queries_of(nq, n_dev, n_off)) return;
     const float *row = list_s + q * cap;
     const int cnt = list_n[q];
     const int want = nprobe < cnt ? nprobe : cnt;
@@ -677,7 +541,8 @@ __global__ void __launch_bounds__(kSelectWarps * 32, KMAX <= 16 ? 8 : 4) k_rank_
     const float *__restrict__ list_s, const int32_t *__restrict__ list_i,
     const int *__restrict__ list_n, const float *__restrict__ list_edge, int64_t nq, int nranges,
     int64_t range_len, int cap, int nprobe, int ccap, int32_t *__restrict__ order,
-    float *__restrict__ cscores, int *__restrict__ ovf_list, int *__restrict__ ovf_n) {
+    float *__restrict__ cscores, int *__restrict__ ovf_list, int *__restrict__ ovf_n, const int *n_dev,
+    int64_t n_off) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     constexpr int kSort = 32 * R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -687,7 +552,7 @@ __global__ void __launch_bounds__(kSelectWarps * 32, KMAX <= 16 ? 8 : 4) k_rank_
     float *bs = reinterpret_cast<float *>(wbase + (size_t)ccap * 8);    // sort buffer
     int *bc = reinterpret_cast<int *>(bs + kSort);
     const int64_t q = (int64_t)blockIdx.x * kSelectWarps + warp;
-    if (q >= nq) return;
+    if (q >= queries_of(nq, n_dev, n_off)) return;
     const unsigned below = (1u << lane) - 1u;
     int n = 0;
     bool over = false;
@@ -754,6 +619,14 @@ __global__ void k_cnorm_max(const float *__restrict__ C, int64_t nlist, int d,
     if (lane == 0) atomicMax(out, __float_as_uint(best));
 }
 
+cudaError_t launch_cnorm_max(const float *C, int64_t nlist, int d, unsigned *out, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(nlist, 8), 4 * (int64_t)num_sms());
+    k_cnorm_max<<<blocks, 256, 0, st>>>(C, nlist, d, out);
+    return cudaGetLastError();
+}
+
 // One warp per query: T = a key reached by at least nprobe of its ng group
 // maxima (warp_threshold; each maximum is a different centroid's score), so
 // at least nprobe centroids score >= T in the first pass.  The second pass
@@ -772,10 +645,10 @@ template <int KPL>
 __global__ void __launch_bounds__(kSelectWarps * 32) k_rank_threshold(
     const float *__restrict__ gmax, int64_t gld, int64_t nq, int ng, int nprobe,
     const float *__restrict__ Q, int d, const unsigned *__restrict__ cmax_bits, int screen,
-    float *__restrict__ init_edge) {
+    float *__restrict__ init_edge, const int *n_dev, int64_t n_off) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t q = (int64_t)blockIdx.x * kSelectWarps + warp;
-    if (q >= nq) return;
+    if (q >= queries_of(nq, n_dev, n_off)) return;
     const float *row = gmax + q * gld;
     uint32_t key[KPL];
 #pragma unroll
@@ -984,7 +857,7 @@ static void launch_final(const RankArgs &a, const RankPlan &L, int64_t n, int32_
         const int kpl = std::max(4, pow2_at_least(ceil_div(L.cap, 32)));
 #define SIEVE_DENSE(KK, RR)                                                                      \
     k_rank_dense_final<KK, RR><<<blocks, kSelectWarps * 32, dense_smem(KK, RR), st>>>(              \
-        a.list_s, a.list_n, n, a.cap, a.nprobe, order, cscores)
+        a.list_s, a.list_n, n, a.cap, a.nprobe, order, cscores, a.n_dev, a.n_off)
 #define SIEVE_DENSE_R(KK)                   \
     switch (sort_regs(a.nprobe)) {          \
         case 2: SIEVE_DENSE(KK, 2); break;  \
@@ -1007,7 +880,7 @@ static void launch_final(const RankArgs &a, const RankPlan &L, int64_t n, int32_
 #define SIEVE_FINAL(RR, KK)                                                                      \
     k_rank_final<RR, KK><<<blocks, kSelectWarps * 32, final_smem(L.ccap, RR), st>>>(                \
         a.list_s, a.list_i, a.list_n, a.list_edge, n, a.nranges, a.range_len, a.cap, a.nprobe,    \
-        L.ccap, order, cscores, ovf, ovf_n)
+        L.ccap, order, cscores, ovf, ovf_n, a.n_dev, a.n_off)
 #define SIEVE_FINAL_R(RR)                   \
     switch (kmax) {                         \
         case 4: SIEVE_FINAL(RR, 4); break;   \
@@ -1027,12 +900,12 @@ static void launch_final(const RankArgs &a, const RankPlan &L, int64_t n, int32_
 
 static void launch_threshold(const RankPlan &L, const float *gmax, int64_t n, int nprobe,
                              const float *Q, int d, const unsigned *cmax, float *init_edge,
-                             cudaStream_t st) {
+                             const int *n_dev, int64_t n_off, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(n, kSelectWarps);
     const int kpl = std::max(1, pow2_at_least(ceil_div(L.ng, 32)));
 #define SIEVE_THR(K)                                                                             \
     k_rank_threshold<K><<<blocks, kSelectWarps * 32, 0, st>>>(gmax, L.gld, n, L.ng, nprobe, Q, d, \
-                                                              cmax, L.screen ? 1 : 0, init_edge)
+                                                              cmax, L.screen ? 1 : 0, init_edge, n_dev, n_off)
     switch (kpl) {
         case 1: SIEVE_THR(1); break;
         case 2: SIEVE_THR(2); break;
@@ -1066,7 +939,7 @@ int rank_tc_mma_launches(int64_t nq, int64_t nlist, int nprobe, int d, int64_t p
 cudaError_t enqueue_rank_tc(const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                             int nprobe, int32_t *order, float *cscores, float *scratch, int *status,
                             cudaStream_t st, const unsigned char *tc_cent, float *mma_ms,
-                            int64_t plan_nq) {
+                            int64_t plan_nq, const int *n_dev, int64_t n_off) {
     if (nq <= 0) return cudaSuccess;
     // the layout of the scratch follows the batch it was sized for; a part of
     // that batch uses the same layout, so it never needs more
@@ -1134,19 +1007,17 @@ cudaError_t enqueue_rank_tc(const float *Q, int64_t nq, const float *C, int64_t 
         if (mma_ms) cudaEventRecord(evs.back(), st);
     };
     if (L.screen) {
-        cudaError_t e = cudaMemsetAsync(cmax, 0, sizeof(unsigned), st);
+        cudaError_t e = launch_cnorm_max(C, nlist, d, cmax, st);
         if (e != cudaSuccess) return e;
-        const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(nlist, 8), 4 * (int64_t)num_sms());
-        k_cnorm_max<<<blocks, 256, 0, st>>>(C, nlist, d, cmax);
     }
     for (int64_t q0 = 0; q0 < nq; q0 += L.chunk) {
         const int64_t n = nq - q0 < L.chunk ? nq - q0 : L.chunk;
         RankArgs a{Q + q0 * d, n, C, nlist, d, status, tc_cent, nprobe, L.nranges,
                    L.range_len, L.cap, list_s, list_i, list_n, list_edge, nullptr, gmax, L.gld,
-                   L.group};
+                   L.group, n_dev, n_off + q0};
         if (L.group) {   // the first pass: group maxima, then each query's starting threshold
             contract(kRankGroupMax, a, n, L.screen);
-            launch_threshold(L, gmax, n, nprobe, Q + q0 * d, d, cmax, init_edge, st);
+            launch_threshold(L, gmax, n, nprobe, Q + q0 * d, d, cmax, init_edge, n_dev, n_off + q0, st);
             a.init_edge = init_edge;
         }
         contract(L.group ? kRankStreamInit : L.mode, a, n, false);

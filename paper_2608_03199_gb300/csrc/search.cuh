@@ -27,6 +27,9 @@ struct SearchArgs {
     int k, nprobe, W, lookahead;
     int serial;                // 1: every (query, rank) item is its own tile (serial traversal)
     int wait_limit;            // polls of the tensor-core scan epilogue's accumulator wait (0: default)
+    // prefix ranking (rank_prefix.cu), nullable: the ranks of each query's
+    // order that are in place, and the queries whose stop line passes them
+    int *limit, *ext;
     int64_t cap;               // items per round
     int max_rounds;
     // per-query state: stop line S (Sec. 4.3) and enqueue cursor E (first
@@ -84,8 +87,8 @@ cudaError_t prepare_scan_kernel(size_t smem);
 cudaError_t launch_init(const SearchArgs &a, cudaStream_t st);
 cudaError_t launch_finalize(const SearchArgs &a, cudaStream_t st);
 cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
-                         cudaGraphConditionalHandle cond, int use_cond, cudaStream_t st,
-                         cudaEvent_t *ev = nullptr);
+                         cudaGraphConditionalHandle cond, cudaGraphConditionalHandle ext_cond,
+                         int use_cond, cudaStream_t st, cudaEvent_t *ev = nullptr);
 constexpr int kRoundKernels = 7;   // issue, bucket, scatter, scan_tc, scan, merge, round_end
 
 // tensor-core scan (scan_tc.cu)
@@ -124,11 +127,15 @@ cudaError_t prepare_rank_tc(int nprobe, int d);
 // mma_ms (nullable): the contraction launches are bracketed by events, the
 // call synchronizes st and adds their summed time (ms) to *mma_ms.
 // plan_nq: the query count scratch was sized for (rank_tc_scratch_bytes), when
-// these nq queries are a part of that batch; 0 = nq
+// these nq queries are a part of that batch; 0 = nq.  n_dev (nullable, device):
+// only the first *n_dev - n_off of the nq queries exist
 cudaError_t enqueue_rank_tc(const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                             int nprobe, int32_t *order, float *cscores, float *scratch, int *status,
                             cudaStream_t st, const unsigned char *tc_cent = nullptr,
-                            float *mma_ms = nullptr, int64_t plan_nq = 0);
+                            float *mma_ms = nullptr, int64_t plan_nq = 0,
+                            const int *n_dev = nullptr, int64_t n_off = 0);
+// the largest Euclidean norm of nlist rows (one float, as its bits)
+cudaError_t launch_cnorm_max(const float *C, int64_t nlist, int d, unsigned *out, cudaStream_t st);
 int rank_tc_mma_launches(int64_t nq, int64_t nlist, int nprobe, int d, int64_t plan_nq,
                          bool bulk);   // contraction launches
 int rank_screen_stages(int d);                   // 0 when the screening first pass does not apply
@@ -138,6 +145,22 @@ cudaError_t enqueue_screen_scores(const float *Q, int64_t nq, int64_t nlist, int
                                   const unsigned char *tc_cent, float *out, int64_t ld,
                                   int *status, cudaStream_t st);
 int rank_bulk_stages(int d);                     // 0 when the bulk ranking does not apply
+
+// the first ranks alone, and the full ranking of the queries that need more
+// (rank_prefix.cu): entries kept per query list, 0 when it does not apply; the
+// scratch (the limits and the extension list first, for the whole search)
+int rank_prefix_len(int64_t nlist, int nprobe, int W, int d);
+size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int d);   // for any W
+int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext);
+cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d);
+int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma);
+cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
+                                int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
+                                void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
+                                float *mma_ms = nullptr);
+cudaError_t enqueue_rank_ext(const float *Q, int64_t nq, const float *C, int64_t nlist, int d, int nprobe,
+                             int W, int32_t *order, float *cscores, void *scratch, const int *ext_n,
+                             int *status, const unsigned char *tc_cent, cudaStream_t st);
 
 // in-call window calibration (calibrate.cu)
 cudaError_t calib_gather(const float *Q, const int64_t *qids, int d, const int64_t *idx, int64_t n,

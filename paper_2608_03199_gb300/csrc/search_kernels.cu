@@ -116,6 +116,13 @@ __global__ void __launch_bounds__(kIssueThreads) k_issue(SearchArgs a) {
         if (q < a.nq) {
             int s = a.S[q];
             e = a.E[q];
+            if (a.limit) {   // ranks past the query's prefix wait for its extension
+                const int lim = a.limit[q];
+                if (s > lim) {
+                    a.ext[atomicAdd(&ctl->n_ext, 1)] = (int)q;
+                    s = lim;
+                }
+            }
             if (e <= s) want = a.lookahead ? s - e + 1 : 1;
         }
         int off = block_exclusive_scan(want, warp_tot, &tot_items);
@@ -556,18 +563,21 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(SearchArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-__global__ void k_round_end(SearchArgs a, cudaGraphConditionalHandle cond, int use_cond) {
+__global__ void k_round_end(SearchArgs a, cudaGraphConditionalHandle cond,
+                            cudaGraphConditionalHandle ext_cond, int use_cond) {
     Ctl *c = a.ctl;
     const int items = c->n_items < a.cap ? c->n_items : (int)a.cap;
     c->tot_items += (unsigned long long)items;
     c->tot_tiles += (unsigned long long)(c->n_tiles + c->n_tc_tiles);
     c->round += 1;
-    int more = (c->n_continue > 0 || c->n_deferred > 0) && c->status == 0 ? 1 : 0;
+    int more = (c->n_continue > 0 || c->n_deferred > 0 || c->n_ext > 0) && c->status == 0 ? 1 : 0;
     if (more && c->round >= a.max_rounds) {
         c->status = SIEVE_ELIMIT;
         more = 0;
     }
     c->more = more;
+    c->ext_n = more ? c->n_ext : 0;
+    c->n_ext = 0;
     c->n_items = 0;
     c->n_active = 0;
     c->n_tiles = 0;
@@ -576,7 +586,10 @@ __global__ void k_round_end(SearchArgs a, cudaGraphConditionalHandle cond, int u
     c->tc_tile_next = 0;
     c->n_deferred = 0;
     c->n_continue = 0;
-    if (use_cond) cudaGraphSetConditional(cond, more ? 1u : 0u);
+    if (use_cond) {
+        cudaGraphSetConditional(cond, more ? 1u : 0u);
+        if (a.limit) cudaGraphSetConditional(ext_cond, c->ext_n > 0 ? 1u : 0u);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -615,8 +628,8 @@ cudaError_t launch_finalize(const SearchArgs &a, cudaStream_t st) {
 }
 
 cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
-                         cudaGraphConditionalHandle cond, int use_cond, cudaStream_t st,
-                         cudaEvent_t *ev) {
+                         cudaGraphConditionalHandle cond, cudaGraphConditionalHandle ext_cond,
+                         int use_cond, cudaStream_t st, cudaEvent_t *ev) {
     // ev (optional): 2 * kRoundKernels events, recorded before/after each kernel
     const int sms = num_sms();
     int slot = 0;
@@ -657,7 +670,7 @@ cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
     k_merge<<<merge_blocks, kMergeThreads, 0, st>>>(a);
     end();
     begin();
-    k_round_end<<<1, 1, 0, st>>>(a, cond, use_cond);
+    k_round_end<<<1, 1, 0, st>>>(a, cond, ext_cond, use_cond);
     end();
     return cudaGetLastError();
 }

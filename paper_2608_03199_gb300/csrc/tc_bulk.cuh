@@ -195,6 +195,18 @@ struct RingPos {
     }
 };
 
+// Modes that pass over a sample of their chunks first (Tile::ns chunks, every
+// Tile::sstep-th one, handed to Epi::sample; then Epi::seed, then all chunks)
+template <class Mode, class = void>
+struct sampled { static constexpr bool value = false; };
+template <class Mode>
+struct sampled<Mode, decltype((void)Mode::kSampled)> { static constexpr bool value = Mode::kSampled; };
+template <class Mode>
+__device__ __forceinline__ int sample_chunks(const typename Mode::Tile &T) {
+    if constexpr (sampled<Mode>::value) return T.ns;
+    return 0;
+}
+
 // one 32-column group of an accumulator row to the mode's epilogue
 template <class Epi, class Args, class Tile>
 __device__ __forceinline__ void hand(Epi &epi, const Args &a, const Tile &T, int64_t col0,
@@ -204,6 +216,14 @@ __device__ __forceinline__ void hand(Epi &epi, const Args &a, const Tile &T, int
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
     const int64_t left = T.nb - col0;
     epi.chunk(a, T, col0, v, left < 32 ? (int)left : 32);
+}
+
+template <class Epi>
+__device__ __forceinline__ void hand_sample(Epi &epi, const uint32_t (&r)[32]) {
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    epi.sample(v);
 }
 
 // What bounds the issuing warp: each chunk's waits, commits and MMAs are one
@@ -471,7 +491,10 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 const int nch = uniform((int)ceil_div(T.nb, kNB));
                 const int nblk = uniform((int)ceil_div(T.nb, kN));   // layout blocks of the tile's B
                 const unsigned char *src0 = uniform_ptr(Mode::b_block(a, T));
-                for (int ch = 0; ok && ch < nch; ++ch) {
+                const int ns = uniform(sample_chunks<Mode>(T));
+                for (int c = 0; ok && c < nch + ns; ++c) {
+                    int ch = c;   // the chunk of the tile's B that this pass takes
+                    if constexpr (sampled<Mode>::value) ch = c < ns ? c * T.sstep : c - ns;
                     if constexpr (kNB != kN) {
                         // a 192-row chunk: rows r0 .. r0 + 191 of the tile's B, from
                         // block r0 / 128 (from its row r0 % 128) and the next block
@@ -546,8 +569,9 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 if (lane == 0) tc::mbar_arrive(&ring_empty[slot]);
                 if (t < 0) break;
                 const typename Mode::Tile T = Mode::tile(a, t);
-                const int nch = uniform((int)ceil_div(T.nb, kNB));
+                int nch = uniform((int)ceil_div(T.nb, kNB));
                 if (nch == 0) continue;
+                nch += uniform(sample_chunks<Mode>(T));
                 for (int ch = 0; ok && ch < nch; ++ch) {
                     if constexpr (kSub == 1) {   // the chunk's accumulator
                         if (!(ok = warp_wait(&dempty_bar[dp.slot], dp.phase ^ 1u))) break;
@@ -612,7 +636,13 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
             const typename Mode::Tile T = Mode::tile(a, t);
             const int nch = (int)ceil_div(T.nb, kNB);
             epi.begin(a, T, slot, epi_smem);
-            for (int ch = 0; ch < nch; ++ch, dp.step(kSub > 1 ? 1u : nacc)) {
+            const int ns = sample_chunks<Mode>(T);
+            for (int c = 0; c < nch + ns; ++c, dp.step(kSub > 1 ? 1u : nacc)) {
+                int ch = c;
+                if constexpr (sampled<Mode>::value) {
+                    if (c == ns && ns > 0) epi.seed();
+                    ch = c < ns ? c * T.sstep : c - ns;
+                }
                 const uint32_t buf = kSub > 1 ? (uint32_t)h : dp.slot, dph = dp.phase;
                 epi.prefetch(a, T, ch);   // per-chunk loads, in flight during the wait
                 ok = __all_sync(0xffffffffu, wait_n(&dfull_bar[buf], dph, epi_wait));
@@ -622,7 +652,10 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 // one copy of the mode's code per load, in a loop that is not
                 // unrolled: each role runs straight code of its own, and with
                 // the loop unrolled the epilogue waits for instructions (join
-                // of 100K queries with 1M x 256, W = 8: scan 1.70 -> 1.23 ms).  The accumulator is released as soon as the
+                // of 100K queries with 1M x 256, W = 8: scan 1.70 -> 1.23 ms;
+                // two sub-tiles, a pair of loads in flight per step: screen
+                // pass + lists over 65,536 x 96 27.6 -> 21.7 ms, 23.8 with
+                // single loads).  The accumulator is released as soon as the
                 // last load has landed, before its columns go to the mode.
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kNB;
                 const int64_t col0 = (int64_t)ch * kNB;
@@ -637,6 +670,13 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                     if (g == kNB / 32 - kLd) {
                         tc::fence_before_sync();
                         tc::mbar_arrive(&dempty_bar[buf]);
+                    }
+                    if constexpr (sampled<Mode>::value) {
+                        if (c < ns) {
+#pragma unroll
+                            for (int u = 0; u < kLd; ++u) hand_sample(epi, r[u]);
+                            continue;
+                        }
                     }
 #pragma unroll
                     for (int u = 0; u < kLd; ++u) hand(epi, a, T, col0 + (g + u) * 32, r[u]);

@@ -1,0 +1,90 @@
+"""The search that ranks a prefix of each query's centroid order first and
+extends it where the stop line passes it, against the same search on a given
+full order: probes, counts and ids must be the same, scores within 1e-5.
+
+Low thresholds make most probes hit, so stop lines run far past the prefix
+(16 or 32 entries less the margin); identical centroids leave no verified
+prefix at all."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    return torch.device("cuda:0")
+
+
+def _index(sieve, dev, n, d, nlist, seed, grouped=False, equal=0):
+    g = torch.Generator().manual_seed(seed)
+    unit = lambda x: x / x.norm(dim=1, keepdim=True)
+    C = unit(torch.randn(nlist, d, generator=g))
+    if grouped:   # neighbours with adjacent ids
+        base = unit(torch.randn(-(-nlist // 32), d, generator=g)).repeat_interleave(32, 0)[:nlist]
+        C = unit(base + 0.3 * C)
+    if equal:     # blocks of identical centroids: exact ties
+        C = C[torch.arange(nlist) // equal * equal].contiguous()
+    a = torch.randint(0, nlist, (n,), generator=g)
+    X = unit(C[a] + 0.9 * torch.randn(n, d, generator=g) / d ** 0.5)
+    return sieve.build_layout(X.to(dev), a.int().to(dev), nlist, C.to(dev)), X
+
+
+CASES = [  # n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal
+    (6_000, 64, 64, 300, 45, 4, 0.30, True, False, 0),
+    (6_000, 64, 65, 257, 64, 8, 0.55, False, False, 0),
+    (9_000, 96, 700, 1_000, 90, 8, 0.35, True, True, 0),
+    (9_000, 128, 129, 513, 33, 10, 0.40, True, False, 0),
+    (9_000, 256, 300, 400, 100, 24, 0.50, True, False, 0),
+    (12_000, 36, 2_500, 300, 77, 2, 0.60, True, False, 0),
+    (12_000, 200, 2_049, 130, 128, 8, 0.45, True, True, 0),
+    (5_000, 32, 192, 200, 40, 8, 0.50, True, False, 8),
+    (5_000, 96, 128, 70, 50, 16, 0.50, True, False, 128),
+    (40_000, 96, 5_000, 600, 64, 8, 0.45, True, True, 0),
+    (40_000, 96, 1_024, 40_000, 64, 8, 0.60, True, True, 0),   # several tiles per block
+    (20_000, 256, 1_024, 20_000, 40, 8, 0.70, True, False, 0),
+    (3_000, 96, 64, 1, 64, 8, 0.20, True, False, 0),
+]
+
+
+@pytest.mark.parametrize("n,d,nlist,nq,nprobe,W,tau,lookahead,grouped,equal", CASES)
+def test_prefix_equals_full_order(dev, n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal):
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, n, d, nlist, seed=n + d + nlist, grouped=grouped, equal=equal)
+    # up to 2,048 centroids a batch takes the prefix from 4,096 queries up: the
+    # small batches repeat theirs
+    rows = torch.randperm(n, generator=torch.Generator().manual_seed(3))[:nq]
+    if nlist <= 2_048 and nq > 1:
+        rows = rows.repeat(-(-4_100 // nq))[:max(nq, 4_100 + nq % 7)]
+    nq = rows.numel()
+    Q, qids = X[rows].to(dev), rows.to(dev)
+    order = sieve.rank_partitions(ix, Q, nprobe)
+    kw = dict(lookahead=lookahead, query_ids=qids, check=True)
+    want = [x.cpu().numpy() for x in sieve.search(ix, Q, tau, 10, nprobe, W, order=order, **kw)]
+    for loop in (0, 1):
+        got = [x.cpu().numpy() for x in sieve.search(ix, Q, tau, 10, nprobe, W, loop=loop, **kw)]
+        # a query may differ only through two centroid scores, or two results,
+        # closer than the rounding of either: at most one here in 500
+        bad = (got[3] != want[3]) | (got[2] != want[2]) | (got[0] != want[0]).any(1)
+        assert bad.sum() <= nq // 500, (int(bad.sum()), np.flatnonzero(bad)[:5])
+        ok = ~bad
+        fin = np.isfinite(want[1][ok])
+        assert np.abs(got[1][ok][fin] - want[1][ok][fin]).max(initial=0) <= 1e-5
+        # no partition visited twice: no result id repeats
+        for r in got[0][got[2] > 1][:2000]:
+            r = r[r >= 0]
+            assert len(set(r.tolist())) == len(r)
+
+
+def test_prefix_host_path(dev):
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 30_000, 96, 300, seed=9)
+    Q = X[:25_000].contiguous()          # two upload chunks
+    ids = torch.arange(25_000)
+    a = sieve.search(ix, Q.to(dev), 0.5, 10, 100, 8, query_ids=ids.to(dev), check=True)
+    b = sieve.search_host(ix, Q.pin_memory(), 0.5, 10, 100, 8, query_ids_host=ids.pin_memory())
+    for x, y in zip(a, b):
+        assert torch.equal(x.cpu(), y)
