@@ -79,6 +79,7 @@ constexpr float kScreenMinTau = 0.85f; // ... and this threshold up (below it ne
 // 1,024 x 256: 60 us less as a prefix)
 constexpr int64_t kPrefixAlwaysNlist = 2048;
 constexpr int64_t kPrefixMinQueries = 4096;
+constexpr int64_t kPrefixMinWide = 256;
 constexpr int64_t kAutoCapMax = int64_t(1) << 24;
 constexpr int64_t kCapMax = int64_t(1) << 30;
 
@@ -375,10 +376,12 @@ struct RqInputs {
     const float *cscores;
 };
 
-// whether a search ranks a prefix of each order first: the bulk pipeline's
-// centroid layout, and a window that visits few of the nprobe ranks
+// whether a search ranks a prefix of each order first: the centroids laid out
+// for the bulk pipeline, and a window that visits few of the nprobe ranks
 bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p) {
-    return ix->tc_centroids && (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
+    // past d = 256 the prefix lays the centroids out itself, which a few queries do not repay
+    if (ix->d <= 256 ? !ix->tc_centroids : nq < kPrefixMinWide) return false;
+    return (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
            rank_prefix_len(ix->nlist, p->nprobe, p->W, ix->d) > 0;
 }
 

@@ -33,7 +33,9 @@
 // in some lane) and the single accumulator per sub-tile they hold meanwhile.
 // Against the full ranking (two contraction passes, ~310 candidates a query
 // sorted): 1M queries x 65,536 x 96, nprobe 256, 52.1 -> 25.0 ms; 1M x 8,192 x
-// 256, nprobe 128, 17.6 -> 7.7 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.35 ms.
+// 256, nprobe 128, 17.6 -> 7.7 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.35 ms;
+// 200K x 16,384 x 512, nprobe 128 (against the converter pipeline's three
+// products), 16.2 -> 5.0 ms.
 #include <cmath>
 #include <vector>
 
@@ -57,12 +59,16 @@ struct PrefixArgs {
 
 __device__ int g_prefix_status_sink;
 
-template <int kL, int kNBT>
+// kSubT = 2: centroids in the tensor-core layout, d <= 256.  kSubT = 1: d <= 512,
+// A's hi half alone fills 256 columns, and the centroids' hi halves in a layout
+// of their own (k_prefix_fill: 16 KB per K-block).
+template <int kL, int kNBT, int kSubT>
 struct PrefixMode {
     using Args = PrefixArgs;
     static constexpr int kProducts = 1;
     static constexpr int kNB = kNBT;
-    static constexpr int kSub = 2;
+    static constexpr int kSub = kSubT;
+    static constexpr bool kBHasLo = kSubT == 2;
     static constexpr int kRows = kSub * tcp::kM;
     static constexpr bool kSampled = true;
     struct Tile {
@@ -91,7 +97,7 @@ struct PrefixMode {
         return i < T.ni ? a.Q + (T.q0 + i) * a.d : nullptr;
     }
     __device__ static const unsigned char *b_block(const Args &a, const Tile &T) {
-        return a.tc_cent + (T.c0 / kTcRows) * (int64_t)((a.d + 63) / 64) * kTcBlockBytes;
+        return a.tc_cent + (T.c0 / kTcRows) * (int64_t)((a.d + 63) / 64) * (kBHasLo ? tcb::kKbBytes : tcb::kKbBytesHi);
     }
     struct Epi {
         float *ks;      // entry j of this query's list at [j * kRows]
@@ -209,10 +215,33 @@ struct PrefixMode {
     };
 };
 
-template <int kL, int kNBT>
+template <int kL, int kNBT, int kSubT>
 __global__ void __launch_bounds__(tcb::kThreads, 1) k_prefix_scan(PrefixArgs a, int stages) {
     extern __shared__ unsigned char smem_raw[];
-    tcb::run_bulk<PrefixMode<kL, kNBT>>(a, smem_raw, stages);
+    tcb::run_bulk<PrefixMode<kL, kNBT, kSubT>>(a, smem_raw, stages);
+}
+
+// The centroids' hi halves in the tensor-core layout's order, for rows wider
+// than an index keeps a layout of by default: a thread per (block, K-block,
+// row, 16-byte chunk), rows past nlist and columns past d zero.  Bound by
+// memory (6d bytes a centroid, once per call).
+__global__ void k_prefix_fill(const float *__restrict__ C, int64_t nlist, int d, int nkb,
+                              unsigned char *__restrict__ out) {
+    const int64_t total = ceil_div(nlist, kTcRows) * nkb * kTcRows * 8;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(u & 7), r = (int)((u >> 3) & (kTcRows - 1));
+        const int64_t bk = u >> 10, row = bk / nkb * kTcRows + r;
+        const int col = (int)(bk % nkb) * 64 + c * 8;
+        const float *src = row < nlist ? C + row * d : nullptr;
+        const float4 x0 = tcp::load_f4(src, col, d), x1 = tcp::load_f4(src, col + 4, d);
+        uint4 h, l;
+        tcp::split2(x0.x, x0.y, h.x, l.x);
+        tcp::split2(x0.z, x0.w, h.y, l.y);
+        tcp::split2(x1.x, x1.y, h.z, l.z);
+        tcp::split2(x1.z, x1.w, h.w, l.w);
+        *reinterpret_cast<uint4 *>(out + bk * tcb::kKbBytesHi + (int64_t)r * 128 + ((c ^ (r & 7)) << 4)) = h;
+    }
 }
 
 // One warp per query.  NT: float4 of a row per lane of a group of eight (d <=
@@ -383,16 +412,23 @@ __global__ void k_ext_merge(const int *__restrict__ ext, const int *__restrict__
 
 // ---------------------------------------------------------------------------
 static bool prefix_wide(int d) { return ceil_div(d, 64) <= 2; }   // 192-centroid chunks, as the screen
+static int prefix_sub(int d) { return ceil_div(d, 64) <= 4 ? 2 : 1; }   // sub-tiles of 128 queries per tile
 static uint32_t prefix_stage_bytes(int d) {
     return prefix_wide(d) ? tcb::kStageBytesHi / tcb::kN * 192 : tcb::kStageBytesHi;
 }
-static size_t prefix_epi_bytes(int L) { return (size_t)2 * tcp::kM * L * 8; }
+static size_t prefix_epi_bytes(int d, int L) { return (size_t)prefix_sub(d) * tcp::kM * L * 8; }
 
 static int prefix_stages(int d, int L) {
     const int nkb = (int)ceil_div(d, 64);
-    return tcb::sub_fits(nkb, 1, 2)
-               ? tcb::stages_for(nkb, prefix_epi_bytes(L), 232448 - 128, prefix_stage_bytes(d))
+    return tcb::sub_fits(nkb, 1, prefix_sub(d))
+               ? tcb::stages_for(nkb, prefix_epi_bytes(d, L), 232448 - 128, prefix_stage_bytes(d), tcb::kStagesMax,
+                                 tcb::kMaxKb)
                : 0;
+}
+
+// bytes of the centroids' hi halves kept in the scratch (k_prefix_fill)
+static int64_t fill_bytes(int64_t nlist, int d) {
+    return prefix_sub(d) == 2 ? 0 : ceil_div(nlist, kTcRows) * ceil_div(d, 64) * tcb::kKbBytesHi;
 }
 
 // Entries kept per list: min(W, nprobe) ranks are visited for certain, a hit at
@@ -418,7 +454,7 @@ struct PrefixPlan {
 // Ranges: enough tiles to fill the SMs in whole waves.  A tile costs its chunks
 // plus about six chunks' time for writing A and filling the lists.
 static PrefixPlan prefix_plan(int64_t nq, int64_t nlist, int d, int L) {
-    const int64_t tiles = std::max<int64_t>(1, ceil_div(nq, 2 * tcp::kM)), sms = num_sms();
+    const int64_t tiles = std::max<int64_t>(1, ceil_div(nq, prefix_sub(d) * tcp::kM)), sms = num_sms();
     const int64_t nb = prefix_wide(d) ? 192 : 128;
     const int64_t most = std::min<int64_t>(ceil_div(nlist, kTcRows), std::min<int64_t>(1024 / L, 32));
     PrefixPlan best{1, round_up(nlist, (int64_t)kTcRows)};
@@ -440,6 +476,7 @@ static PrefixPlan prefix_plan(int64_t nq, int64_t nlist, int d, int L) {
 // queries (the prefix) or the extension's buffers, which are never live at once.
 struct PrefixScratch {
     int64_t limit, ext, rest;      // byte offsets
+    int64_t fill, lists;           // the prefix's part: the centroids' hi halves, the lists
     int64_t chunk;                 // queries per prefix pass
     int64_t ext_chunk;             // queries per extension pass
     int64_t ext_q, ext_order, ext_s;   // byte offsets of the extension's buffers (after its ranking scratch)
@@ -474,8 +511,10 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
     S.total = std::max(end, plain);
     const PrefixPlan P = prefix_plan(nq, nlist, d, L);
     const int64_t per = (int64_t)P.nranges * (L * 8 + 4);
-    S.total = std::max(S.total, S.rest + std::min<int64_t>(nq, 2 * tcp::kM) * per + 512);
-    S.chunk = std::min(nq, std::max<int64_t>(2 * tcp::kM, (S.total - S.rest - 512) / per / (2 * tcp::kM) * (2 * tcp::kM)));
+    S.fill = S.rest + 256;
+    S.lists = S.fill + fill_bytes(nlist, d);
+    S.total = std::max(S.total, S.lists + std::min<int64_t>(nq, 2 * tcp::kM) * per + 256);
+    S.chunk = std::min(nq, std::max<int64_t>(2 * tcp::kM, (S.total - S.lists - 256) / per / (2 * tcp::kM) * (2 * tcp::kM)));
     return S;
 }
 
@@ -495,29 +534,33 @@ int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int
     return reinterpret_cast<int *>(w + S.limit);
 }
 
-template <int kL, int kNBT>
-static cudaError_t set_scan_attr(int d) {
-    return cudaFuncSetAttribute(
-        k_prefix_scan<kL, kNBT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)tcb::smem_bytes(prefix_stages(d, kL), prefix_epi_bytes(kL), prefix_stage_bytes(d)));
+static size_t scan_smem(int d, int L) {
+    return tcb::smem_bytes(prefix_stages(d, L), prefix_epi_bytes(d, L), prefix_stage_bytes(d));
+}
+
+// the scan kernel of this d and list length
+using PrefixScan = void (*)(PrefixArgs, int);
+static PrefixScan scan_kernel(int d, int L) {
+    if (prefix_sub(d) == 1) return L == 16 ? k_prefix_scan<16, 128, 1> : k_prefix_scan<32, 128, 1>;
+    if (prefix_wide(d)) return L == 16 ? k_prefix_scan<16, 192, 2> : k_prefix_scan<32, 192, 2>;
+    return L == 16 ? k_prefix_scan<16, 128, 2> : k_prefix_scan<32, 128, 2>;
 }
 
 cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d) {
     const int L = rank_prefix_len(nlist, nprobe, W, d);
-    if (prefix_wide(d)) return L == 16 ? set_scan_attr<16, 192>(d) : set_scan_attr<32, 192>(d);
-    return L == 16 ? set_scan_attr<16, 128>(d) : set_scan_attr<32, 128>(d);
+    return cudaFuncSetAttribute(scan_kernel(d, L), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)scan_smem(d, L));
 }
 
 template <int kL, int KPL>
 static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, const unsigned *cmax,
                                 int32_t *order, float *cscores, int *limit, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(a.nq, kFinalWarps);
-    if (a.d <= 128)
-        k_prefix_final<kL, KPL, 4><<<blocks, kFinalWarps * 32, 0, st>>>(
-            a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe, cmax, order, cscores, limit);
-    else
-        k_prefix_final<kL, KPL, 8><<<blocks, kFinalWarps * 32, 0, st>>>(
-            a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe, cmax, order, cscores, limit);
+    auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 4>
+             : a.d <= 256 ? k_prefix_final<kL, KPL, 8>
+                          : k_prefix_final<kL, KPL, 16>;
+    f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe,
+                                           cmax, order, cscores, limit);
 }
 
 // kernel launches of one prefix ranking of nq queries (and its contraction
@@ -527,7 +570,7 @@ int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe,
     const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
     const int chunks = (int)ceil_div(nq, S.chunk);
     *mma = chunks;
-    return 2 * chunks + 1;
+    return 2 * chunks + 1 + (prefix_sub(d) == 1 ? 1 : 0);
 }
 
 // The prefix of nq queries q0 .. q0 + nq - 1 of a batch of plan_nq (whose
@@ -543,12 +586,13 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     unsigned char *w = static_cast<unsigned char *>(scratch);
     int *limit = reinterpret_cast<int *>(w + S.limit);
     unsigned *cmax = reinterpret_cast<unsigned *>(w + S.rest);
-    float *list_s = reinterpret_cast<float *>(w + S.rest + 256);
+    float *list_s = reinterpret_cast<float *>(w + S.lists);
     const int64_t slots = S.chunk * P.nranges * L;
     int32_t *list_i = reinterpret_cast<int32_t *>(list_s + slots);
     float *list_t = reinterpret_cast<float *>(list_i + slots);
     const int stages = prefix_stages(d, L);
-    const size_t smem = tcb::smem_bytes(stages, prefix_epi_bytes(L), prefix_stage_bytes(d));
+    const size_t smem = scan_smem(d, L);
+    const PrefixScan scan = scan_kernel(d, L);
     struct Events {
         std::vector<cudaEvent_t> v;
         ~Events() {
@@ -557,23 +601,23 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     } ev;
     cudaError_t e = launch_cnorm_max(C, nlist, d, cmax, st);
     if (e != cudaSuccess) return e;
+    if (prefix_sub(d) == 1) {
+        const int64_t pieces = ceil_div(nlist, kTcRows) * ceil_div(d, 64) * kTcRows * 8;
+        k_prefix_fill<<<(unsigned)std::min<int64_t>(ceil_div(pieces, 256), 16 * num_sms()), 256, 0, st>>>(
+            C, nlist, d, (int)ceil_div(d, 64), w + S.fill);
+        tc_cent = w + S.fill;
+    }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);
         const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, tc_cent, P.nranges, P.range_len, list_s, list_i, list_t};
-        const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 2 * tcp::kM) * P.nranges, num_sms());
+        const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, prefix_sub(d) * tcp::kM) * P.nranges, num_sms());
         if (mma_ms) {
             ev.v.resize(ev.v.size() + 2);
             cudaEventCreate(&ev.v[ev.v.size() - 2]);
             cudaEventCreate(&ev.v.back());
             cudaEventRecord(ev.v[ev.v.size() - 2], st);
         }
-        if (prefix_wide(d)) {
-            if (L == 16) k_prefix_scan<16, 192><<<grid, tcb::kThreads, smem, st>>>(a, stages);
-            else k_prefix_scan<32, 192><<<grid, tcb::kThreads, smem, st>>>(a, stages);
-        } else {
-            if (L == 16) k_prefix_scan<16, 128><<<grid, tcb::kThreads, smem, st>>>(a, stages);
-            else k_prefix_scan<32, 128><<<grid, tcb::kThreads, smem, st>>>(a, stages);
-        }
+        scan<<<grid, tcb::kThreads, smem, st>>>(a, stages);
         if (mma_ms) cudaEventRecord(ev.v.back(), st);
         int32_t *o = order + (q0 + b) * nprobe;
         float *cs = cscores ? cscores + (q0 + b) * nprobe : nullptr;

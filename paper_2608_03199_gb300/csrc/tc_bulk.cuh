@@ -68,7 +68,8 @@ constexpr int kAWriterWarps = 8;
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kThreads = 14 * 32;
-constexpr int kMaxKb = 4;                     // A in tensor memory: d <= 256
+constexpr int kMaxKb = 8;                     // A in tensor memory: d <= 256, or d <= 512 when only
+                                              // one sub-tile's hi half is kept
 constexpr int kMaxStages = 8;                 // barrier slots for B stages
 constexpr int kStagesMax = 5;                 // stages beyond five did not time faster
 constexpr uint32_t kKbBytes = 32768;          // one K-block of 128 rows: hi 16 KB + lo 16 KB
@@ -93,8 +94,8 @@ __host__ __device__ inline size_t smem_bytes(int stages, size_t epi_bytes,
 
 // B stages that fit beside the epilogue (0 when the pipeline does not apply)
 inline int stages_for(int nkb, size_t epi_bytes, size_t smem_limit, uint32_t stage_bytes = kStageBytes,
-                      int max_stages = kStagesMax) {
-    if (nkb > kMaxKb) return 0;
+                      int max_stages = kStagesMax, int max_kb = 4) {
+    if (nkb > max_kb) return 0;
     const size_t base = smem_bytes(0, epi_bytes, stage_bytes);
     if (smem_limit < base) return 0;
     int s = (int)((smem_limit - base) / stage_bytes);
@@ -143,11 +144,11 @@ __host__ __device__ constexpr uint32_t a_cols(int nkb, int products) {
 }
 
 // 128-column accumulators beside A: one sub-tile takes three when its A
-// takes at most 128 columns, else two; two sub-tiles take two, accumulator j
+// takes at most 128 columns, else two (A up to 256 columns); two sub-tiles take two, accumulator j
 // always sub-tile j's, so that each accumulator's barriers have one reader
 // group and phases cannot be skipped
 __host__ __device__ constexpr uint32_t acc_slots(int nkb, int products, int sub) {
-    return sub == 1 ? ((products == 1 || nkb <= 2) ? 3u : 2u) : 2u;
+    return sub == 1 && a_cols(nkb, products) <= 128u ? 3u : 2u;
 }
 
 // whether a pipeline of sub sub-tiles fits tensor memory at this d

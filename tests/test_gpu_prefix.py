@@ -46,6 +46,9 @@ CASES = [  # n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal
     (40_000, 96, 5_000, 600, 64, 8, 0.45, True, True, 0),
     (40_000, 96, 1_024, 40_000, 64, 8, 0.60, True, True, 0),   # several tiles per block
     (20_000, 256, 1_024, 20_000, 40, 8, 0.70, True, False, 0),
+    (20_000, 512, 3_000, 1_000, 90, 8, 0.45, True, False, 0),   # past the layout's width
+    (12_000, 260, 2_100, 300, 64, 16, 0.45, True, True, 0),
+    (12_000, 448, 300, 129, 64, 8, 0.50, False, False, 0),
     (3_000, 96, 64, 1, 64, 8, 0.20, True, False, 0),
 ]
 
