@@ -245,11 +245,12 @@ __global__ void k_prefix_fill(const float *__restrict__ C, int64_t nlist, int d,
 }
 
 // One warp per query.  NT: float4 of a row per lane of a group of eight (d <=
-// 32 NT); KPL: list entries per lane (nranges * kL <= 32 KPL).
+// 32 NT); KPL: list entries per lane (nranges * kL <= 32 KPL).  Ids are checked
+// against nlist: the lists of a pass that gave up are not read as rows.
 constexpr int kFinalWarps = 8;
 template <int kL, int KPL, int NT>
 __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
-    const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int d,
+    const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int64_t nlist, int d,
     const float *__restrict__ list_s, const int32_t *__restrict__ list_i,
     const float *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits, int32_t *__restrict__ order, float *__restrict__ cscores,
     int *__restrict__ limit) {
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
 #pragma unroll
     for (int j = 0; j < KPL; ++j) {
         const int c = j * 32 + lane;
-        key[j] = (c < M && li[c] >= 0) ? order_key(ls[c]) : 0u;
+        key[j] = (c < M && (uint32_t)li[c] < (uint64_t)nlist) ? order_key(ls[c]) : 0u;
     }
     for (int r = lane; r < nranges; r += 32) {
         const float t = list_t[q * nranges + r];
@@ -346,8 +347,9 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const float fp32 = (0x1p-20f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
     const float scr = (0x1p-10f + 0x1p-12f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
     const float margin = (scr + fp32) * (1.f + 0x1p-16f);
-    // scores past fp16's range (|256 x| above 65,504) are not screened soundly
-    const bool sound = fits && qn < 200.f && cn < 200.f;
+    // scores past fp16's range (|256 x| above 65,504) are not screened soundly,
+    // and a NaN row is left out by every maximum
+    const bool sound = fits && cmax_bits[1] == 0u && qn < 200.f && cn < 200.f;
     const bool first = sound && cid[0] != INT32_MAX &&
                        (un == 0u || s[0] > __fadd_ru(key_score(un), margin));
     const unsigned b = __ballot_sync(0xffffffffu, first);
@@ -559,7 +561,7 @@ static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe,
     auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 4>
              : a.d <= 256 ? k_prefix_final<kL, KPL, 8>
                           : k_prefix_final<kL, KPL, 16>;
-    f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe,
+    f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe,
                                            cmax, order, cscores, limit);
 }
 

@@ -602,12 +602,14 @@ __global__ void __launch_bounds__(kSelectWarps * 32, KMAX <= 16 ? 8 : 4) k_rank_
     }
 }
 
-// The largest centroid norm (one float, zeroed before the launch; norms are
-// non-negative, so their bit patterns order like the floats)
+// The largest centroid norm (out[0], zeroed before the launch; norms are
+// non-negative, so their bit patterns order like the floats), NaN left out;
+// out[1]: whether there is a NaN
 __global__ void k_cnorm_max(const float *__restrict__ C, int64_t nlist, int d,
                             unsigned *__restrict__ out) {
     const int lane = threadIdx.x & 31;
     float best = 0.f;
+    unsigned bad = 0u;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nlist; c += warps) {
         float ss = 0.f;
@@ -615,12 +617,16 @@ __global__ void k_cnorm_max(const float *__restrict__ C, int64_t nlist, int d,
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
         best = fmaxf(best, sqrtf(ss));
+        bad |= ss != ss ? 1u : 0u;
     }
-    if (lane == 0) atomicMax(out, __float_as_uint(best));
+    if (lane == 0) {
+        atomicMax(out, __float_as_uint(best));
+        if (bad) out[1] = 1u;
+    }
 }
 
 cudaError_t launch_cnorm_max(const float *C, int64_t nlist, int d, unsigned *out, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned), st);
+    cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(nlist, 8), 4 * (int64_t)num_sms());
     k_cnorm_max<<<blocks, 256, 0, st>>>(C, nlist, d, out);
@@ -750,7 +756,7 @@ struct RankPlan {
         return (int64_t)nranges * ((int64_t)cap * entry + 8) + 4 + (group ? gld * 4 + 4 : 0);
     }
 };
-constexpr int64_t kRankFixedBytes = 256;   // the overflow count and the largest centroid norm
+constexpr int64_t kRankFixedBytes = 256;   // the overflow count, the largest centroid norm and its NaN flag
 
 static RankPlan rank_plan(int64_t nq, int64_t nlist, int nprobe, int d, bool bulk) {
     RankPlan L{};

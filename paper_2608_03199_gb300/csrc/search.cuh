@@ -134,7 +134,7 @@ cudaError_t enqueue_rank_tc(const float *Q, int64_t nq, const float *C, int64_t 
                             cudaStream_t st, const unsigned char *tc_cent = nullptr,
                             float *mma_ms = nullptr, int64_t plan_nq = 0,
                             const int *n_dev = nullptr, int64_t n_off = 0);
-// the largest Euclidean norm of nlist rows (one float, as its bits)
+// the largest Euclidean norm of nlist rows (out[0], as its bits) and whether one is NaN (out[1])
 cudaError_t launch_cnorm_max(const float *C, int64_t nlist, int d, unsigned *out, cudaStream_t st);
 int rank_tc_mma_launches(int64_t nq, int64_t nlist, int nprobe, int d, int64_t plan_nq,
                          bool bulk);   // contraction launches

@@ -91,3 +91,19 @@ def test_prefix_host_path(dev):
     b = sieve.search_host(ix, Q.pin_memory(), 0.5, 10, 100, 8, query_ids_host=ids.pin_memory())
     for x, y in zip(a, b):
         assert torch.equal(x.cpu(), y)
+
+
+def test_nan_centroid_is_ranked_as_by_the_full_order(dev):
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 10_000, 96, 320, seed=4)
+    C = ix.centroids.clone()
+    C[17, 3] = float("nan")
+    ix = sieve.build_layout(ix.vectors, torch.repeat_interleave(
+        torch.arange(320, device=dev), ix.list_offsets.diff()).int(), 320, C)
+    Q = X[:5_000].to(dev)
+    qids = torch.full((5_000,), -1, dtype=torch.int64, device=dev)
+    order = sieve.rank_partitions(ix, Q, 64)
+    want = sieve.search(ix, Q, 0.5, 10, 64, 8, query_ids=qids, order=order, check=True)
+    got = sieve.search(ix, Q, 0.5, 10, 64, 8, query_ids=qids, check=True)
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
