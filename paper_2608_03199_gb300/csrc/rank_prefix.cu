@@ -8,34 +8,48 @@
 //
 //   k_prefix_scan   one contraction pass on the screen (one fp16 product of
 //              the hi halves per score, tiles of two 128-query sub-tiles).
-//              Each epilogue thread owns one query and keeps its kL largest
-//              screened scores with their centroid ids, unordered, in shared
-//              memory.  An entry costs about 500 cycles of its warp and holds
-//              the accumulator meanwhile, so the tile first passes over an
+//              Each epilogue thread owns one query and keeps its kL groups of
+//              32 centroids with the largest maxima: the maxima sorted in
+//              registers, each with its slot in the lowest bits, the 32 scores
+//              stored as they are to the slot in global memory.  A group that
+//              enters costs no search and no read: the smallest maximum names
+//              the slot.  The kL largest scores lie in the kL groups with the
+//              largest maxima, and a score of another group is no larger than
+//              the smallest of those maxima.  The tile first passes over an
 //              eighth of its chunks and keeps only the kL largest group
-//              maxima, in registers and without a branch: kL centroids reach
-//              the kL-th, and starting from there a list takes about
-//              kL (1 + ln 8) entries instead of kL (1 + ln(nlist / kL)) in a
-//              random order (1M queries x 8,192 x 256, kL = 16: 6.1 -> 5.7 ms).
-//   k_prefix_final  one warp per query: the kept centroids scored again in
-//              fp32 and sorted by (score desc, id asc).  A centroid that was
-//              not kept screens at most u, the largest of the lists'
-//              thresholds, so its fp32 score is below u plus the error
-//              bounds of both scores; the kept centroids above that are
-//              exactly the first ranks of the order, and their number is the
-//              query's limit.
+//              maxima, without a branch: kL groups reach the kL-th, and
+//              starting from there about kL (1 + ln 8) groups enter instead
+//              of kL (1 + ln(groups / kL)) in a random order.
+//   k_prefix_final  one warp per query: of the kept groups' scores the kL best
+//              (the scores that reach the smallest kept maximum), scored again
+//              in fp32 and sorted by (score desc, id asc).  A centroid that
+//              is not among them screens at most u, the largest of the lists'
+//              bounds and of what was left out here, so its fp32 score is
+//              below u plus the error bounds of both scores; the candidates
+//              above that are exactly the first ranks of the order, and their
+//              number is the query's limit.  Bound by latency: the scores and
+//              the query are loaded before anything depends on them, and the
+//              rows of eight candidates are in flight together (1M x 8,192 x
+//              256: 4.6 ms with eight lanes a row and four rows at a time, 1.6).
 //   k_ext_gather / k_ext_merge  the extension: the listed queries gathered
 //              for the full ranking, whose order follows the prefix with the
 //              prefix's centroids left out, so that no partition is visited
 //              twice should the two disagree on a near-tie.
 //
-// Bound by the epilogue's entries (about half of the 32-score groups have one,
-// in some lane) and the single accumulator per sub-tile they hold meanwhile.
+// The scan is bound by the epilogue and the single accumulator per sub-tile it
+// holds meanwhile: two fifths of the tensor pipe's cycles are used at 8,192 x
+// 256 (issue slots 21% busy: latency).  Against lists of single scores in
+// shared memory, searched at each entry: 1M queries x 65,536 x 96 21.7 -> 13.4
+// ms, 1M x 8,192 x 256 5.7 -> 4.7 ms; for 1,500 centroids, where two thirds of
+// the groups enter, 0.22 ms per 100K both ways, and the final, which reads 2 KB
+// a query and not 128 bytes, takes 0.17 ms, not 0.14.
+// 12 slots instead of 16 (kL) scan faster (12.5 ms for the first) but extend
+// more queries than that saves (the whole search 24.5 -> 25.4 ms).
 // Against the full ranking (two contraction passes, ~310 candidates a query
-// sorted): 1M queries x 65,536 x 96, nprobe 256, 52.1 -> 25.0 ms; 1M x 8,192 x
-// 256, nprobe 128, 17.6 -> 7.7 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.35 ms;
+// sorted): 1M queries x 65,536 x 96, nprobe 256, 52.1 -> 15.0 ms; 1M x 8,192 x
+// 256, nprobe 128, 17.6 -> 6.3 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.39 ms;
 // 200K x 16,384 x 512, nprobe 128 (against the converter pipeline's three
-// products), 16.2 -> 5.0 ms.
+// products), 16.2 -> 4.3 ms.
 #include <cmath>
 #include <vector>
 
@@ -52,9 +66,10 @@ struct PrefixArgs {
     const unsigned char *tc_cent;
     int nranges;         // centroid ranges per query tile
     int64_t range_len;   // centroids per range, a multiple of 128
-    float *list_s;       // [nq][nranges][kL] kept screened scores ...
-    int32_t *list_i;     // ... and their centroids (-1: an unused entry)
-    float *list_t;       // [nq][nranges] what a score left out can be at most (-inf: none was)
+    float *list_s;       // [nq][nranges][kL][32] the kept groups' screened scores (raw: x 2^16) ...
+    int2 *list_g;        // [nq][nranges][kL] ... their largest (raw, as bits) and first centroid
+    float2 *list_t;      // [nq][nranges] x: what a score left out can be at most (raw; -inf: none
+                         // was); y: groups kept, as bits (the last of the kL slots fill first)
 };
 
 __device__ int g_prefix_status_sink;
@@ -100,115 +115,85 @@ struct PrefixMode {
         return a.tc_cent + (T.c0 / kTcRows) * (int64_t)((a.d + 63) / 64) * (kBHasLo ? tcb::kKbBytes : tcb::kKbBytesHi);
     }
     struct Epi {
-        float *ks;      // entry j of this query's list at [j * kRows]
-        int32_t *ki;
+        float *os;       // this query's kL slots of 32 scores
+        int2 *og;
         int64_t at;
-        int n, pos;     // entries in the list; the smallest one's place once it is full
-        float thr;      // raw units: scores up to it are out (-inf: none yet; +inf: no query)
-        bool valid;
-        float top[kL];  // the sample's kL largest group maxima, largest first
-        __device__ void begin(const Args &a, const Tile &T, int slot, unsigned char *smem) {
-            ks = reinterpret_cast<float *>(smem) + slot;
-            ki = reinterpret_cast<int32_t *>(smem + (size_t)kRows * kL * 4) + slot;
-            valid = slot < T.ni;
-            at = (T.q0 + slot) * a.nranges + T.c0 / a.range_len;
-            n = 0;
-            pos = 0;
-            thr = valid ? -__int_as_float(0x7f800000) : __int_as_float(0x7f800000);
+        int n;           // groups taken so far
+        float floor;     // the sample's threshold (-inf: none; +inf: no query)
+        float thr;       // raw units: groups whose maximum is no larger are out
+        // the largest first: the sample's group maxima, then those of the kept
+        // groups, each with its slot in the lowest bits (2^-18 of the value)
+        float top[kL];
+        __device__ __forceinline__ void clear() {
 #pragma unroll
-            for (int j = 0; j < kL; ++j) top[j] = -__int_as_float(0x7f800000);
+            for (int j = 0; j < kL; ++j) top[j] = __uint_as_float(0xff7fffe0u | (unsigned)j);   // about -3.4e38
         }
-        // a sample chunk's scores: the maximum of each 16 into the sorted
-        // registers, without a branch (whole chunks only: no column is past
-        // the range)
-        __device__ __forceinline__ void sample(const float (&v)[32]) {
+        __device__ void begin(const Args &a, const Tile &T, int slot, unsigned char *) {
+            const bool valid = slot < T.ni;
+            at = (T.q0 + slot) * a.nranges + T.c0 / a.range_len;
+            os = a.list_s + at * (kL * 32);
+            og = a.list_g + at * kL;
+            n = 0;
+            clear();
+            floor = valid ? -__int_as_float(0x7f800000) : __int_as_float(0x7f800000);
+            thr = fmaxf(floor, top[kL - 1]);
+        }
+        __device__ __forceinline__ void insert(float x) {   // the smallest leaves
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                float x = fmax3f(fmax3f(v[16 * g], v[16 * g + 1], v[16 * g + 2]),
-                                 fmax3f(v[16 * g + 3], v[16 * g + 4], v[16 * g + 5]),
-                                 fmax3f(v[16 * g + 6], v[16 * g + 7], v[16 * g + 8]));
-                x = fmax3f(x, fmax3f(v[16 * g + 9], v[16 * g + 10], v[16 * g + 11]),
-                           fmax3f(fmaxf(v[16 * g + 12], v[16 * g + 13]), v[16 * g + 14], v[16 * g + 15]));
-#pragma unroll
-                for (int j = 0; j < kL; ++j) {
-                    const float hi = fmaxf(top[j], x);
-                    x = fminf(top[j], x);
-                    top[j] = hi;
-                }
+            for (int j = 0; j < kL; ++j) {
+                const float hi = fmaxf(top[j], x);
+                x = fminf(top[j], x);
+                top[j] = hi;
             }
         }
-        // the sample is through: kL different centroids reach top[kL - 1], so
-        // only scores from there up are listed (the threshold is the value
-        // just below it; the list then fills)
+        // a sample chunk's scores: the maximum of the 32 into the sorted
+        // registers, without a branch (whole chunks only: no column is past
+        // the range)
+        __device__ __forceinline__ void sample(const float (&v)[32]) { insert(max_of_32(v)); }
+        // the sample is through: kL different groups reach top[kL - 1], so
+        // only groups from there up are kept (the threshold is the value just
+        // below it; the slots then fill)
         __device__ __forceinline__ void seed() {
             const float t = top[kL - 1];
-            if (valid && t > -3.402823466e38f && t < 3.402823466e38f)
-                thr = t - fmaxf(fabsf(t), 1.f) * 0x1p-22f;
+            if (floor < 0.f && t > -3.4e38f && t < 3.4e38f) floor = t - fmaxf(fabsf(t), 1.f) * 0x1p-22f;
+            clear();
+            thr = fmaxf(floor, top[kL - 1]);
         }
-        __device__ __forceinline__ void find_smallest() {
-            float w[kL];
+        // a group whose maximum mx passes the threshold takes the slot of the
+        // one that leaves
+        __device__ __forceinline__ void take(const float (&v)[32], float mx, int32_t id0) {
+            const unsigned slot = __float_as_uint(top[kL - 1]) & (unsigned)(kL - 1);
+            insert(__uint_as_float((__float_as_uint(mx) & ~(unsigned)(kL - 1)) | slot));
+            thr = fmaxf(floor, top[kL - 1]);
+            ++n;
+            float4 *o = reinterpret_cast<float4 *>(os + slot * 32);
 #pragma unroll
-            for (int j = 0; j < kL; ++j) w[j] = ks[j * kRows];
-            float t = w[0];
-#pragma unroll
-            for (int j = 1; j < kL; ++j) t = fminf(t, w[j]);
-            int p = 0;
-#pragma unroll
-            for (int j = 1; j < kL; ++j) p = w[j] == t ? j : p;
-            thr = t;
-            pos = p;
+            for (int j = 0; j < 8; ++j) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            og[slot] = make_int2(__float_as_int(mx), id0);
         }
         // v: the chunk's raw accumulator values (scores x 2^16) of centroids
         // T.c0 + col0 + j, j < ncol (warp-uniform)
         __device__ __forceinline__ void chunk(const Args &, const Tile &T, int64_t col0,
                                               const float (&v)[32], int ncol) {
             if (ncol <= 0) return;
-            float mx = v[0];
-            if (ncol == 32) {
-                mx = max_of_32(v);
-            } else {
-#pragma unroll
-                for (int j = 1; j < 32; ++j) mx = j < ncol ? fmaxf(mx, v[j]) : mx;
-            }
-            const bool any = mx > thr;
-            if (!__any_sync(0xffffffffu, any)) return;
-            unsigned m = 0;
-            if (any) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) m |= v[j] > thr ? (1u << j) : 0u;
-                if (ncol < 32) m &= (1u << ncol) - 1u;
-            }
             const int32_t id0 = (int32_t)(T.c0 + col0);
-            while (m) {
-                const int j = __ffs(m) - 1;
-                m &= m - 1u;
-                const float x = pick32(v, j);
-                if (!(x > thr)) continue;   // the threshold rose within this group
-                const int p = n < kL ? n : pos;
-                ks[p * kRows] = x;
-                ki[p * kRows] = id0 + j;
-                if (n < kL) ++n;
-                if (n == kL) find_smallest();
+            if (ncol == 32) {
+                const float mx = max_of_32(v);
+                if (mx > thr) take(v, mx, id0);
+            } else {   // the range's last group: -inf past its end
+                float w[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) w[j] = j < ncol ? v[j] : -__int_as_float(0x7f800000);
+                const float mx = max_of_32(w);
+                if (mx > thr) take(w, mx, id0);
             }
             __syncwarp();
         }
         __device__ void end(const Args &a, const Tile &) {
-            if (!valid) return;
-            a.list_t[at] = thr * (1.f / 65536.f);
-            float4 *os = reinterpret_cast<float4 *>(a.list_s + at * kL);
-            int4 *oi = reinterpret_cast<int4 *>(a.list_i + at * kL);
-#pragma unroll
-            for (int j = 0; j < kL; j += 4) {
-                float s[4];
-                int32_t c[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    s[u] = j + u < n ? ks[(j + u) * kRows] * (1.f / 65536.f) : 0.f;
-                    c[u] = j + u < n ? ki[(j + u) * kRows] : -1;
-                }
-                os[j / 4] = make_float4(s[0], s[1], s[2], s[3]);
-                oi[j / 4] = make_int4(c[0], c[1], c[2], c[3]);
-            }
+            if (floor > 3.4e38f) return;
+            // a group left out had a maximum of thr at most, give or take the slot bits
+            const float t = thr + (fabsf(thr) * 0x1p-18f + 0x1p-100f);
+            a.list_t[at] = make_float2(n >= kL ? t : -__int_as_float(0x7f800000), __int_as_float(n < kL ? n : kL));
         }
         __device__ void prefetch(const Args &, const Tile &, int) {}
         __device__ void start(const Args &, const Tile &, int) {}
@@ -244,100 +229,194 @@ __global__ void k_prefix_fill(const float *__restrict__ C, int64_t nlist, int d,
     }
 }
 
-// One warp per query.  NT: float4 of a row per lane of a group of eight (d <=
-// 32 NT); KPL: list entries per lane (nranges * kL <= 32 KPL).  Ids are checked
-// against nlist: the lists of a pass that gave up are not read as rows.
+// The B partial sums of each lane added up over the warp, halving the sums a
+// lane holds at each step: the sum of acc[j] ends in lanes j * 32 / B and on.
+template <int B>
+__device__ __forceinline__ float warp_sum_each(float (&acc)[B]) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int c = B; c > 1; c >>= 1, off >>= 1) {
+        const bool hi = lane & off;
+#pragma unroll
+        for (int i = 0; i < c / 2; ++i) {
+            const float keep = hi ? acc[i + c / 2] : acc[i], send = hi ? acc[i] : acc[i + c / 2];
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+#pragma unroll
+    for (int o = 16 / B; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+    return acc[0];
+}
+
+// One warp per query.  NV: float4 of a row per lane (d <= 128 NV); KPL: kept
+// groups per lane (nranges * kL <= 32 KPL).
 constexpr int kFinalWarps = 8;
-template <int kL, int KPL, int NT>
+template <int kL, int KPL, int NV>
 __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int64_t nlist, int d,
-    const float *__restrict__ list_s, const int32_t *__restrict__ list_i,
-    const float *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits, int32_t *__restrict__ order, float *__restrict__ cscores,
-    int *__restrict__ limit) {
+    const float *__restrict__ list_s, const int2 *__restrict__ list_g,
+    const float2 *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits,
+    int32_t *__restrict__ order, float *__restrict__ cscores, int *__restrict__ limit) {
+    constexpr float kS = 1.f / 65536.f;
     __shared__ int s_id[kFinalWarps][32];
+    __shared__ int s_slot[kFinalWarps][kL], s_c0[kFinalWarps][kL];   // the groups taken on: slot, first centroid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
     const int64_t q = (int64_t)blockIdx.x * kFinalWarps + warp;
     if (q >= nq) return;
     const int M = nranges * kL;
-    const float *ls = list_s + q * M;
-    const int32_t *li = list_i + q * M;
-    uint32_t key[KPL];
+    // one list: its scores and the query's row are on their way at once
+    float raw[kL];
+    if (M == kL) {
+#pragma unroll
+        for (int g = 0; g < kL; ++g) raw[g] = __ldg(list_s + (q * kL + g) * 32 + lane);
+    }
+    float4 x[NV];
+#pragma unroll
+    for (int t = 0; t < NV; ++t) {
+        const int c = 4 * lane + 128 * t;
+        x[t] = c < d ? __ldg(reinterpret_cast<const float4 *>(Q + q * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     uint32_t un = 0;   // the largest screened score a centroid outside the candidates can have
+    for (int r = lane; r < nranges; r += 32) {
+        const float t = list_t[q * nranges + r].x;
+        if (t > -__int_as_float(0x7f800000)) un = max(un, order_key(t * kS));
+    }
+    // the kL groups with the largest maxima of all ranges (ids are checked
+    // against nlist: lists of a pass that gave up are not read as rows)
+    uint32_t gkey[KPL];
+    int c0[KPL];
 #pragma unroll
     for (int j = 0; j < KPL; ++j) {
         const int c = j * 32 + lane;
-        key[j] = (c < M && (uint32_t)li[c] < (uint64_t)nlist) ? order_key(ls[c]) : 0u;
+        gkey[j] = 0u;
+        c0[j] = -1;
+        if (c < M) {
+            const int used = __float_as_int(list_t[q * nranges + c / kL].y);
+            const int2 g = list_g[q * M + c];
+            if (c % kL >= kL - used && (uint32_t)g.y < (uint64_t)nlist) {
+                gkey[j] = order_key(__int_as_float(g.x) * kS);
+                c0[j] = g.y;
+            }
+        }
     }
-    for (int r = lane; r < nranges; r += 32) {
-        const float t = list_t[q * nranges + r];
-        if (t > -__int_as_float(0x7f800000)) un = max(un, order_key(t));
-    }
-    // the candidates, one per lane: every entry, or the kL largest of several lists
-    int id = -1, n = 0;
-    bool fits = true;
-    if constexpr (KPL == 1) {
-        id = key[0] ? li[lane] : -1;
-        n = M < 32 ? M : 32;
+    uint32_t T = 1u, least = 0xffffffffu;
+    int cnt, ng = 0;
+    if (M == kL) {
+        ng = __popc(__ballot_sync(0xffffffffu, gkey[0] > 0u));
+        if (gkey[0] > 0u) least = gkey[0];
+        if (lane < kL) s_c0[warp][lane] = c0[0];
     } else {
-        uint32_t T;
-        int C32;
-        warp_threshold(key, kL, 32, T, C32);
+        warp_threshold(gkey, kL, kL, T, cnt);
         T = max(T, 1u);
-        const unsigned below = (1u << lane) - 1u;
 #pragma unroll
         for (int j = 0; j < KPL; ++j) {
-            const bool sel = key[j] >= T;
+            const bool sel = gkey[j] >= T;
             const unsigned b = __ballot_sync(0xffffffffu, sel);
-            const int p = n + __popc(b & below);
-            if (sel && p < 32) s_id[warp][p] = li[j * 32 + lane];
-            if (!sel) un = max(un, key[j]);
+            const int p = ng + __popc(b & below);
+            if (sel && p < kL) {
+                s_slot[warp][p] = j * 32 + lane;
+                s_c0[warp][p] = c0[j];
+                least = min(least, gkey[j]);
+            } else {   // not among them (or one of too many equal ones)
+                un = max(un, gkey[j]);
+            }
+            ng += __popc(b);
+        }
+        ng = ng < kL ? ng : kL;
+        __syncwarp();
+#pragma unroll
+        for (int g = 0; g < kL; ++g)
+            raw[g] = g < ng ? list_s[(q * M + s_slot[warp][g]) * 32 + lane] : 0.f;
+    }
+    __syncwarp();
+    // the kL best of their scores (or a few more), one candidate per lane: the
+    // scores that reach the least of the groups' maxima are at least kL, and
+    // seldom more than 32 (neighbours in one group): only then a search
+    int id = -1, n = 0;
+    T = __reduce_min_sync(0xffffffffu, least);
+    const float t_raw = key_score(T) * 65536.f;
+    int reach = 0;
+    if (ng == kL) {
+#pragma unroll
+        for (int g = 0; g < kL; ++g) reach += __popc(__ballot_sync(0xffffffffu, raw[g] >= t_raw));
+    }
+    if (ng == kL && reach <= 32) {   // every other score is below T
+        un = max(un, T);
+#pragma unroll
+        for (int g = 0; g < kL; ++g) {
+            const bool sel = raw[g] >= t_raw;
+            const unsigned b = __ballot_sync(0xffffffffu, sel);
+            if (sel) s_id[warp][n + __popc(b & below)] = s_c0[warp][g] + lane;
             n += __popc(b);
         }
-        fits = n <= 32;   // more: equal scores at the threshold
-        n = n < 32 ? n : 32;
-        __syncwarp();
-        if (lane < n) id = s_id[warp][lane];
+    } else {
+        uint32_t key[kL];
+#pragma unroll
+        for (int g = 0; g < kL; ++g) {
+            const int b = M == kL || g < ng ? s_c0[warp][g] : -1;
+            key[g] = b >= 0 && b + (int64_t)lane < nlist ? order_key(raw[g] * kS) : 0u;
+        }
+        warp_threshold(key, kL, 32, T, cnt);
+        T = max(T, 1u);
+#pragma unroll
+        for (int g = 0; g < kL; ++g) {
+            const bool sel = key[g] >= T;
+            const unsigned b = __ballot_sync(0xffffffffu, sel);
+            const int p = n + __popc(b & below);
+            if (sel && p < 32)
+                s_id[warp][p] = s_c0[warp][g] + lane;
+            else
+                un = max(un, key[g]);
+            n += __popc(b);
+        }
     }
+    n = n < 32 ? n : 32;
+    __syncwarp();
+    if (lane < n) id = s_id[warp][lane];
     un = __reduce_max_sync(0xffffffffu, un);
-    // fp32 scores: eight lanes per candidate, four candidates at a time
-    const int g = lane >> 3, sub = lane & 7;
-    float4 x[NT];
-    float qq = 0.f;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        const int c = 4 * sub + 32 * t;
-        x[t] = c < d ? __ldg(reinterpret_cast<const float4 *>(Q + q * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        qq = fmaf(x[t].x, x[t].x, fmaf(x[t].y, x[t].y, fmaf(x[t].z, x[t].z, fmaf(x[t].w, x[t].w, qq))));
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) qq += __shfl_xor_sync(0xffffffffu, qq, o);
+    // fp32 scores: the whole warp on a candidate, the rows of kB of them in
+    // flight together
+    constexpr int kB = NV == 1 ? 8 : 16 / NV;
     float s[1] = {-__int_as_float(0x7f800000)};
     int cid[1] = {id >= 0 ? id : INT32_MAX};
-#pragma unroll 2
-    for (int it = 0; it < (n + 3) / 4; ++it) {
-        const int ci = __shfl_sync(0xffffffffu, id, it * 4 + g);
-        float acc = 0.f;
-        if (ci >= 0) {
-            const float *row = C + (int64_t)ci * d;
-            float4 y[NT];
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += kB) {
+        float4 y[kB][NV];
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const int c = 4 * sub + 32 * t;
-                y[t] = c < d ? __ldg(reinterpret_cast<const float4 *>(row + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+        for (int i = 0; i < kB; ++i) {
+            // without a branch: past the last candidate the last again, past
+            // the row its start (times x = 0)
+            const float *row = C + (int64_t)s_id[warp][i0 + i < n ? i0 + i : n - 1] * d;
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                acc = fmaf(x[t].x, y[t].x, acc);
-                acc = fmaf(x[t].y, y[t].y, acc);
-                acc = fmaf(x[t].z, y[t].z, acc);
-                acc = fmaf(x[t].w, y[t].w, acc);
+            for (int t = 0; t < NV; ++t) {
+                const int c = 4 * lane + 128 * t;
+                y[i][t] = __ldg(reinterpret_cast<const float4 *>(row + (c < d ? c : 0)));
             }
         }
+        float acc[kB];
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        const float mine = __shfl_sync(0xffffffffu, acc, (lane & 3) * 8);
-        if ((lane >> 2) == it && id >= 0) s[0] = mine;
+        for (int i = 0; i < kB; ++i) {
+            acc[i] = 0.f;
+#pragma unroll
+            for (int t = 0; t < NV; ++t) {
+                acc[i] = fmaf(x[t].x, y[i][t].x, acc[i]);
+                acc[i] = fmaf(x[t].y, y[i][t].y, acc[i]);
+                acc[i] = fmaf(x[t].z, y[i][t].z, acc[i]);
+                acc[i] = fmaf(x[t].w, y[i][t].w, acc[i]);
+            }
+        }
+        const float sum = warp_sum_each<kB>(acc);
+        const float mine = __shfl_sync(0xffffffffu, sum, (lane - i0) * (32 / kB) & 31);
+        if (lane >= i0 && lane < i0 + kB && id >= 0) s[0] = mine;
     }
+    float qq = 0.f;
+#pragma unroll
+    for (int t = 0; t < NV; ++t)
+        qq = fmaf(x[t].x, x[t].x, fmaf(x[t].y, x[t].y, fmaf(x[t].z, x[t].z, fmaf(x[t].w, x[t].w, qq))));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) qq += __shfl_xor_sync(0xffffffffu, qq, o);
     warp_sort_regs<1>(s, cid);
     // the norms and the margin rounded upward (the bounds of k_rank_threshold:
     // the screen's, and one that covers fp32 sums with room)
@@ -349,7 +428,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const float margin = (scr + fp32) * (1.f + 0x1p-16f);
     // scores past fp16's range (|256 x| above 65,504) are not screened soundly,
     // and a NaN row is left out by every maximum
-    const bool sound = fits && cmax_bits[1] == 0u && qn < 200.f && cn < 200.f;
+    const bool sound = cmax_bits[1] == 0u && qn < 200.f && cn < 200.f;
     const bool first = sound && cid[0] != INT32_MAX &&
                        (un == 0u || s[0] > __fadd_ru(key_score(un), margin));
     const unsigned b = __ballot_sync(0xffffffffu, first);
@@ -418,12 +497,11 @@ static int prefix_sub(int d) { return ceil_div(d, 64) <= 4 ? 2 : 1; }   // sub-t
 static uint32_t prefix_stage_bytes(int d) {
     return prefix_wide(d) ? tcb::kStageBytesHi / tcb::kN * 192 : tcb::kStageBytesHi;
 }
-static size_t prefix_epi_bytes(int d, int L) { return (size_t)prefix_sub(d) * tcp::kM * L * 8; }
 
-static int prefix_stages(int d, int L) {
+static int prefix_stages(int d) {
     const int nkb = (int)ceil_div(d, 64);
     return tcb::sub_fits(nkb, 1, prefix_sub(d))
-               ? tcb::stages_for(nkb, prefix_epi_bytes(d, L), 232448 - 128, prefix_stage_bytes(d), tcb::kStagesMax,
+               ? tcb::stages_for(nkb, 0, 232448 - 128, prefix_stage_bytes(d), tcb::kStagesMax,
                                  tcb::kMaxKb)
                : 0;
 }
@@ -433,13 +511,13 @@ static int64_t fill_bytes(int64_t nlist, int d) {
     return prefix_sub(d) == 2 ? 0 : ceil_div(nlist, kTcRows) * ceil_div(d, 64) * tcb::kKbBytesHi;
 }
 
-// Entries kept per list: min(W, nprobe) ranks are visited for certain, a hit at
-// rank j adds up to rank j + W, and one or two entries are lost to the margin.
-// 16 entries serve windows up to 10 and 32 up to 24; 0: rank all of nprobe (a
+// Groups kept per list, and so ranks found: min(W, nprobe) are visited for
+// certain, a hit at rank j adds up to rank j + W, and one or two are lost to
+// the margin.  16 serve windows up to 10 and 32 up to 24; 0: rank all of nprobe (a
 // wider window reads most of the order anyway, and a list of fewer than 64
 // centroids is ranked whole as cheaply).
 static bool prefix_fits(int64_t nlist, int nprobe, int d, int L) {
-    return nlist >= 4 * (int64_t)L && nprobe >= 4 && prefix_stages(d, L) > 0;
+    return nlist >= 4 * (int64_t)L && nprobe >= 4 && prefix_stages(d) > 0;
 }
 
 int rank_prefix_len(int64_t nlist, int nprobe, int W, int d) {
@@ -447,6 +525,10 @@ int rank_prefix_len(int64_t nlist, int nprobe, int W, int d) {
     const int L = need <= 10 ? 16 : need <= 24 ? 32 : 0;
     return L && prefix_fits(nlist, nprobe, d, L) ? L : 0;
 }
+
+// bytes of one (query, range)'s list: the scores, maxima and first centroids of
+// L groups, the bound and the count
+static int64_t list_bytes(int L) { return (int64_t)L * (32 * 4 + 8) + 8; }
 
 struct PrefixPlan {
     int nranges;
@@ -496,8 +578,10 @@ static int64_t ext_bytes(int64_t x, int64_t nlist, int nprobe, int d, PrefixScra
     return off;
 }
 
-// The scratch stays within what the full ranking takes (plain) wherever a
-// chunk of queries fits it; a smaller chunk only means more passes.
+// The scratch is what the full ranking takes (plain), or up to kPrefixListBytes
+// of lists where that is more; a smaller chunk only means more passes, and a
+// chunk past one wave of tiles is a number of whole waves.
+constexpr int64_t kPrefixListBytes = int64_t(1) << 30;
 static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d, int L) {
     PrefixScratch S{};
     const int64_t plain = (int64_t)rank_tc_scratch_bytes(nq, nlist, nprobe, d);
@@ -512,11 +596,16 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
     }
     S.total = std::max(end, plain);
     const PrefixPlan P = prefix_plan(nq, nlist, d, L);
-    const int64_t per = (int64_t)P.nranges * (L * 8 + 4);
+    const int64_t per = (int64_t)P.nranges * list_bytes(L), least = std::min<int64_t>(nq, 2 * tcp::kM) * per;
     S.fill = S.rest + 256;
     S.lists = S.fill + fill_bytes(nlist, d);
-    S.total = std::max(S.total, S.lists + std::min<int64_t>(nq, 2 * tcp::kM) * per + 256);
-    S.chunk = std::min(nq, std::max<int64_t>(2 * tcp::kM, (S.total - S.lists - 256) / per / (2 * tcp::kM) * (2 * tcp::kM)));
+    S.total = std::max(S.total, S.lists + std::max(least, std::min(nq * per, kPrefixListBytes)) + 256);
+    S.chunk = (S.total - S.lists - 256) / per;
+    if (S.chunk < nq) {
+        const int64_t tile = 2 * tcp::kM, wave = tile * num_sms();
+        S.chunk = std::max(tile, S.chunk / (S.chunk < wave ? tile : wave) * (S.chunk < wave ? tile : wave));
+    }
+    S.chunk = std::min(nq, S.chunk);
     return S;
 }
 
@@ -536,8 +625,8 @@ int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int
     return reinterpret_cast<int *>(w + S.limit);
 }
 
-static size_t scan_smem(int d, int L) {
-    return tcb::smem_bytes(prefix_stages(d, L), prefix_epi_bytes(d, L), prefix_stage_bytes(d));
+static size_t scan_smem(int d) {
+    return tcb::smem_bytes(prefix_stages(d), 0, prefix_stage_bytes(d));
 }
 
 // the scan kernel of this d and list length
@@ -551,17 +640,17 @@ static PrefixScan scan_kernel(int d, int L) {
 cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d) {
     const int L = rank_prefix_len(nlist, nprobe, W, d);
     return cudaFuncSetAttribute(scan_kernel(d, L), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)scan_smem(d, L));
+                                (int)scan_smem(d));
 }
 
 template <int kL, int KPL>
 static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, const unsigned *cmax,
                                 int32_t *order, float *cscores, int *limit, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(a.nq, kFinalWarps);
-    auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 4>
-             : a.d <= 256 ? k_prefix_final<kL, KPL, 8>
-                          : k_prefix_final<kL, KPL, 16>;
-    f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_i, a.list_t, a.nranges, nprobe,
+    auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 1>
+             : a.d <= 256 ? k_prefix_final<kL, KPL, 2>
+                          : k_prefix_final<kL, KPL, 4>;
+    f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_g, a.list_t, a.nranges, nprobe,
                                            cmax, order, cscores, limit);
 }
 
@@ -590,10 +679,10 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     unsigned *cmax = reinterpret_cast<unsigned *>(w + S.rest);
     float *list_s = reinterpret_cast<float *>(w + S.lists);
     const int64_t slots = S.chunk * P.nranges * L;
-    int32_t *list_i = reinterpret_cast<int32_t *>(list_s + slots);
-    float *list_t = reinterpret_cast<float *>(list_i + slots);
-    const int stages = prefix_stages(d, L);
-    const size_t smem = scan_smem(d, L);
+    int2 *list_g = reinterpret_cast<int2 *>(list_s + slots * 32);
+    float2 *list_t = reinterpret_cast<float2 *>(list_g + slots);
+    const int stages = prefix_stages(d);
+    const size_t smem = scan_smem(d);
     const PrefixScan scan = scan_kernel(d, L);
     struct Events {
         std::vector<cudaEvent_t> v;
@@ -611,7 +700,7 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);
-        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, tc_cent, P.nranges, P.range_len, list_s, list_i, list_t};
+        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, tc_cent, P.nranges, P.range_len, list_s, list_g, list_t};
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, prefix_sub(d) * tcp::kM) * P.nranges, num_sms());
         if (mma_ms) {
             ev.v.resize(ev.v.size() + 2);
