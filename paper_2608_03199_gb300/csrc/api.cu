@@ -201,8 +201,8 @@ cudaError_t launch_search_rank(const SearchArgs &a, int rank_tc, cudaStream_t st
 }
 
 // the end of a round that met queries whose stop line passes their prefix
-cudaError_t launch_search_ext(const SearchArgs &a, cudaStream_t st) {
-    return enqueue_rank_ext(a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, const_cast<int32_t *>(a.order),
+cudaError_t launch_search_ext(const SearchArgs &a, int part, cudaStream_t st) {
+    return enqueue_rank_ext(part, a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, const_cast<int32_t *>(a.order),
                             a.cscores, a.rank_scratch, &a.ctl->ext_n, &a.ctl->status, a.tc_cent, st);
 }
 
@@ -241,15 +241,16 @@ sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_
     SIEVE_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaSuccess;
-    cudaGraphConditionalHandle cond = 0, ext_cond = 0;
-    cudaGraph_t body = nullptr, ext_body = nullptr;
+    RoundConds conds{};
+    cudaGraphConditionalHandle more_ext = 0;
+    cudaGraph_t body = nullptr, ext_body = nullptr, more_body = nullptr;
     do {
         // outer graph: init -> [rank] -> WHILE(rounds) -> finalize
         if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
         e = launch_init(a, cs);
         if (e == cudaSuccess && a.rq) e = launch_search_rotate(a, cs);
         if (e == cudaSuccess && key.with_rank) e = launch_search_rank(a, key.rank_tc, cs);
-        if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeWhile, 1, &cond, &body);
+        if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeWhile, 1, &conds.more, &body);
         if (e == cudaSuccess) e = launch_finalize(a, cs);
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         if (e == cudaSuccess) e = e2;
@@ -258,9 +259,9 @@ sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_
         if ((e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0,
                                                cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             break;
-        if (a.limit) e = cudaGraphConditionalHandleCreate(&ext_cond, body, 0, cudaGraphCondAssignDefault);
-        if (e == cudaSuccess) e = launch_round(a, key.scan_smem, key.scan_blocks, cond, ext_cond, 1, cs);
-        if (e == cudaSuccess && a.limit) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &ext_cond, &ext_body);
+        if (a.limit) e = cudaGraphConditionalHandleCreate(&conds.ext, body, 0, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) e = launch_round(a, key.scan_smem, key.scan_blocks, &conds, cs);
+        if (e == cudaSuccess && a.limit) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &conds.ext, &ext_body);
         e2 = cudaStreamEndCapture(cs, &body);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess) break;
@@ -268,8 +269,23 @@ sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_
             if ((e = cudaStreamBeginCaptureToGraph(cs, ext_body, nullptr, nullptr, 0,
                                                    cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
                 break;
-            e = launch_search_ext(a, cs);
+            e = launch_search_ext(a, 0, cs);
+            if (a.nq > kExtFirst) {
+                if (e == cudaSuccess)
+                    e = cudaGraphConditionalHandleCreate(&more_ext, ext_body, 0, cudaGraphCondAssignDefault);
+                if (e == cudaSuccess) e = launch_ext_more(a, more_ext, cs);
+                if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &more_ext, &more_body);
+            }
             e2 = cudaStreamEndCapture(cs, &ext_body);
+            if (e == cudaSuccess) e = e2;
+            if (e != cudaSuccess) break;
+        }
+        if (more_body) {
+            if ((e = cudaStreamBeginCaptureToGraph(cs, more_body, nullptr, nullptr, 0,
+                                                   cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+                break;
+            e = launch_search_ext(a, 1, cs);
+            e2 = cudaStreamEndCapture(cs, &more_body);
             if (e == cudaSuccess) e = e2;
             if (e != cudaSuccess) break;
         }
@@ -551,7 +567,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                 return launch_search_rank(a, rank_tc, st, p->profile ? &ms[SIEVE_K_RANK_MMA] : nullptr);
             }));
         for (;;) {
-            SIEVE_CUDA(launch_round(a, smem, blocks, 0, 0, 0, st, p->profile ? ev.e : nullptr));
+            SIEVE_CUDA(launch_round(a, smem, blocks, nullptr, st, p->profile ? ev.e : nullptr));
             // the status word, the loop flag and the extension's count are
             // adjacent in the control block
             static_assert(offsetof(Ctl, more) == offsetof(Ctl, status) + sizeof(int) &&
@@ -572,7 +588,8 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                 }
             }
             if (!more) break;
-            if (prefix && word[2] > 0) SIEVE_CUDA(timed(SIEVE_K_RANK, [&] { return launch_search_ext(a, st); }));
+            for (int i = 0; prefix && i < 2 && word[2] > (i ? kExtFirst : 0); ++i)
+                SIEVE_CUDA(timed(SIEVE_K_RANK, [&] { return launch_search_ext(a, i, st); }));
         }
         SIEVE_CUDA(timed(SIEVE_K_FINALIZE, [&] { return launch_finalize(a, st); }));
     }

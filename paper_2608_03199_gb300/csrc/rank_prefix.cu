@@ -562,20 +562,21 @@ struct PrefixScratch {
     int64_t limit, ext, rest;      // byte offsets
     int64_t fill, lists;           // the prefix's part: the centroids' hi halves, the lists
     int64_t chunk;                 // queries per prefix pass
-    int64_t ext_chunk;             // queries per extension pass
-    int64_t ext_q, ext_order, ext_s;   // byte offsets of the extension's buffers (after its ranking scratch)
+    struct Ext {                   // a part of the extension: queries per pass, and byte offsets
+        int64_t chunk;             // of its buffers (after its ranking scratch)
+        int64_t q, order, s, end;
+    } ext_part[2];
     int64_t total;
 };
 
-static int64_t ext_bytes(int64_t x, int64_t nlist, int nprobe, int d, PrefixScratch *S) {
-    int64_t off = S->rest + round_up((int64_t)rank_tc_scratch_bytes(x, nlist, nprobe, d), 256);
-    S->ext_q = off;
-    off += round_up(x * d * 4, 256);
-    S->ext_order = off;
-    off += round_up(x * nprobe * 4, 256);
-    S->ext_s = off;
-    off += round_up(x * nprobe * 4, 256);
-    return off;
+static PrefixScratch::Ext ext_part(int64_t rest, int64_t x, int64_t nlist, int nprobe, int d) {
+    PrefixScratch::Ext E{};
+    E.chunk = x;
+    E.q = rest + round_up((int64_t)rank_tc_scratch_bytes(x, nlist, nprobe, d), 256);
+    E.order = E.q + round_up(x * d * 4, 256);
+    E.s = E.order + round_up(x * nprobe * 4, 256);
+    E.end = E.s + round_up(x * nprobe * 4, 256);
+    return E;
 }
 
 // The scratch is what the full ranking takes (plain), or up to kPrefixListBytes
@@ -588,13 +589,15 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
     S.limit = 0;
     S.ext = round_up(nq * 4, 256);
     S.rest = S.ext + round_up(nq * 4, 256);
-    S.ext_chunk = nq;
-    int64_t end = ext_bytes(nq, nlist, nprobe, d, &S);
-    while (end > plain && S.ext_chunk > 128) {
-        S.ext_chunk = std::max<int64_t>(128, round_up(ceil_div(S.ext_chunk, 2), 128));
-        end = ext_bytes(S.ext_chunk, nlist, nprobe, d, &S);
+    S.ext_part[0] = ext_part(S.rest, std::min(nq, kExtFirst), nlist, nprobe, d);
+    S.total = std::max(S.ext_part[0].end, plain);
+    if (nq > kExtFirst) {
+        PrefixScratch::Ext &E = S.ext_part[1];
+        E = ext_part(S.rest, nq - kExtFirst, nlist, nprobe, d);
+        while (E.end > S.total && E.chunk > kExtFirst)
+            E = ext_part(S.rest, std::max(kExtFirst, round_up(ceil_div(E.chunk, 2), (int64_t)128)), nlist, nprobe, d);
+        S.total = std::max(S.total, E.end);
     }
-    S.total = std::max(end, plain);
     const PrefixPlan P = prefix_plan(nq, nlist, d, L);
     const int64_t per = (int64_t)P.nranges * list_bytes(L), least = std::min<int64_t>(nq, 2 * tcp::kM) * per;
     S.fill = S.rest + 256;
@@ -738,24 +741,27 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
 }
 
 // The extension: the full ranking of the queries ext[0 .. *ext_n - 1], behind
-// their prefixes.  Every pass is launched; passes past *ext_n find no work.
-cudaError_t enqueue_rank_ext(const float *Q, int64_t nq, const float *C, int64_t nlist, int d, int nprobe,
-                             int W, int32_t *order, float *cscores, void *scratch, const int *ext_n,
-                             int *status, const unsigned char *tc_cent, cudaStream_t st) {
+// their prefixes; part 0 the first kExtFirst of them, part 1 the others.
+// Every pass is launched; passes past *ext_n find no work.
+cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
+                             int nprobe, int W, int32_t *order, float *cscores, void *scratch,
+                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st) {
     const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    const PrefixScratch::Ext &E = S.ext_part[part];
     unsigned char *w = static_cast<unsigned char *>(scratch);
     int *limit = reinterpret_cast<int *>(w + S.limit);
     const int *ext = reinterpret_cast<const int *>(w + S.ext);
-    float *Qx = reinterpret_cast<float *>(w + S.ext_q);
-    int32_t *full = reinterpret_cast<int32_t *>(w + S.ext_order);
-    float *full_s = cscores ? reinterpret_cast<float *>(w + S.ext_s) : nullptr;
+    float *Qx = reinterpret_cast<float *>(w + E.q);
+    int32_t *full = reinterpret_cast<int32_t *>(w + E.order);
+    float *full_s = cscores ? reinterpret_cast<float *>(w + E.s) : nullptr;
     const int blocks = 4 * num_sms();
-    for (int64_t b = 0; b < nq; b += S.ext_chunk) {
-        const int64_t n = std::min(S.ext_chunk, nq - b);
+    const int64_t lo = part ? kExtFirst : 0, hi = part ? nq : std::min(nq, kExtFirst);
+    for (int64_t b = lo; b < hi; b += E.chunk) {
+        const int64_t n = std::min(E.chunk, hi - b);
         k_ext_gather<<<blocks, 256, 0, st>>>(Q, d, ext, ext_n, b, n, Qx);
         cudaError_t e = enqueue_rank_tc(Qx, n, C, nlist, d, nprobe, full, full_s,
                                         reinterpret_cast<float *>(w + S.rest), status, st, tc_cent, nullptr,
-                                        S.ext_chunk, ext_n, b);
+                                        E.chunk, ext_n, b);
         if (e != cudaSuccess) return e;
         k_ext_merge<<<blocks, 256, 0, st>>>(ext, ext_n, b, n, nprobe, full, full_s, order, cscores, limit);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -86,9 +86,13 @@ int scan_blocks_for(size_t smem);
 cudaError_t prepare_scan_kernel(size_t smem);
 cudaError_t launch_init(const SearchArgs &a, cudaStream_t st);
 cudaError_t launch_finalize(const SearchArgs &a, cudaStream_t st);
-cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
-                         cudaGraphConditionalHandle cond, cudaGraphConditionalHandle ext_cond,
-                         int use_cond, cudaStream_t st, cudaEvent_t *ev = nullptr);
+// the loop's condition and that of the ranking's extension
+struct RoundConds {
+    cudaGraphConditionalHandle more, ext;
+};
+// conds: null outside a graph
+cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks, const RoundConds *conds,
+                         cudaStream_t st, cudaEvent_t *ev = nullptr);
 constexpr int kRoundKernels = 7;   // issue, bucket, scatter, scan_tc, scan, merge, round_end
 
 // tensor-core scan (scan_tc.cu)
@@ -158,9 +162,15 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
                                 float *mma_ms = nullptr);
-cudaError_t enqueue_rank_ext(const float *Q, int64_t nq, const float *C, int64_t nlist, int d, int nprobe,
-                             int W, int32_t *order, float *cscores, void *scratch, const int *ext_n,
-                             int *status, const unsigned char *tc_cent, cudaStream_t st);
+// an extension in two parts: the first kExtFirst queries as a small batch, cut
+// into ranges that fill the SMs (as part of a batch of all queries they were a
+// few tiles that each went over all centroids), and the rest, if there are any
+constexpr int64_t kExtFirst = 4096;
+// sets cond (of a node that follows in the same graph) where part 1 has queries
+cudaError_t launch_ext_more(const SearchArgs &a, cudaGraphConditionalHandle cond, cudaStream_t st);
+cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
+                             int nprobe, int W, int32_t *order, float *cscores, void *scratch,
+                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st);
 
 // in-call window calibration (calibrate.cu)
 cudaError_t calib_gather(const float *Q, const int64_t *qids, int d, const int64_t *idx, int64_t n,

@@ -563,8 +563,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(SearchArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-__global__ void k_round_end(SearchArgs a, cudaGraphConditionalHandle cond,
-                            cudaGraphConditionalHandle ext_cond, int use_cond) {
+__global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
     Ctl *c = a.ctl;
     const int items = c->n_items < a.cap ? c->n_items : (int)a.cap;
     c->tot_items += (unsigned long long)items;
@@ -587,9 +586,13 @@ __global__ void k_round_end(SearchArgs a, cudaGraphConditionalHandle cond,
     c->n_deferred = 0;
     c->n_continue = 0;
     if (use_cond) {
-        cudaGraphSetConditional(cond, more ? 1u : 0u);
-        if (a.limit) cudaGraphSetConditional(ext_cond, c->ext_n > 0 ? 1u : 0u);
+        cudaGraphSetConditional(conds.more, more ? 1u : 0u);
+        if (a.limit) cudaGraphSetConditional(conds.ext, c->ext_n > 0 ? 1u : 0u);
     }
+}
+
+__global__ void k_ext_more(const Ctl *c, cudaGraphConditionalHandle cond) {
+    cudaGraphSetConditional(cond, c->ext_n > kExtFirst ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -627,9 +630,13 @@ cudaError_t launch_finalize(const SearchArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
-                         cudaGraphConditionalHandle cond, cudaGraphConditionalHandle ext_cond,
-                         int use_cond, cudaStream_t st, cudaEvent_t *ev) {
+cudaError_t launch_ext_more(const SearchArgs &a, cudaGraphConditionalHandle cond, cudaStream_t st) {
+    k_ext_more<<<1, 1, 0, st>>>(a.ctl, cond);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks, const RoundConds *conds,
+                         cudaStream_t st, cudaEvent_t *ev) {
     // ev (optional): 2 * kRoundKernels events, recorded before/after each kernel
     const int sms = num_sms();
     int slot = 0;
@@ -670,7 +677,7 @@ cudaError_t launch_round(const SearchArgs &a, size_t scan_smem, int scan_blocks,
     k_merge<<<merge_blocks, kMergeThreads, 0, st>>>(a);
     end();
     begin();
-    k_round_end<<<1, 1, 0, st>>>(a, cond, ext_cond, use_cond);
+    k_round_end<<<1, 1, 0, st>>>(a, conds ? *conds : RoundConds{}, conds != nullptr);
     end();
     return cudaGetLastError();
 }

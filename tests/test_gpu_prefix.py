@@ -50,6 +50,7 @@ CASES = [  # n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal
     (12_000, 260, 2_100, 300, 64, 16, 0.45, True, True, 0),
     (12_000, 448, 300, 129, 64, 8, 0.50, False, False, 0),
     (3_000, 96, 64, 1, 64, 8, 0.20, True, False, 0),
+    (12_000, 64, 2_500, 9_001, 64, 8, 0.20, True, False, 0),   # nearly every query extended: both parts
     (8_000, 96, 2_309, 5_000, 64, 16, 0.45, True, True, 0),    # a last group of five centroids
 ]
 
