@@ -49,7 +49,7 @@
 // sorted): 1M queries x 65,536 x 96, nprobe 256, 52.1 -> 15.0 ms; 1M x 8,192 x
 // 256, nprobe 128, 17.6 -> 6.3 ms; 100K x 1,500 x 96, nprobe 90, 1.35 -> 0.39 ms;
 // 200K x 16,384 x 512, nprobe 128 (against the converter pipeline's three
-// products), 16.2 -> 4.3 ms.
+// products), 16.2 -> 4.1 ms.
 #include <cmath>
 #include <vector>
 
