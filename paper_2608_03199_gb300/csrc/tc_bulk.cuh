@@ -655,8 +655,8 @@ __device__ __forceinline__ void run_bulk(const typename Mode::Args &a, unsigned 
                 // the loop unrolled the epilogue waits for instructions (join
                 // of 100K queries with 1M x 256, W = 8: scan 1.70 -> 1.23 ms;
                 // two sub-tiles, a pair of loads in flight per step: screen
-                // pass + lists over 65,536 x 96 27.6 -> 21.7 ms, 23.8 with
-                // single loads).  The accumulator is released as soon as the
+                // pass + lists of single scores over 65,536 x 96 27.6 -> 21.7
+                // ms, 23.8 with single loads; 13.4 ms with lists of groups).  The accumulator is released as soon as the
                 // last load has landed, before its columns go to the mode.
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + buf * kNB;
                 const int64_t col0 = (int64_t)ch * kNB;
