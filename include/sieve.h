@@ -94,8 +94,10 @@ typedef struct {
  *              (query, rank) item is its own partition call, one query
  *              against the partition's rows, with the same stopping rule and
  *              the same results; a baseline for measurement
- *   wait_limit iteration limit of one device wait: the tensor-core scan
- *              epilogue's wait for an accumulator (a wait with no
+ *   wait_limit iteration limit of one device wait: the wait for an
+ *              accumulator in the epilogue of the tensor-core scan and of
+ *              the pass that ranks the first centroids of a search with a
+ *              small window (a wait with no
  *              asynchronous work of its own outstanding); 0 = the default,
  *              2^24 polls.  A testing aid for the bounded waits: a wait that
  *              gives up records SIEVE_ETIMEOUT in the call's status word,

@@ -193,7 +193,7 @@ cudaError_t launch_search_rank(const SearchArgs &a, int rank_tc, cudaStream_t st
     int32_t *order = const_cast<int32_t *>(a.order);
     if (a.limit)
         return enqueue_rank_prefix(a.Q, 0, a.nq, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, order, a.cscores,
-                                   a.rank_scratch, &a.ctl->status, a.tc_cent, st, mma_ms);
+                                   a.rank_scratch, &a.ctl->status, a.tc_cent, st, mma_ms, a.wait_limit);
     if (rank_tc)
         return enqueue_rank_tc(a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, order, a.cscores,
                                a.rank_scratch, &a.ctl->status, st, a.tc_cent, mma_ms);
@@ -988,7 +988,8 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
         if (prefix) {
             SIEVE_CUDA(enqueue_rank_prefix(dQ, q0, n, nq, ix->centroids, ix->nlist, ix->d, p->nprobe, p->W,
                                            dorder, nullptr, w + L.rank_scratch, dstatus,
-                                           static_cast<const unsigned char *>(ix->tc_centroids), st));
+                                           static_cast<const unsigned char *>(ix->tc_centroids), st, nullptr,
+                                           p->wait_limit));
             int mma = 0;
             rank_launches += rank_prefix_launches(n, nq, ix->nlist, p->nprobe, p->W, ix->d, &mma);
             mma_launches += mma;

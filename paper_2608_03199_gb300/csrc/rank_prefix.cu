@@ -63,6 +63,7 @@ struct PrefixArgs {
     int64_t nq, nlist;
     int d;
     int *status;
+    int wait_limit;      // polls of the epilogue's accumulator wait (0: default)
     const unsigned char *tc_cent;
     int nranges;         // centroid ranges per query tile
     int64_t range_len;   // centroids per range, a multiple of 128
@@ -96,6 +97,7 @@ struct PrefixMode {
     __device__ static int *tile_counter(const Args &) { return nullptr; }
     __device__ static int d(const Args &a) { return a.d; }
     __device__ static int *status(const Args &a) { return a.status ? a.status : &g_prefix_status_sink; }
+    __device__ static uint32_t epi_wait_polls(const Args &a) { return (uint32_t)a.wait_limit; }
     __device__ static Tile tile(const Args &a, int t) {
         Tile T;
         T.q0 = (int64_t)(t / a.nranges) * kRows;
@@ -250,14 +252,18 @@ __device__ __forceinline__ float warp_sum_each(float (&acc)[B]) {
 }
 
 // One warp per query.  NV: float4 of a row per lane (d <= 128 NV); KPL: kept
-// groups per lane (nranges * kL <= 32 KPL).
+// groups per lane (nranges * kL <= 32 KPL).  A scan that gave up on a wait
+// leaves lists that an earlier call wrote, or nobody: with the status word set
+// no list is read, and every prefix is empty.  A row is read only where its id
+// is below nlist (a group at the end of the centroids has fewer than 32).
 constexpr int kFinalWarps = 8;
 template <int kL, int KPL, int NV>
 __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int64_t nlist, int d,
     const float *__restrict__ list_s, const int2 *__restrict__ list_g,
     const float2 *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits,
-    int32_t *__restrict__ order, float *__restrict__ cscores, int *__restrict__ limit) {
+    const int *__restrict__ status, int32_t *__restrict__ order, float *__restrict__ cscores,
+    int *__restrict__ limit) {
     constexpr float kS = 1.f / 65536.f;
     __shared__ int s_id[kFinalWarps][32];
     __shared__ int s_slot[kFinalWarps][kL], s_c0[kFinalWarps][kL];   // the groups taken on: slot, first centroid
@@ -265,6 +271,10 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const unsigned below = (1u << lane) - 1u;
     const int64_t q = (int64_t)blockIdx.x * kFinalWarps + warp;
     if (q >= nq) return;
+    if (status && *status != 0) {
+        if (lane == 0) limit[q] = 0;
+        return;
+    }
     const int M = nranges * kL;
     // one list: its scores and the query's row are on their way at once
     float raw[kL];
@@ -283,8 +293,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
         const float t = list_t[q * nranges + r].x;
         if (t > -__int_as_float(0x7f800000)) un = max(un, order_key(t * kS));
     }
-    // the kL groups with the largest maxima of all ranges (ids are checked
-    // against nlist: lists of a pass that gave up are not read as rows)
+    // the kL groups with the largest maxima of all ranges
     uint32_t gkey[KPL];
     int c0[KPL];
 #pragma unroll
@@ -346,7 +355,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
         un = max(un, T);
 #pragma unroll
         for (int g = 0; g < kL; ++g) {
-            const bool sel = raw[g] >= t_raw;
+            const bool sel = raw[g] >= t_raw && s_c0[warp][g] + lane < nlist;
             const unsigned b = __ballot_sync(0xffffffffu, sel);
             if (sel) s_id[warp][n + __popc(b & below)] = s_c0[warp][g] + lane;
             n += __popc(b);
@@ -654,7 +663,7 @@ static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe,
              : a.d <= 256 ? k_prefix_final<kL, KPL, 2>
                           : k_prefix_final<kL, KPL, 4>;
     f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_g, a.list_t, a.nranges, nprobe,
-                                           cmax, order, cscores, limit);
+                                           cmax, a.status, order, cscores, limit);
 }
 
 // kernel launches of one prefix ranking of nq queries (and its contraction
@@ -672,7 +681,7 @@ int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe,
 cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
-                                float *mma_ms) {
+                                float *mma_ms, int wait_limit) {
     if (nq <= 0) return cudaSuccess;
     const int L = rank_prefix_len(nlist, nprobe, W, d);
     const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
@@ -703,7 +712,8 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);
-        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, tc_cent, P.nranges, P.range_len, list_s, list_g, list_t};
+        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, wait_limit, tc_cent, P.nranges, P.range_len,
+                           list_s, list_g, list_t};
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, prefix_sub(d) * tcp::kM) * P.nranges, num_sms());
         if (mma_ms) {
             ev.v.resize(ev.v.size() + 2);

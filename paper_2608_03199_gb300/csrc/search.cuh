@@ -26,7 +26,8 @@ struct SearchArgs {
     float tau;
     int k, nprobe, W, lookahead;
     int serial;                // 1: every (query, rank) item is its own tile (serial traversal)
-    int wait_limit;            // polls of the tensor-core scan epilogue's accumulator wait (0: default)
+    int wait_limit;            // polls of the accumulator wait in the epilogues of the tensor-core scan
+                               // and of the prefix ranking's scan (0: default)
     // prefix ranking (rank_prefix.cu), nullable: the ranks of each query's
     // order that are in place, and the queries whose stop line passes them
     int *limit, *ext;
@@ -161,7 +162,7 @@ int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe,
 cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
-                                float *mma_ms = nullptr);
+                                float *mma_ms = nullptr, int wait_limit = 0);
 // an extension in two parts: the first kExtFirst queries as a small batch, cut
 // into ranges that fill the SMs (as part of a batch of all queries they were a
 // few tiles that each went over all centroids), and the rest, if there are any
