@@ -269,7 +269,10 @@ sieve_status sieve_screen_scores(const sieve_index_view *ix, const float *Q, int
 
 /* Workspace bytes sieve_search needs for nq queries with these parameters.
  * host_io = 1 sizes it for sieve_search_host (adds device staging for the
- * queries and results). */
+ * queries and results).  With a small window it includes the lists with which
+ * a search ranks the first centroids of each order before the rest; a search
+ * takes a workspace without room for them (one sized for other parameters)
+ * all the same, and ranks every order whole. */
 sieve_status sieve_search_workspace_size(const sieve_index_view *ix, int64_t nq,
                                          const sieve_params *p, int32_t host_io,
                                          size_t *bytes);
@@ -340,8 +343,9 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
  * graph (rounds are host-driven, one stream sync per round, whatever
  * p->loop says), no events (p->profile must be 0).
  *   - A call whose scratch need (sieve_search_workspace_size with
- *     host_io = 0) exceeds SIEVE_NOALLOC_SCRATCH_BYTES returns
- *     SIEVE_ESCRATCH and touches nothing.
+ *     host_io = 0, less the lists named there where they do not fit)
+ *     exceeds SIEVE_NOALLOC_SCRATCH_BYTES returns SIEVE_ESCRATCH and
+ *     touches nothing.
  *   - Every call looks the array's device address up on the current device
  *     (cudaGetSymbolAddress; the address is not cached, so it stays valid
  *     across a cudaDeviceReset).  Under CUDA's lazy module loading the first

@@ -101,10 +101,28 @@ struct Layout {
     size_t qrot, cscores;   // quantized search: rotated queries, centroid scores
     size_t total;
     int64_t cap, max_tiles;
+    bool prefix;            // the ranking scratch has room for a prefix ranking
 };
 
+// Whether a search ranks a prefix of each order first: a tensor-core ranking,
+// the centroids laid out for the bulk pipeline, and a window that visits few
+// of the nprobe ranks.  any_window: whether one of its windows would.
+bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p, bool any_window = false) {
+    if (p->scan_path == 1 || !rank_tc_supported(ix->nlist, p->nprobe)) return false;
+    // past d = 256 the prefix lays the centroids out itself, which a few queries do not repay
+    if (ix->d <= 256 ? !ix->tc_centroids : nq < kPrefixMinWide) return false;
+    return (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
+           rank_prefix_len(ix->nlist, p->nprobe, any_window ? 1 : p->W, ix->d) > 0;
+}
+
+// What a layout's ranking scratch has room for: the full ranking alone (the
+// least a call takes), a prefix ranking too where the call would use one, or
+// one of any window (a calibrated search picks its window after it has its
+// workspace).
+enum class Room { kFull, kPrefix, kPrefixAnyWindow };
+
 Layout make_layout(const sieve_index_view *ix, int64_t nq, const sieve_params *p, bool host_io,
-                   bool rq = false) {
+                   Room room, bool rq = false) {
     Layout L{};
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -138,10 +156,14 @@ Layout make_layout(const sieve_index_view *ix, int64_t nq, const sieve_params *p
     L.res_cnt = take((size_t)cap * 4);
     L.res_s = take((size_t)cap * p->k * 4);
     L.res_id = take((size_t)cap * p->k * 8);
-    L.rank_scratch = (p->scan_path != 1 && rank_tc_supported(ix->nlist, p->nprobe))
-                         ? take(std::max(rank_tc_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d),
-                                         rank_prefix_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d)))
-                         : 0;
+    if (p->scan_path != 1 && rank_tc_supported(ix->nlist, p->nprobe)) {
+        const bool any = room == Room::kPrefixAnyWindow;
+        L.prefix = room != Room::kFull && !rq && use_prefix(ix, nq, p, any);
+        size_t scratch = rank_tc_scratch_bytes(nq, ix->nlist, p->nprobe, ix->d);
+        if (L.prefix)
+            scratch = std::max(scratch, rank_prefix_scratch_bytes(nq, ix->nlist, p->nprobe, any ? 0 : p->W, ix->d));
+        L.rank_scratch = take(scratch);
+    }
     if (host_io) {
         L.h_Q = take((size_t)nq * ix->d * 4);
         L.h_qids = take((size_t)nq * 8);
@@ -157,6 +179,16 @@ Layout make_layout(const sieve_index_view *ix, int64_t nq, const sieve_params *p
     }
     L.total = off;
     return L;
+}
+
+// The layout of a call with ws_bytes of scratch: with room for a prefix
+// ranking if that fits, else for the full ranking alone (a workspace sized for
+// other parameters, or the fixed array of sieve_search_noalloc).  The caller
+// compares its total with ws_bytes.
+Layout fitting_layout(const sieve_index_view *ix, int64_t nq, const sieve_params *p, bool host_io,
+                      size_t ws_bytes) {
+    const Layout L = make_layout(ix, nq, p, host_io, Room::kPrefix);
+    return L.total <= ws_bytes ? L : make_layout(ix, nq, p, host_io, Room::kFull);
 }
 
 // ---------------------------------------------------------------------------
@@ -392,15 +424,6 @@ struct RqInputs {
     const float *cscores;
 };
 
-// whether a search ranks a prefix of each order first: the centroids laid out
-// for the bulk pipeline, and a window that visits few of the nprobe ranks
-bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p) {
-    // past d = 256 the prefix lays the centroids out itself, which a few queries do not repay
-    if (ix->d <= 256 ? !ix->tc_centroids : nq < kPrefixMinWide) return false;
-    return (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
-           rank_prefix_len(ix->nlist, p->nprobe, p->W, ix->d) > 0;
-}
-
 sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t nq,
                            const int64_t *qids, const int32_t *order, const sieve_params *p,
                            int64_t *out_ids, float *out_scores, int32_t *out_count,
@@ -510,7 +533,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
     // it already), and rounds extend the orders that turn out too short; not
     // for codes, whose estimates carry the full ranking's centroid scores (a
     // given order with its scores must give the same bits)
-    const bool prefix = prefix_given || (rank_tc && !rq && use_prefix(ix, nq, p));
+    const bool prefix = prefix_given || (rank_tc && L.prefix);
     if (prefix) {
         a.limit = rank_prefix_limit(a.rank_scratch, nq, ix->nlist, p->nprobe, p->W, ix->d, &a.ext);
         a.max_rounds = (int)std::min<int64_t>(INT32_MAX, (int64_t)a.max_rounds + p->nprobe);
@@ -790,7 +813,7 @@ sieve_status sieve_search_workspace_size(const sieve_index_view *ix, int64_t nq,
     if (rc != SIEVE_OK) return rc;
     if ((rc = check_params(ix, p)) != SIEVE_OK) return rc;
     if (nq < 0 || nq > INT32_MAX / 2) return SIEVE_EINVAL;
-    *bytes = make_layout(ix, nq, p, host_io != 0).total;
+    *bytes = make_layout(ix, nq, p, host_io != 0, Room::kPrefix).total;
     return SIEVE_OK;
 }
 
@@ -806,7 +829,7 @@ sieve_status sieve_search(const sieve_index_view *ix, const float *Q, int64_t nq
     if ((rc = check_device()) != SIEVE_OK) return rc;
     if (stats) std::memset(stats, 0, sizeof(*stats));
     if (nq == 0) return SIEVE_OK;
-    const Layout L = make_layout(ix, nq, p, false);
+    const Layout L = order ? make_layout(ix, nq, p, false, Room::kFull) : fitting_layout(ix, nq, p, false, ws_bytes);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total)
         return SIEVE_EWORKSPACE;
     return search_device(ix, Q, nq, query_ids, order, p, out_ids, out_scores, out_count,
@@ -892,7 +915,7 @@ sieve_status sieve_rq_search_workspace_size(const sieve_index_view *ix, int64_t 
     if (rc != SIEVE_OK) return rc;
     if ((rc = check_params(ix, p)) != SIEVE_OK) return rc;
     if (nq < 0 || nq > INT32_MAX / 2) return SIEVE_EINVAL;
-    *bytes = make_layout(ix, nq, p, false, true).total;
+    *bytes = make_layout(ix, nq, p, false, Room::kFull, true).total;
     return SIEVE_OK;
 }
 
@@ -915,7 +938,7 @@ sieve_status sieve_rq_search(const sieve_index_view *ix, const sieve_rq_view *rq
     if ((rc = check_device()) != SIEVE_OK) return rc;
     if (stats) std::memset(stats, 0, sizeof(*stats));
     if (nq == 0) return SIEVE_OK;
-    const Layout L = make_layout(ix, nq, p, false, true);
+    const Layout L = make_layout(ix, nq, p, false, Room::kFull, true);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total)
         return SIEVE_EWORKSPACE;
     const RqInputs in{rq, order ? cscores : nullptr};
@@ -936,7 +959,7 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
     if ((rc = check_device()) != SIEVE_OK) return rc;
     if (stats) std::memset(stats, 0, sizeof(*stats));
     if (nq == 0) return SIEVE_OK;
-    const Layout L = make_layout(ix, nq, p, true);
+    const Layout L = fitting_layout(ix, nq, p, true, ws_bytes);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total)
         return SIEVE_EWORKSPACE;
     unsigned char *w = static_cast<unsigned char *>(ws);
@@ -960,7 +983,7 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
     const int64_t chunk = round_up(ceil_div(nq, kHostChunks), wave);
     const int nchunks = p->profile ? 0 : (int)std::min<int64_t>(kHostChunks, ceil_div(nq, chunk));
     const bool rank_tc = p->scan_path != 1 && L.rank_scratch != 0;
-    const bool prefix = rank_tc && nchunks > 0 && use_prefix(ix, nq, p);
+    const bool prefix = rank_tc && nchunks > 0 && L.prefix;
     SIEVE_CUDA(rank_tc ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
     if (prefix) SIEVE_CUDA(prepare_rank_prefix(ix->nlist, p->nprobe, p->W, ix->d));
     SIEVE_CUDA(cudaMemsetAsync(dstatus, 0, sizeof(int), st));
@@ -1039,12 +1062,12 @@ struct CalibLayout {
 };
 
 static CalibLayout make_calib_layout(const sieve_index_view *ix, int64_t nq, int64_t ns,
-                                     const sieve_params *p) {
+                                     const sieve_params *p, Room room) {
     CalibLayout C{};
     sieve_params wide = *p;
     wide.W = p->nprobe;
     const int64_t nr = nq - ns;
-    const Layout a = make_layout(ix, ns, &wide, false), b = make_layout(ix, nr, &wide, false);
+    const Layout a = make_layout(ix, ns, &wide, false, room), b = make_layout(ix, nr, &wide, false, room);
     C.inner = a.total >= b.total ? a : b;
     size_t off = C.inner.total;
     auto take = [&](size_t bytes) {
@@ -1085,8 +1108,8 @@ sieve_status sieve_calibrated_search_workspace_size(const sieve_index_view *ix, 
     if (rc != SIEVE_OK) return rc;
     if ((rc = check_params(ix, p)) != SIEVE_OK) return rc;
     if (nq < 0 || nq > INT32_MAX / 2 || ns < 0 || ns > nq) return SIEVE_EINVAL;
-    const Layout plain = make_layout(ix, nq, p, false);
-    *bytes = std::max(plain.total, make_calib_layout(ix, nq, ns, p).total);
+    const Layout plain = make_layout(ix, nq, p, false, Room::kPrefixAnyWindow);
+    *bytes = std::max(plain.total, make_calib_layout(ix, nq, ns, p, Room::kPrefixAnyWindow).total);
     return SIEVE_OK;
 }
 
@@ -1116,13 +1139,14 @@ sieve_status sieve_calibrated_search(const sieve_index_view *ix, const float *Q,
         *W_out = fallback_W;
         sieve_params q = *p;
         q.W = fallback_W;
-        const Layout L = make_layout(ix, nq, &q, false);
+        const Layout L = fitting_layout(ix, nq, &q, false, ws_bytes);
         if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total)
             return SIEVE_EWORKSPACE;
         return search_device(ix, Q, nq, query_ids, nullptr, &q, out_ids, out_scores, out_count,
                              out_probes, nullptr, w, L, st);
     }
-    const CalibLayout C = make_calib_layout(ix, nq, ns, p);
+    CalibLayout C = make_calib_layout(ix, nq, ns, p, Room::kPrefixAnyWindow);
+    if (C.total > ws_bytes) C = make_calib_layout(ix, nq, ns, p, Room::kFull);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < C.total)
         return SIEVE_EWORKSPACE;
     const int k = p->k, d = ix->d;
@@ -1137,7 +1161,7 @@ sieve_status sieve_calibrated_search(const sieve_index_view *ix, const float *Q,
     sieve_params full = *p;
     full.W = p->nprobe;
     SearchExtras ex{I32(C.s_rank), reinterpret_cast<uint32_t *>(w + C.s_hits)};
-    const Layout Ls = make_layout(ix, ns, &full, false);
+    const Layout Ls = fitting_layout(ix, ns, &full, false, C.inner.total);
     rc = search_device(ix, F(C.Qs), ns, query_ids ? I64(C.qs) : nullptr, nullptr, &full,
                        I64(C.s_ids), F(C.s_sc), I32(C.s_cnt), I32(C.s_pr), nullptr, w, Ls, st, &ex);
     if (rc != SIEVE_OK) return rc;
@@ -1162,7 +1186,7 @@ sieve_status sieve_calibrated_search(const sieve_index_view *ix, const float *Q,
         SIEVE_CUDA(calib_gather(Q, query_ids, d, I64(C.rest), nr, F(C.Qr), I64(C.qr), st));
         sieve_params rest = *p;
         rest.W = w_star;
-        const Layout Lr = make_layout(ix, nr, &rest, false);
+        const Layout Lr = fitting_layout(ix, nr, &rest, false, C.inner.total);
         rc = search_device(ix, F(C.Qr), nr, query_ids ? I64(C.qr) : nullptr, nullptr, &rest,
                            I64(C.r_ids), F(C.r_sc), I32(C.r_cnt), I32(C.r_pr), nullptr, w, Lr, st);
         if (rc != SIEVE_OK) return rc;
@@ -1193,12 +1217,12 @@ static sieve_status shard_params(const sieve_params *p, const int32_t *W_per_sha
 }
 
 static ShardLayout make_shard_layout(const sieve_index_view *shards, int nshards, int64_t nq,
-                                     const sieve_params *p, const int32_t *W_per_shard) {
+                                     const sieve_params *p, const int32_t *W_per_shard, Room room) {
     ShardLayout S{};
     for (int s = 0; s < nshards; ++s) {
         sieve_params ps;
         shard_params(p, W_per_shard, s, &ps);
-        const Layout L = make_layout(&shards[s], nq, &ps, false);
+        const Layout L = make_layout(&shards[s], nq, &ps, false, room);
         if (L.total > S.inner.total) S.inner = L;
     }
     size_t off = S.inner.total;
@@ -1236,7 +1260,7 @@ sieve_status sieve_sharded_search_workspace_size(const sieve_index_view *shards,
     sieve_status rc = check_shards(shards, nshards, p, W_per_shard);
     if (rc != SIEVE_OK) return rc;
     if (nq < 0 || nq > INT32_MAX / 2) return SIEVE_EINVAL;
-    *bytes = make_shard_layout(shards, nshards, nq, p, W_per_shard).total;
+    *bytes = make_shard_layout(shards, nshards, nq, p, W_per_shard, Room::kPrefix).total;
     return SIEVE_OK;
 }
 
@@ -1254,7 +1278,8 @@ sieve_status sieve_sharded_search(const sieve_index_view *shards, int32_t nshard
     if (p->profile || (nq > 0 && !aligned16(Q))) return SIEVE_EINVAL;
     if ((rc = check_device()) != SIEVE_OK) return rc;
     if (nq == 0) return SIEVE_OK;
-    const ShardLayout S = make_shard_layout(shards, nshards, nq, p, W_per_shard);
+    ShardLayout S = make_shard_layout(shards, nshards, nq, p, W_per_shard, Room::kPrefix);
+    if (S.total > ws_bytes) S = make_shard_layout(shards, nshards, nq, p, W_per_shard, Room::kFull);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < S.total)
         return SIEVE_EWORKSPACE;
     unsigned char *w = static_cast<unsigned char *>(ws);
@@ -1267,7 +1292,7 @@ sieve_status sieve_sharded_search(const sieve_index_view *shards, int32_t nshard
     for (int s = 0; s < nshards; ++s) {   // each shard ranks and stops on its own
         sieve_params ps;
         shard_params(p, W_per_shard, s, &ps);
-        const Layout L = make_layout(&shards[s], nq, &ps, false);
+        const Layout L = fitting_layout(&shards[s], nq, &ps, false, S.inner.total);
         rc = search_device(&shards[s], Q, nq, query_ids, nullptr, &ps, ids + (int64_t)s * nq * k,
                            sc + (int64_t)s * nq * k, cnt + (int64_t)s * nq, pr + (int64_t)s * nq,
                            nullptr, w, L, st);
@@ -1342,7 +1367,8 @@ extern "C" sieve_status sieve_search_noalloc(const sieve_index_view *ix, const f
     if ((rc = check_device()) != SIEVE_OK) return rc;
     if (stats) std::memset(stats, 0, sizeof(*stats));
     if (nq == 0) return SIEVE_OK;
-    const Layout L = make_layout(ix, nq, p, false);
+    const Layout L = order ? make_layout(ix, nq, p, false, Room::kFull)
+                           : fitting_layout(ix, nq, p, false, kNoallocScratchBytes);
     if (L.total > kNoallocScratchBytes) return SIEVE_ESCRATCH;
     void *ws = nullptr;
     if ((rc = noalloc_scratch(&ws)) != SIEVE_OK) return rc;

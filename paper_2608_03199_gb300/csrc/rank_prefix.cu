@@ -621,11 +621,11 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
     return S;
 }
 
-// for any window: a calibrated search sizes its workspace before it picks one
-size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int d) {
+// W = 0: for any window
+size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int W, int d) {
     int64_t b = 0;
     for (int L : {16, 32})
-        if (nq > 0 && prefix_fits(nlist, nprobe, d, L))
+        if (nq > 0 && (W == 0 ? prefix_fits(nlist, nprobe, d, L) : rank_prefix_len(nlist, nprobe, W, d) == L))
             b = std::max(b, prefix_scratch(nq, nlist, nprobe, d, L).total);
     return (size_t)b;
 }

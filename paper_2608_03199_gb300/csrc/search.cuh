@@ -155,7 +155,7 @@ int rank_bulk_stages(int d);                     // 0 when the bulk ranking does
 // (rank_prefix.cu): entries kept per query list, 0 when it does not apply; the
 // scratch (the limits and the extension list first, for the whole search)
 int rank_prefix_len(int64_t nlist, int nprobe, int W, int d);
-size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int d);   // for any W
+size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int W, int d);   // W = 0: any window
 int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext);
 cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d);
 int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma);

@@ -110,3 +110,29 @@ def test_screen_scores_rejects_bad_arguments_without_gpu():
     assert lib.sieve_screen_scores(ctypes.byref(v), q, -1, out, 128, None) == -1   # nq < 0
     assert lib.sieve_screen_scores(ctypes.byref(v), ctypes.c_void_p(260), 10, out, 128, None) == -1
     assert lib.sieve_screen_scores(ctypes.byref(v), q, 10, None, 128, None) == -1
+
+
+def test_workspace_has_prefix_lists_only_where_a_search_uses_them_without_gpu():
+    """A search's workspace is that of the FP32 path plus the full ranking's
+    scratch, unless the call ranks a prefix of each order (a layout of the
+    centroids, a window of up to 24, and 2,048 centroids or 4,096 queries)."""
+    lib = sieve.lib()
+
+    def size(nlist, d, nq, nprobe, W, path="auto", layout=True):
+        v = sieve.IndexViewC(n=1000, nlist=nlist, d=d, vectors=16, ids=16, list_offsets=16, centroids=16)
+        if layout:
+            v.tc_rows = v.tc_row_blocks = v.tc_centroids = 256
+        p = sieve._params(0.9, 10, nprobe, W, True, 0, 0, 0, path)
+        total, rank = ctypes.c_size_t(), ctypes.c_size_t()
+        assert lib.sieve_search_workspace_size(ctypes.byref(v), nq, ctypes.byref(p), 0, ctypes.byref(total)) == 0
+        assert lib.sieve_rank_workspace_size(ctypes.byref(v), nq, nprobe, ctypes.byref(rank)) == 0
+        return total.value, rank.value
+
+    for nlist, d, nq, nprobe, W, layout in ((1024, 256, 2_000, 64, 8, True), (149, 100, 4_000, 24, 4, True),
+                                            (1024, 256, 20_000, 64, 64, True), (8192, 96, 20_000, 128, 8, False),
+                                            (8192, 512, 200, 128, 8, False)):
+        total, rank = size(nlist, d, nq, nprobe, W, layout=layout)
+        assert total <= size(nlist, d, nq, nprobe, W, "simt", layout)[0] + rank + 512, (nlist, d, nq, nprobe, W)
+    # where it is used, the lists and the extension's buffers come on top
+    total, rank = size(8192, 96, 2_000, 128, 8)
+    assert total > size(8192, 96, 2_000, 128, 8, "simt")[0] + rank + 512

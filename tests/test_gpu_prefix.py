@@ -109,3 +109,58 @@ def test_nan_centroid_is_ranked_as_by_the_full_order(dev):
     got = sieve.search(ix, Q, 0.5, 10, 64, 8, query_ids=qids, check=True)
     for x, y in zip(got, want):
         assert torch.equal(x, y)
+
+
+class _Fixed:
+    """A workspace of a given size, whatever a call asks for."""
+
+    def __init__(self, nbytes, device):
+        self.buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
+
+    def get(self, nbytes, device):
+        return self.buf
+
+
+@pytest.mark.parametrize("call", ["search", "host", "sharded", "calibrated"])
+def test_workspace_without_room_for_the_lists(dev, call):
+    """A workspace of the full ranking's size (what the same index without the
+    centroids' layout asks for) is taken, and the orders are ranked whole; half
+    of it is refused, as ever."""
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 12_000, 96, 2_309, seed=6)
+    nq, k, nprobe, W = 2_000, 10, 64, 8
+    Q, qids = X[:nq].contiguous(), torch.arange(nq)
+    Qd, qd = Q.to(dev), qids.to(dev)
+    sample = torch.arange(0, nq, 10, device=dev)
+    asked = []
+
+    class Asks(sieve.Workspace):
+        def get(self, nbytes, device):
+            asked.append(nbytes)
+            return super().get(nbytes, device)
+
+    def run(index, ws):
+        if call == "search":
+            return sieve.search(index, Qd, 0.9, k, nprobe, W, query_ids=qd, workspace=ws, check=True)
+        if call == "host":
+            return sieve.search_host(index, Q.pin_memory(), 0.9, k, nprobe, W,
+                                     query_ids_host=qids.pin_memory(), workspace=ws)
+        if call == "sharded":
+            return sieve.sharded_search([index], Qd, 0.9, k, nprobe, W, query_ids=qd, workspace=ws)
+        return sieve.calibrated_search(index, Qd, 0.9, k, nprobe, sample, 0.1, min_queries=1,
+                                       query_ids=qd, workspace=ws)[:4]
+
+    want = [x.cpu() for x in run(ix, Asks())]
+    bare = sieve.Index(ix.vectors, ix.ids, ix.list_offsets, ix.centroids, ix.tc_rows, ix.tc_row_blocks, None)
+    bare.view = lambda v=bare.without_tc_layout().view(): v
+    run(bare, Asks())
+    full, least = asked
+    assert least < full
+    got = [x.cpu() for x in run(ix, _Fixed(least, dev))]
+    for x, y in zip(got, want):
+        # near-ties of centroids and of the two scan paths' sums apart
+        same = (x == y) if x.dtype != torch.float32 else ((x - y).abs() <= 1e-5) | (x == y)
+        assert (~same).reshape(nq, -1).any(1).sum() <= 2
+    with pytest.raises(sieve.SieveError) as e:
+        run(ix, _Fixed(least // 2, dev))
+    assert e.value.status == -3

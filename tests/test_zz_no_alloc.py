@@ -83,6 +83,31 @@ def test_noalloc_refuses_calls_beyond_its_scratch(setup):
     assert sieve.lib().sieve_status_str(rc).startswith(b"call needs more scratch")
 
 
+@pytest.mark.parametrize("nlist,d,nprobe,W,nq", [(1_024, 256, 64, 8, 12_000), (149, 100, 24, 4, 38_700),
+                                                 (1_500, 96, 90, 8, 8_690), (1_024, 256, 64, 64, 4_980)])
+def test_noalloc_takes_what_fits_a_whole_ranking(setup, nlist, d, nprobe, W, nq):
+    """The lists of a prefix ranking are no reason to refuse a call: these
+    batches fill the array to its last parts with the full ranking alone."""
+    dev = setup[3]
+    g = torch.Generator().manual_seed(nlist)
+    X = torch.randn(4 * nlist, d, generator=g)
+    X = (X / X.norm(dim=1, keepdim=True)).to(dev)
+    C0 = X[:nlist].contiguous()
+    index = sieve.build_layout(X, (X @ C0.T).argmax(1).int(), nlist, C0)
+    Q = X[torch.randint(0, 4 * nlist, (nq,), generator=g).to(dev)]
+    qids = torch.full((nq,), -1, dtype=torch.int64, device=dev)
+    outs = (torch.empty((nq, 10), dtype=torch.int64, device=dev),
+            torch.empty((nq, 10), dtype=torch.float32, device=dev),
+            torch.empty(nq, dtype=torch.int32, device=dev),
+            torch.empty(nq, dtype=torch.int32, device=dev))
+    rc, _ = _noalloc(index, Q, qids, 0.90, 10, nprobe, W, True, outs)
+    assert rc == 0, sieve.lib().sieve_status_str(rc)
+    order = sieve.rank_partitions(index, Q, nprobe)
+    ref = sieve.search(index, Q, 0.90, 10, nprobe, W, query_ids=qids, order=order, check=True)
+    for x, y in zip(outs, ref):
+        assert torch.equal(x, y)
+
+
 def test_noalloc_takes_no_device_memory(setup):
     """A repeated call (its kernels already loaded by the first) leaves the
     device's free memory where it was: the scratch is the fixed array."""
