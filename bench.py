@@ -227,12 +227,8 @@ def roofline(prof, cfg, dev, bulk=True, rank_on_tensor=True, rq=False, screen=Fa
     km, kl = dict(prof["kernel_ms"]), dict(prof["kernel_launches"])
     # the ranking's contraction is timed on its own ("rank_mma", a part of
     # "rank"); the rest of "rank" is its selection
-    prefix = False
+    prefix = prof["extended"] >= 0   # a prefix ranking, and so many queries ranked whole after it
     if km.get("rank_mma", 0) > 0:
-        # a prefix ranking: a scan and a final per chunk, once the largest norm
-        # (and, past d = 256, the layout); a full one of as many centroids takes
-        # five launches a chunk, two of them contractions
-        prefix = cfg.nlist > 2048 and kl["rank"] - 2 * kl["rank_mma"] in (1, 2)
         km["rank_select"] = km["rank"] - km["rank_mma"]
         kl["rank_select"] = kl["rank"] - kl["rank_mma"]
         del km["rank"], kl["rank"]
@@ -291,16 +287,19 @@ def roofline(prof, cfg, dev, bulk=True, rank_on_tensor=True, rq=False, screen=Fa
                    hbm_view={"achieved_gbs": bytes_ / launches / (ms_per_launch * 1e-3) / 1e9,
                              "peak_gbs": hbm})
     elif top == "rank_mma" and prefix:
-        # the screen over all centroids, one product per score (and an eighth
-        # of them twice, for the sample)
+        # the screen over all centroids, one product per score, and the full
+        # ranking's two passes for the extended queries; the sample, an eighth of
+        # a long range's chunks screened twice, is not counted
+        first_products = rank_passes(cfg, bulk)[1]
+        products = 1 + (3 + first_products) * prof["extended"] / cfg.nq
         ach = 2.0 * cfg.nq * cfg.nlist * d / launches / (ms_per_launch * 1e-3) / 1e12
         d_mma = 16 * -(-d // 16)
         out.update(kernel="k_prefix_scan", bound="tensor", achieved=ach, peak=f16_tflops,
                    unit="TFLOP/s", frac=ach / f16_tflops,
                    peak_source=(f"one kind::f16 MMA per score; fp16 dense peak {f16_tflops:.0f} "
                                 f"TFLOP/s = measured bf16 cuBLAS burst (of measured); achieved = "
-                                f"every score once"),
-                   passes=1, tensor_pipe_tflops=1.125 * ach * d_mma / d,
+                                f"every score once over the summed time of all contraction launches"),
+                   passes=1, extended=prof["extended"], tensor_pipe_tflops=products * ach * d_mma / d,
                    rank_select_ms=km.get("rank_select"))
     elif top == "rank_mma":
         # the score contraction of the ranking (tensor cores, three fp16
@@ -717,7 +716,8 @@ def run_sieve(args, cfg, world, rank, local):
                              rank_on_tensor=args.scan_path != "simt",
                              screen=uses_screen(args, cfg, cfg.W, index.tc_rows is not None)),
         "profile": {"kernel_ms": prof["kernel_ms"], "kernel_launches": prof["kernel_launches"],
-                    "rounds": prof["rounds"], "items": prof["items"], "groups": prof["groups"],
+                    "rounds": prof["rounds"], "extended": prof["extended"],
+                    "items": prof["items"], "groups": prof["groups"],
                     "mean_group": prof["items"] / max(1, prof["groups"]),
                     "pairs": prof["pairs"], "rows_read": prof["rows_read"],
                     "pairs_tc": prof["pairs_tc"], "rows_read_tc": prof["rows_read_tc"]},

@@ -180,7 +180,12 @@ enum {
  *   rows_read    partition rows streamed by the scan (one read per tile)
  *   pairs        query-row similarities computed
  *   rows_read_tc, pairs_tc  the part of rows_read / pairs done on the tensor cores
- *   status       device status word (0, or a SIEVE_E* code) */
+ *   status       device status word (0, or a SIEVE_E* code)
+ *   extended     -1: every order was ranked whole, or was given; else the call
+ *                ranked the first centroids of each order (a small window),
+ *                and this many queries went past them and were ranked whole
+ *                as well (the launches and time of both are SIEVE_K_RANK's and
+ *                SIEVE_K_RANK_MMA's) */
 typedef struct {
     int64_t rounds;
     int64_t items;
@@ -191,7 +196,7 @@ typedef struct {
     int64_t rows_read_tc;
     int64_t pairs_tc;
     int32_t status;
-    int32_t reserved0;
+    int32_t extended;
     float kernel_ms[SIEVE_NKERNELS];          /* profile = 1: summed launch durations */
     int32_t kernel_launches[SIEVE_NKERNELS];  /* launches per kernel in the call */
 } sieve_stats;

@@ -59,7 +59,7 @@ class StatsC(C.Structure):
     _fields_ = [("rounds", C.c_int64), ("items", C.c_int64), ("groups", C.c_int64),
                 ("tiles", C.c_int64), ("rows_read", C.c_int64), ("pairs", C.c_int64),
                 ("rows_read_tc", C.c_int64), ("pairs_tc", C.c_int64),
-                ("status", C.c_int32), ("reserved0", C.c_int32),
+                ("status", C.c_int32), ("extended", C.c_int32),
                 ("kernel_ms", C.c_float * 12), ("kernel_launches", C.c_int32 * 12)]
 
 

@@ -233,9 +233,9 @@ cudaError_t launch_search_rank(const SearchArgs &a, int rank_tc, cudaStream_t st
 }
 
 // the end of a round that met queries whose stop line passes their prefix
-cudaError_t launch_search_ext(const SearchArgs &a, int part, cudaStream_t st) {
+cudaError_t launch_search_ext(const SearchArgs &a, int part, cudaStream_t st, float *mma_ms = nullptr) {
     return enqueue_rank_ext(part, a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, const_cast<int32_t *>(a.order),
-                            a.cscores, a.rank_scratch, &a.ctl->ext_n, &a.ctl->status, a.tc_cent, st);
+                            a.cscores, a.rank_scratch, &a.ctl->ext_n, &a.ctl->status, a.tc_cent, st, mma_ms);
 }
 
 // quantized search: q' = P^T q for the batch, after init (which clears the
@@ -612,7 +612,9 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
             }
             if (!more) break;
             for (int i = 0; prefix && i < 2 && word[2] > (i ? kExtFirst : 0); ++i)
-                SIEVE_CUDA(timed(SIEVE_K_RANK, [&] { return launch_search_ext(a, i, st); }));
+                SIEVE_CUDA(timed(SIEVE_K_RANK, [&] {
+                    return launch_search_ext(a, i, st, p->profile ? &ms[SIEVE_K_RANK_MMA] : nullptr);
+                }));
         }
         SIEVE_CUDA(timed(SIEVE_K_FINALIZE, [&] { return launch_finalize(a, st); }));
     }
@@ -629,19 +631,24 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         stats->rows_read_tc = (int64_t)c.tot_rows_tc;
         stats->pairs_tc = (int64_t)c.tot_pairs_tc;
         stats->status = c.status;
-        stats->reserved0 = 0;
+        stats->extended = prefix ? (int32_t)c.tot_ext : -1;
         for (int i = 0; i < SIEVE_NKERNELS; ++i) stats->kernel_ms[i] = ms[i];
         const int per_round[] = {SIEVE_K_ISSUE, SIEVE_K_BUCKET, SIEVE_K_SCATTER, SIEVE_K_SCAN,
                                  SIEVE_K_MERGE, SIEVE_K_ROUND_END};
-        int prefix_mma = 0;
-        const int prefix_launches =
-            prefix && with_rank
-                ? rank_prefix_launches(a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma) : 0;
+        const bool bulk = a.tc_cent && rank_bulk_stages(a.d) > 0;
+        int prefix_mma = 0, prefix_launches = 0;   // the prefix ranking, if it ran here, and its extensions
+        if (prefix && with_rank)
+            prefix_launches = rank_prefix_launches(a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma);
+        for (int i = 0; prefix && i < 2; ++i)
+            if (c.ext_runs[i] > 0) {
+                int mma = 0;
+                prefix_launches += c.ext_runs[i] * rank_ext_launches(i, a.nq, a.nlist, a.nprobe, a.W, a.d, bulk, &mma);
+                prefix_mma += c.ext_runs[i] * mma;
+            }
         stats->kernel_launches[SIEVE_K_RANK] =
-            !with_rank ? 0
-            : prefix   ? prefix_launches
-            : rank_tc ? rank_tc_launches(a.nq, a.nlist, a.nprobe, a.d, 0,
-                                         a.tc_cent && rank_bulk_stages(a.d) > 0)
+            prefix       ? prefix_launches
+            : !with_rank ? 0
+            : rank_tc ? rank_tc_launches(a.nq, a.nlist, a.nprobe, a.d, 0, bulk)
                       : 1;
         stats->kernel_launches[SIEVE_K_INIT] = a.tc_screen ? 2 : 1;   // + the query norms
         stats->kernel_launches[SIEVE_K_FINALIZE] = 1;
@@ -649,9 +656,8 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         stats->kernel_launches[SIEVE_K_SCAN_TC] = a.tc_min > 0 ? c.round : 0;
         stats->kernel_launches[SIEVE_K_RQ_ROTATE] = a.rq ? 1 : 0;
         stats->kernel_launches[SIEVE_K_RANK_MMA] =
-            prefix && with_rank ? prefix_mma
-            : with_rank && rank_tc ? rank_tc_mma_launches(a.nq, a.nlist, a.nprobe, a.d, 0,
-                                                         a.tc_cent && rank_bulk_stages(a.d) > 0)
+            prefix ? prefix_mma
+            : with_rank && rank_tc ? rank_tc_mma_launches(a.nq, a.nlist, a.nprobe, a.d, 0, bulk)
                                   : 0;
         if (a.tc_min == 1) stats->kernel_launches[SIEVE_K_SCAN] = 0;
         if (c.status != 0) return c.status;
@@ -1044,8 +1050,8 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
                                sizeof(int), cudaMemcpyDeviceToHost, st));
     SIEVE_CUDA(cudaStreamSynchronize(st));
     if (stats && nchunks > 0) {   // ran here
-        stats->kernel_launches[SIEVE_K_RANK] = rank_launches;
-        stats->kernel_launches[SIEVE_K_RANK_MMA] = mma_launches;
+        stats->kernel_launches[SIEVE_K_RANK] += rank_launches;   // to the extensions of a prefix ranking
+        stats->kernel_launches[SIEVE_K_RANK_MMA] += mma_launches;
     }
     return rank_status != 0 ? rank_status : search_status != 0 ? search_status : SIEVE_OK;
 }

@@ -36,9 +36,11 @@ struct Ctl {
     int n_ext;         // the same, counted while the round issues
     int n_tc_tiles;    // tensor-core scan tiles this round
     int tc_tile_next;  // tensor-core scan work counter
-    int pad[3];
+    int ext_runs[2];   // rounds that ended with the extension's first part, and with its second
+    int pad;
     unsigned long long tot_items, tot_groups, tot_tiles, tot_rows, tot_pairs;
     unsigned long long tot_rows_tc, tot_pairs_tc;   // the tensor-core share of the two above
+    unsigned long long tot_ext;                     // queries extended
 };
 
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

@@ -755,7 +755,8 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
 // Every pass is launched; passes past *ext_n find no work.
 cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                              int nprobe, int W, int32_t *order, float *cscores, void *scratch,
-                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st) {
+                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st,
+                             float *mma_ms) {
     const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
     const PrefixScratch::Ext &E = S.ext_part[part];
     unsigned char *w = static_cast<unsigned char *>(scratch);
@@ -770,13 +771,26 @@ cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *
         const int64_t n = std::min(E.chunk, hi - b);
         k_ext_gather<<<blocks, 256, 0, st>>>(Q, d, ext, ext_n, b, n, Qx);
         cudaError_t e = enqueue_rank_tc(Qx, n, C, nlist, d, nprobe, full, full_s,
-                                        reinterpret_cast<float *>(w + S.rest), status, st, tc_cent, nullptr,
+                                        reinterpret_cast<float *>(w + S.rest), status, st, tc_cent, mma_ms,
                                         E.chunk, ext_n, b);
         if (e != cudaSuccess) return e;
         k_ext_merge<<<blocks, 256, 0, st>>>(ext, ext_n, b, n, nprobe, full, full_s, order, cscores, limit);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+int rank_ext_launches(int part, int64_t nq, int64_t nlist, int nprobe, int W, int d, bool bulk, int *mma) {
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    const int64_t chunk = S.ext_part[part].chunk;
+    int n = 0;
+    *mma = 0;
+    for (int64_t b = part ? kExtFirst : 0, hi = part ? nq : std::min(nq, kExtFirst); b < hi; b += chunk) {
+        const int64_t m = std::min(chunk, hi - b);
+        n += 2 + rank_tc_launches(m, nlist, nprobe, d, chunk, bulk);
+        *mma += rank_tc_mma_launches(m, nlist, nprobe, d, chunk, bulk);
+    }
+    return n;
 }
 
 }  // namespace sieve

@@ -171,7 +171,10 @@ constexpr int64_t kExtFirst = 4096;
 cudaError_t launch_ext_more(const SearchArgs &a, cudaGraphConditionalHandle cond, cudaStream_t st);
 cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                              int nprobe, int W, int32_t *order, float *cscores, void *scratch,
-                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st);
+                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st,
+                             float *mma_ms = nullptr);
+// kernel launches of one run of a part (and its contraction launches)
+int rank_ext_launches(int part, int64_t nq, int64_t nlist, int nprobe, int W, int d, bool bulk, int *mma);
 
 // in-call window calibration (calibrate.cu)
 cudaError_t calib_gather(const float *Q, const int64_t *qids, int d, const int64_t *idx, int64_t n,

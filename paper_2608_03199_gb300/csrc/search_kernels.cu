@@ -577,6 +577,9 @@ __global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
     c->more = more;
     c->ext_n = more ? c->n_ext : 0;
     c->n_ext = 0;
+    c->tot_ext += (unsigned long long)c->ext_n;
+    c->ext_runs[0] += c->ext_n > 0;
+    c->ext_runs[1] += c->ext_n > kExtFirst;
     c->n_items = 0;
     c->n_active = 0;
     c->n_tiles = 0;

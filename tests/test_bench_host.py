@@ -86,3 +86,23 @@ def test_parity_sample_counts_divergences():
     got[0][b, 0] = 10**9
     rep = bench.parity_sample(oracle, idx, w["Q"], w["qids"], cfg, cfg.W, ref, tuple(got))
     assert rep["exact"] == rep["queries"] - 2 and rep["unexplained"] == 2
+
+
+def test_roofline_names_the_ranking_that_ran(monkeypatch):
+    """Launch counts do not tell a full ranking in one chunk (six launches, two
+    of them contractions) from a prefix ranking: the library's count of
+    extended queries does (-1: every order was ranked whole)."""
+    monkeypatch.setattr(torch.cuda, "get_device_properties",
+                        lambda dev: types.SimpleNamespace(multi_processor_count=152))
+    cfg = types.SimpleNamespace(name="10m", nq=1_000_000, nlist=8192, d=256, nprobe=128)
+    prof = {"kernel_ms": {"rank": 20.0, "rank_mma": 15.0, "scan_tc": 1.0},
+            "kernel_launches": {"rank": 6, "rank_mma": 2, "scan_tc": 3}}
+    full = bench.roofline({**prof, "extended": -1}, cfg, None)
+    assert full["kernel"] == "k_rank_bulk + k_rank_screen" and full["passes"] == 2
+    prefix = bench.roofline({**prof, "extended": 0}, cfg, None)
+    assert prefix["kernel"] == "k_prefix_scan" and prefix["passes"] == 1
+    assert abs(prefix["tensor_pipe_tflops"] - prefix["achieved"]) < 1e-9
+    assert abs(prefix["frac"] * 3 - full["frac"]) < 1e-9
+    # a tenth of the queries extended: 0.4 products more per score
+    some = bench.roofline({**prof, "extended": 100_000}, cfg, None)
+    assert abs(some["tensor_pipe_tflops"] - 1.4 * some["achieved"]) < 1e-9

@@ -164,3 +164,27 @@ def test_workspace_without_room_for_the_lists(dev, call):
     with pytest.raises(sieve.SieveError) as e:
         run(ix, _Fixed(least // 2, dev))
     assert e.value.status == -3
+
+
+@pytest.mark.parametrize("nq", [200, 9_001])
+def test_stats_tell_which_ranking_ran(dev, nq):
+    """extended: -1 where every order is ranked whole or given, else the queries
+    ranked whole after their prefix, whose launches count as the ranking's."""
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 12_000, 64, 2_500, seed=2)
+    Q, qids = X[:nq].to(dev), torch.arange(nq, device=dev)
+    run = lambda tau, W, **kw: sieve.search(ix, Q, tau, 10, 64, W, query_ids=qids, stats=True, **kw)[4]
+    assert run(0.9, 8, order=sieve.rank_partitions(ix, Q, 64))["extended"] == -1
+    assert run(0.9, 64)["extended"] == -1
+    assert run(0.9, 8, scan_path="simt")["extended"] == -1
+    none = run(0.999, 8)
+    assert none["extended"] == 0
+    assert none["kernel_launches"]["rank"] == 3 and none["kernel_launches"]["rank_mma"] == 1
+    for loop in (0, 1):
+        some = run(0.2, 8, loop=loop)
+        assert nq // 2 < some["extended"] <= nq
+        # a part of an extension is a gather, a full ranking and a merge
+        assert some["kernel_launches"]["rank"] >= 3 + 8 and some["kernel_launches"]["rank_mma"] >= 1 + 2
+    prof = sieve.search(ix, Q, 0.2, 10, 64, 8, query_ids=qids, profile=True)[4]
+    assert prof["kernel_launches"]["rank_mma"] == some["kernel_launches"]["rank_mma"]
+    assert prof["kernel_ms"]["rank"] > prof["kernel_ms"]["rank_mma"] > 0
