@@ -33,7 +33,7 @@ struct Ctl {
     int status;        // 0 or a SIEVE_E* code
     int more;          // 1 while another round is needed
     int ext_n;         // queries whose ranking the end of this round extends
-    int n_ext;         // the same, counted while the round issues
+    int n_ext;         // the same, counted while the round issues and merges
     int n_tc_tiles;    // tensor-core scan tiles this round
     int tc_tile_next;  // tensor-core scan work counter
     int ext_runs[2];   // rounds that ended with the extension's first part, and with its second

@@ -188,3 +188,20 @@ def test_stats_tell_which_ranking_ran(dev, nq):
     prof = sieve.search(ix, Q, 0.2, 10, 64, 8, query_ids=qids, profile=True)[4]
     assert prof["kernel_launches"]["rank_mma"] == some["kernel_launches"]["rank_mma"]
     assert prof["kernel_ms"]["rank"] > prof["kernel_ms"]["rank_mma"] > 0
+
+
+@pytest.mark.parametrize("lookahead", [True, False])
+@pytest.mark.parametrize("nq,d,nlist,W", [(300, 64, 2_500, 8), (9_001, 96, 2_309, 8), (1_000, 128, 2_100, 16)])
+def test_an_extension_takes_no_round_of_its_own(dev, lookahead, nq, d, nlist, W):
+    """A query is listed in the round that raises its stop line, so the rounds
+    are those of the same search on the whole order."""
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 12_000, d, nlist, seed=8)
+    Q, qids = X[:nq].to(dev), torch.arange(nq, device=dev)
+    kw = dict(lookahead=lookahead, query_ids=qids, stats=True)
+    want = sieve.search(ix, Q, 0.3, 10, 64, W, order=sieve.rank_partitions(ix, Q, 64), **kw)
+    for loop in (0, 1):
+        got = sieve.search(ix, Q, 0.3, 10, 64, W, loop=loop, **kw)
+        assert got[4]["extended"] > 0
+        assert got[4]["rounds"] == want[4]["rounds"]
+        assert got[4]["items"] == want[4]["items"]
