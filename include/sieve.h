@@ -182,8 +182,8 @@ enum {
  *   rows_read_tc, pairs_tc  the part of rows_read / pairs done on the tensor cores
  *   status       device status word (0, or a SIEVE_E* code)
  *   extended     -1: every order was ranked whole, or was given; else the call
- *                ranked the first centroids of each order (a small window),
- *                and this many queries went past them and were ranked whole
+ *                ranked the first centroids of each order (a small window
+ *                and a tight threshold), and this many queries went past them and were ranked whole
  *                as well (the launches and time of both are SIEVE_K_RANK's and
  *                SIEVE_K_RANK_MMA's) */
 typedef struct {
@@ -274,8 +274,9 @@ sieve_status sieve_screen_scores(const sieve_index_view *ix, const float *Q, int
 
 /* Workspace bytes sieve_search needs for nq queries with these parameters.
  * host_io = 1 sizes it for sieve_search_host (adds device staging for the
- * queries and results).  With a small window it includes the lists with which
- * a search ranks the first centroids of each order before the rest; a search
+ * queries and results).  With a small window and a tight threshold it
+ * includes the lists with which a search ranks the first centroids of each
+ * order before the rest; a search
  * takes a workspace without room for them (one sized for other parameters)
  * all the same, and ranks every order whole. */
 sieve_status sieve_search_workspace_size(const sieve_index_view *ix, int64_t nq,

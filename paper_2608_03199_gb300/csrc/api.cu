@@ -80,6 +80,19 @@ constexpr float kScreenMinTau = 0.85f; // ... and this threshold up (below it ne
 constexpr int64_t kPrefixAlwaysNlist = 2048;
 constexpr int64_t kPrefixMinQueries = 4096;
 constexpr int64_t kPrefixMinWide = 256;
+// A loose threshold makes probes hit and stop lines run past the prefix: then
+// a search pays the prefix and the full ranking both.  A small batch pays the
+// full ranking's latency with the first query that goes past; a large one is
+// bound by its rate, and pays by the share of them.  W = 8, prefix against
+// full ranking, on synthetic mixtures and on groups of neighbouring centroids:
+//   tau 0.80, 1,024 queries x 16,384 x 96: 2,527 and 2,221 us; x 4,096 x 256:
+//     437 and 573
+//   tau 0.70, 1,024 x 2,049 x 96: 315 and 275; 65,536 of them 920 and 1,749;
+//     131,072 x 16,384 x 96 30.1 and 30.5 ms
+//   tau 0.45, 16 x 2,049 x 96: 339 and 238; 16,384 x 8,192 x 96 3,510 and
+//     2,971; 131,072 x 8,192 x 256 8.2 and 6.8 ms
+constexpr int64_t kPrefixLargeBatch = 16384;
+constexpr float kPrefixMinTau = 0.85f, kPrefixMinTauLarge = 0.70f;
 constexpr int64_t kAutoCapMax = int64_t(1) << 24;
 constexpr int64_t kCapMax = int64_t(1) << 30;
 
@@ -105,10 +118,11 @@ struct Layout {
 };
 
 // Whether a search ranks a prefix of each order first: a tensor-core ranking,
-// the centroids laid out for the bulk pipeline, and a window that visits few
-// of the nprobe ranks.  any_window: whether one of its windows would.
+// the centroids laid out for the bulk pipeline, and a window and a threshold
+// with which few of the nprobe ranks are visited.  any_window: whether one of its windows would.
 bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p, bool any_window = false) {
     if (p->scan_path == 1 || !rank_tc_supported(ix->nlist, p->nprobe)) return false;
+    if (!(p->tau >= (nq < kPrefixLargeBatch ? kPrefixMinTau : kPrefixMinTauLarge))) return false;
     // past d = 256 the prefix lays the centroids out itself, which a few queries do not repay
     if (ix->d <= 256 ? !ix->tc_centroids : nq < kPrefixMinWide) return false;
     return (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&

@@ -4,7 +4,9 @@ full order: probes, counts and ids must be the same, scores within 1e-5.
 
 Low thresholds make most probes hit, so stop lines run far past the prefix
 (16 or 32 entries less the margin); identical centroids leave no verified
-prefix at all."""
+prefix at all.  A search takes a prefix only at a tight threshold, so a low one
+is reached by longer vectors: rows and queries times a turn a threshold of tau
+into tau a^2 (``_stretch``), with the same hits."""
 import numpy as np
 import pytest
 import torch
@@ -19,7 +21,13 @@ def dev():
     return torch.device("cuda:0")
 
 
-def _index(sieve, dev, n, d, nlist, seed, grouped=False, equal=0):
+def _stretch(tau, at=0.9):
+    """The factor with which rows and queries meet the threshold `at` where the
+    unit ones meet tau."""
+    return (at / tau) ** 0.5
+
+
+def _index(sieve, dev, n, d, nlist, seed, grouped=False, equal=0, tau=0.9):
     g = torch.Generator().manual_seed(seed)
     unit = lambda x: x / x.norm(dim=1, keepdim=True)
     C = unit(torch.randn(nlist, d, generator=g))
@@ -29,7 +37,7 @@ def _index(sieve, dev, n, d, nlist, seed, grouped=False, equal=0):
     if equal:     # blocks of identical centroids: exact ties
         C = C[torch.arange(nlist) // equal * equal].contiguous()
     a = torch.randint(0, nlist, (n,), generator=g)
-    X = unit(C[a] + 0.9 * torch.randn(n, d, generator=g) / d ** 0.5)
+    X = unit(C[a] + 0.9 * torch.randn(n, d, generator=g) / d ** 0.5) * _stretch(tau)
     return sieve.build_layout(X.to(dev), a.int().to(dev), nlist, C.to(dev)), X
 
 
@@ -58,7 +66,7 @@ CASES = [  # n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal
 @pytest.mark.parametrize("n,d,nlist,nq,nprobe,W,tau,lookahead,grouped,equal", CASES)
 def test_prefix_equals_full_order(dev, n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal):
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, n, d, nlist, seed=n + d + nlist, grouped=grouped, equal=equal)
+    ix, X = _index(sieve, dev, n, d, nlist, seed=n + d + nlist, grouped=grouped, equal=equal, tau=tau)
     # up to 2,048 centroids a batch takes the prefix from 4,096 queries up: the
     # small batches repeat theirs
     rows = torch.randperm(n, generator=torch.Generator().manual_seed(3))[:nq]
@@ -68,16 +76,16 @@ def test_prefix_equals_full_order(dev, n, d, nlist, nq, nprobe, W, tau, lookahea
     Q, qids = X[rows].to(dev), rows.to(dev)
     order = sieve.rank_partitions(ix, Q, nprobe)
     kw = dict(lookahead=lookahead, query_ids=qids, check=True)
-    want = [x.cpu().numpy() for x in sieve.search(ix, Q, tau, 10, nprobe, W, order=order, **kw)]
+    want = [x.cpu().numpy() for x in sieve.search(ix, Q, 0.9, 10, nprobe, W, order=order, **kw)]
     for loop in (0, 1):
-        got = [x.cpu().numpy() for x in sieve.search(ix, Q, tau, 10, nprobe, W, loop=loop, **kw)]
+        got = [x.cpu().numpy() for x in sieve.search(ix, Q, 0.9, 10, nprobe, W, loop=loop, **kw)]
         # a query may differ only through two centroid scores, or two results,
         # closer than the rounding of either: at most one here in 500
         bad = (got[3] != want[3]) | (got[2] != want[2]) | (got[0] != want[0]).any(1)
         assert bad.sum() <= nq // 500, (int(bad.sum()), np.flatnonzero(bad)[:5])
         ok = ~bad
         fin = np.isfinite(want[1][ok])
-        assert np.abs(got[1][ok][fin] - want[1][ok][fin]).max(initial=0) <= 1e-5
+        assert np.abs(got[1][ok][fin] - want[1][ok][fin]).max(initial=0) <= 1e-5 * _stretch(tau) ** 2
         # no partition visited twice: no result id repeats
         for r in got[0][got[2] > 1][:2000]:
             r = r[r >= 0]
@@ -86,18 +94,18 @@ def test_prefix_equals_full_order(dev, n, d, nlist, nq, nprobe, W, tau, lookahea
 
 def test_prefix_host_path(dev):
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 30_000, 96, 300, seed=9)
+    ix, X = _index(sieve, dev, 30_000, 96, 300, seed=9, tau=0.5)
     Q = X[:25_000].contiguous()          # two upload chunks
     ids = torch.arange(25_000)
-    a = sieve.search(ix, Q.to(dev), 0.5, 10, 100, 8, query_ids=ids.to(dev), check=True)
-    b = sieve.search_host(ix, Q.pin_memory(), 0.5, 10, 100, 8, query_ids_host=ids.pin_memory())
+    a = sieve.search(ix, Q.to(dev), 0.9, 10, 100, 8, query_ids=ids.to(dev), check=True)
+    b = sieve.search_host(ix, Q.pin_memory(), 0.9, 10, 100, 8, query_ids_host=ids.pin_memory())
     for x, y in zip(a, b):
         assert torch.equal(x.cpu(), y)
 
 
 def test_nan_centroid_is_ranked_as_by_the_full_order(dev):
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 10_000, 96, 320, seed=4)
+    ix, X = _index(sieve, dev, 10_000, 96, 320, seed=4, tau=0.5)
     C = ix.centroids.clone()
     C[17, 3] = float("nan")
     ix = sieve.build_layout(ix.vectors, torch.repeat_interleave(
@@ -105,8 +113,8 @@ def test_nan_centroid_is_ranked_as_by_the_full_order(dev):
     Q = X[:5_000].to(dev)
     qids = torch.full((5_000,), -1, dtype=torch.int64, device=dev)
     order = sieve.rank_partitions(ix, Q, 64)
-    want = sieve.search(ix, Q, 0.5, 10, 64, 8, query_ids=qids, order=order, check=True)
-    got = sieve.search(ix, Q, 0.5, 10, 64, 8, query_ids=qids, check=True)
+    want = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, order=order, check=True)
+    got = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, check=True)
     for x, y in zip(got, want):
         assert torch.equal(x, y)
 
@@ -171,21 +179,21 @@ def test_stats_tell_which_ranking_ran(dev, nq):
     """extended: -1 where every order is ranked whole or given, else the queries
     ranked whole after their prefix, whose launches count as the ranking's."""
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 12_000, 64, 2_500, seed=2)
+    ix, X = _index(sieve, dev, 12_000, 64, 2_500, seed=2, tau=0.2)
     Q, qids = X[:nq].to(dev), torch.arange(nq, device=dev)
     run = lambda tau, W, **kw: sieve.search(ix, Q, tau, 10, 64, W, query_ids=qids, stats=True, **kw)[4]
     assert run(0.9, 8, order=sieve.rank_partitions(ix, Q, 64))["extended"] == -1
     assert run(0.9, 64)["extended"] == -1
     assert run(0.9, 8, scan_path="simt")["extended"] == -1
-    none = run(0.999, 8)
+    none = run(0.999 * _stretch(0.2) ** 2, 8)
     assert none["extended"] == 0
     assert none["kernel_launches"]["rank"] == 3 and none["kernel_launches"]["rank_mma"] == 1
     for loop in (0, 1):
-        some = run(0.2, 8, loop=loop)
+        some = run(0.9, 8, loop=loop)
         assert nq // 2 < some["extended"] <= nq
         # a part of an extension is a gather, a full ranking and a merge
         assert some["kernel_launches"]["rank"] >= 3 + 8 and some["kernel_launches"]["rank_mma"] >= 1 + 2
-    prof = sieve.search(ix, Q, 0.2, 10, 64, 8, query_ids=qids, profile=True)[4]
+    prof = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, profile=True)[4]
     assert prof["kernel_launches"]["rank_mma"] == some["kernel_launches"]["rank_mma"]
     assert prof["kernel_ms"]["rank"] > prof["kernel_ms"]["rank_mma"] > 0
 
@@ -196,12 +204,28 @@ def test_an_extension_takes_no_round_of_its_own(dev, lookahead, nq, d, nlist, W)
     """A query is listed in the round that raises its stop line, so the rounds
     are those of the same search on the whole order."""
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 12_000, d, nlist, seed=8)
+    ix, X = _index(sieve, dev, 12_000, d, nlist, seed=8, tau=0.3)
     Q, qids = X[:nq].to(dev), torch.arange(nq, device=dev)
     kw = dict(lookahead=lookahead, query_ids=qids, stats=True)
-    want = sieve.search(ix, Q, 0.3, 10, 64, W, order=sieve.rank_partitions(ix, Q, 64), **kw)
+    want = sieve.search(ix, Q, 0.9, 10, 64, W, order=sieve.rank_partitions(ix, Q, 64), **kw)
     for loop in (0, 1):
-        got = sieve.search(ix, Q, 0.3, 10, 64, W, loop=loop, **kw)
+        got = sieve.search(ix, Q, 0.9, 10, 64, W, loop=loop, **kw)
         assert got[4]["extended"] > 0
         assert got[4]["rounds"] == want[4]["rounds"]
         assert got[4]["items"] == want[4]["items"]
+
+
+@pytest.mark.parametrize("nq,tau,prefix", [(1_000, 0.85, True), (1_000, 0.84, False), (16_383, 0.84, False),
+                                           (16_384, 0.70, True), (16_384, 0.69, False)])
+def test_a_loose_threshold_ranks_whole(dev, nq, tau, prefix):
+    """Below the threshold lines every order is ranked whole at once."""
+    import paper_2608_03199_gb300 as sieve
+    ix, X = _index(sieve, dev, 20_000, 32, 2_100, seed=12)
+    Q = X[:nq].to(dev)
+    order = sieve.rank_partitions(ix, Q, 32)
+    want = sieve.search(ix, Q, tau, 10, 32, 8, order=order)
+    got = sieve.search(ix, Q, tau, 10, 32, 8, stats=True)
+    assert (got[4]["extended"] >= 0) == prefix
+    if not prefix:
+        for x, y in zip(got[:4], want):
+            assert torch.equal(x, y)
