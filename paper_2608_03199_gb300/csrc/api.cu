@@ -75,11 +75,13 @@ constexpr float kScreenMinTau = 0.85f; // ... and this threshold up (below it ne
                                        // of a probed partition needs its fp32 rescore)
 // Up to 2,048 centroids the full ranking is two short launches, and a small
 // batch pays the latency of filling the prefix's lists instead of bandwidth
-// (1,003 queries x 149 x 100: ranking 42 us whole, 58 us as a prefix; 10,007 x
-// 1,024 x 256: 60 us less as a prefix)
+// (tau 0.9, W 8, prefix against full: 64 queries x 149 x 100 110 and 100 us,
+// 1,024 x 512 x 96 122 and 115, 1,024 x 1,024 x 256 158 and 154, 4,096 x 1,024 x 96
+// 158 and 188, 16,384 x 1,024 x 96 243 and 358).  Above it is quicker from one
+// query on, past d = 256, where it lays the centroids out itself, too (one query
+// x 8,192 x 96 78 and 140, x 65,536 x 96 243 and 473, x 4,096 x 512 85 and 156).
 constexpr int64_t kPrefixAlwaysNlist = 2048;
 constexpr int64_t kPrefixMinQueries = 4096;
-constexpr int64_t kPrefixMinWide = 256;
 // A loose threshold makes probes hit and stop lines run past the prefix: then
 // a search pays the prefix and the full ranking both.  A small batch pays the
 // full ranking's latency with the first query that goes past; a large one is
@@ -123,10 +125,9 @@ struct Layout {
 bool use_prefix(const sieve_index_view *ix, int64_t nq, const sieve_params *p, bool any_window = false) {
     if (p->scan_path == 1 || !rank_tc_supported(ix->nlist, p->nprobe)) return false;
     if (!(p->tau >= (nq < kPrefixLargeBatch ? kPrefixMinTau : kPrefixMinTauLarge))) return false;
-    // past d = 256 the prefix lays the centroids out itself, which a few queries do not repay
-    if (ix->d <= 256 ? !ix->tc_centroids : nq < kPrefixMinWide) return false;
+    if (ix->d <= 256 && !ix->tc_centroids) return false;   // past that the prefix lays them out itself
     return (ix->nlist > kPrefixAlwaysNlist || nq >= kPrefixMinQueries) &&
-           rank_prefix_len(ix->nlist, p->nprobe, any_window ? 1 : p->W, ix->d) > 0;
+           rank_prefix_len(nq, ix->nlist, p->nprobe, any_window ? 1 : p->W, ix->d) > 0;
 }
 
 // What a layout's ranking scratch has room for: the full ranking alone (the
@@ -564,7 +565,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
     }
     if (with_rank || prefix)
         SIEVE_CUDA(rank_tc || prefix ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
-    if (prefix) SIEVE_CUDA(prepare_rank_prefix(ix->nlist, p->nprobe, p->W, ix->d));
+    if (prefix) SIEVE_CUDA(prepare_rank_prefix(nq, ix->nlist, p->nprobe, p->W, ix->d));
     const int blocks = scan_blocks_for(smem);
 
     float ms[SIEVE_NKERNELS] = {0};
@@ -1005,7 +1006,7 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
     const bool rank_tc = p->scan_path != 1 && L.rank_scratch != 0;
     const bool prefix = rank_tc && nchunks > 0 && L.prefix;
     SIEVE_CUDA(rank_tc ? prepare_rank_tc(p->nprobe, ix->d) : prepare_rank(p->nprobe));
-    if (prefix) SIEVE_CUDA(prepare_rank_prefix(ix->nlist, p->nprobe, p->W, ix->d));
+    if (prefix) SIEVE_CUDA(prepare_rank_prefix(nq, ix->nlist, p->nprobe, p->W, ix->d));
     SIEVE_CUDA(cudaMemsetAsync(dstatus, 0, sizeof(int), st));
     SIEVE_CUDA(cudaEventRecord(cl.start, st));             // earlier work on the staging
     SIEVE_CUDA(cudaStreamWaitEvent(cl.stream, cl.start, 0));

@@ -523,16 +523,34 @@ static int64_t fill_bytes(int64_t nlist, int d) {
 // Groups kept per list, and so ranks found: min(W, nprobe) are visited for
 // certain, a hit at rank j adds up to rank j + W, and one or two are lost to
 // the margin.  16 serve windows up to 10 and 32 up to 24; 0: rank all of nprobe (a
-// wider window reads most of the order anyway, and a list of fewer than 64
-// centroids is ranked whole as cheaply).
+// wider window reads most of the order anyway).
+//
+// Fewer than L groups of 32 in all are all kept, and nothing is left out: the
+// full ranking is as quick or quicker (W 8, tau 0.9, prefix against full:
+// 16,384 queries x 64 x 96 313 and 287 us, x 512 x 96 258 and 276, 8,192 x 768 x
+// 96 192 and 229; W 20: 8,192 x 512 x 96 279 and 249, 16,384 x 1,500 x 96 411
+// and 692).
+//
+// About 0.15% of the queries go past 13 ranks at W 8 and tau 0.9 on the
+// synthetic mixtures, and 6e-5 past 20.  The first of them costs a small batch
+// a full ranking's latency (1,024 x 16,384 x 96: about 215 us of 595), so where
+// a batch is likely to have one and its time is latency still, 32 groups are
+// kept: 1,024 x 16,384 x 96 595 -> 450 us (526 ranked whole), 4,096 925 -> 748
+// (822), 4,096 x 1,024 x 256 572 -> 502 (505); where nobody goes past 16 it
+// costs 5 to 10% (1,024 x 8,192 x 256 301 -> 317, 4,096 440 -> 485).  From 8,192
+// queries the longer lists cost more than they save (easy: 8,192 x 8,192 x 96
+// 408 -> 489; mixture: 8,192 x 16,384 x 96 1,071 -> 1,040), below 256 such a
+// query is rare (64 x 16,384 x 96 180 -> 197).
+constexpr int64_t kLongLists = 256, kLongListsEnd = 8192;
 static bool prefix_fits(int64_t nlist, int nprobe, int d, int L) {
-    return nlist >= 4 * (int64_t)L && nprobe >= 4 && prefix_stages(d) > 0;
+    return nlist >= 32 * (int64_t)L && nprobe >= 4 && prefix_stages(d) > 0;
 }
 
-int rank_prefix_len(int64_t nlist, int nprobe, int W, int d) {
+int rank_prefix_len(int64_t nq, int64_t nlist, int nprobe, int W, int d) {
     const int need = W < nprobe ? W : nprobe;
-    const int L = need <= 10 ? 16 : need <= 24 ? 32 : 0;
-    return L && prefix_fits(nlist, nprobe, d, L) ? L : 0;
+    if (need > 24) return 0;
+    if ((need > 10 || (nq >= kLongLists && nq < kLongListsEnd)) && prefix_fits(nlist, nprobe, d, 32)) return 32;
+    return need <= 10 && prefix_fits(nlist, nprobe, d, 16) ? 16 : 0;
 }
 
 // bytes of one (query, range)'s list: the scores, maxima and first centroids of
@@ -625,13 +643,13 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
 size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int W, int d) {
     int64_t b = 0;
     for (int L : {16, 32})
-        if (nq > 0 && (W == 0 ? prefix_fits(nlist, nprobe, d, L) : rank_prefix_len(nlist, nprobe, W, d) == L))
+        if (nq > 0 && (W == 0 ? prefix_fits(nlist, nprobe, d, L) : rank_prefix_len(nq, nlist, nprobe, W, d) == L))
             b = std::max(b, prefix_scratch(nq, nlist, nprobe, d, L).total);
     return (size_t)b;
 }
 
 int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext) {
-    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nq, nlist, nprobe, W, d));
     unsigned char *w = static_cast<unsigned char *>(scratch);
     *ext = reinterpret_cast<int *>(w + S.ext);
     return reinterpret_cast<int *>(w + S.limit);
@@ -649,8 +667,8 @@ static PrefixScan scan_kernel(int d, int L) {
     return L == 16 ? k_prefix_scan<16, 128, 2> : k_prefix_scan<32, 128, 2>;
 }
 
-cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d) {
-    const int L = rank_prefix_len(nlist, nprobe, W, d);
+cudaError_t prepare_rank_prefix(int64_t nq, int64_t nlist, int nprobe, int W, int d) {
+    const int L = rank_prefix_len(nq, nlist, nprobe, W, d);
     return cudaFuncSetAttribute(scan_kernel(d, L), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)scan_smem(d));
 }
@@ -669,7 +687,7 @@ static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe,
 // kernel launches of one prefix ranking of nq queries (and its contraction
 // launches), for scratch sized for plan_nq
 int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma) {
-    const int L = rank_prefix_len(nlist, nprobe, W, d);
+    const int L = rank_prefix_len(plan_nq, nlist, nprobe, W, d);
     const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
     const int chunks = (int)ceil_div(nq, S.chunk);
     *mma = chunks;
@@ -683,7 +701,7 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
                                 float *mma_ms, int wait_limit) {
     if (nq <= 0) return cudaSuccess;
-    const int L = rank_prefix_len(nlist, nprobe, W, d);
+    const int L = rank_prefix_len(plan_nq, nlist, nprobe, W, d);
     const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
     const PrefixPlan P = prefix_plan(plan_nq, nlist, d, L);
     unsigned char *w = static_cast<unsigned char *>(scratch);
@@ -757,7 +775,7 @@ cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *
                              int nprobe, int W, int32_t *order, float *cscores, void *scratch,
                              const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st,
                              float *mma_ms) {
-    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nq, nlist, nprobe, W, d));
     const PrefixScratch::Ext &E = S.ext_part[part];
     unsigned char *w = static_cast<unsigned char *>(scratch);
     int *limit = reinterpret_cast<int *>(w + S.limit);
@@ -781,7 +799,7 @@ cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *
 }
 
 int rank_ext_launches(int part, int64_t nq, int64_t nlist, int nprobe, int W, int d, bool bulk, int *mma) {
-    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nlist, nprobe, W, d));
+    const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nq, nlist, nprobe, W, d));
     const int64_t chunk = S.ext_part[part].chunk;
     int n = 0;
     *mma = 0;

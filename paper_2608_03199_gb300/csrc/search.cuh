@@ -154,10 +154,10 @@ int rank_bulk_stages(int d);                     // 0 when the bulk ranking does
 // the first ranks alone, and the full ranking of the queries that need more
 // (rank_prefix.cu): entries kept per query list, 0 when it does not apply; the
 // scratch (the limits and the extension list first, for the whole search)
-int rank_prefix_len(int64_t nlist, int nprobe, int W, int d);
+int rank_prefix_len(int64_t nq, int64_t nlist, int nprobe, int W, int d);
 size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int W, int d);   // W = 0: any window
 int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext);
-cudaError_t prepare_rank_prefix(int64_t nlist, int nprobe, int W, int d);
+cudaError_t prepare_rank_prefix(int64_t nq, int64_t nlist, int nprobe, int W, int d);
 int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma);
 cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,

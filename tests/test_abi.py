@@ -130,7 +130,7 @@ def test_workspace_has_prefix_lists_only_where_a_search_uses_them_without_gpu():
 
     for nlist, d, nq, nprobe, W, layout in ((1024, 256, 2_000, 64, 8, True), (149, 100, 4_000, 24, 4, True),
                                             (1024, 256, 20_000, 64, 64, True), (8192, 96, 20_000, 128, 8, False),
-                                            (8192, 512, 200, 128, 8, False)):
+                                            (8192, 516, 200, 128, 8, False)):
         total, rank = size(nlist, d, nq, nprobe, W, layout=layout)
         assert total <= size(nlist, d, nq, nprobe, W, "simt", layout)[0] + rank + 512, (nlist, d, nq, nprobe, W)
     # where it is used, the lists and the extension's buffers come on top
