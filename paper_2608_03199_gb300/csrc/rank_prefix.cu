@@ -65,6 +65,7 @@ struct PrefixArgs {
     int *status;
     int wait_limit;      // polls of the epilogue's accumulator wait (0: default)
     const unsigned char *tc_cent;
+    const unsigned *cmax;   // launch_cnorm_max of the centroids
     int nranges;         // centroid ranges per query tile
     int64_t range_len;   // centroids per range, a multiple of 128
     float *list_s;       // [nq][nranges][kL][32] the kept groups' screened scores (raw: x 2^16) ...
@@ -74,6 +75,17 @@ struct PrefixArgs {
 };
 
 __device__ int g_prefix_status_sink;
+
+// Scores past fp16's range (|256 x| above 65,504) are not screened soundly, and
+// a NaN row is left out by every maximum: with such centroids no prefix is
+// found, and neither kernel goes over anything.
+constexpr float kScreenMaxNorm = 200.f;
+__device__ __forceinline__ float cmax_norm(const unsigned *cmax) {   // rounded upward
+    return __uint_as_float(cmax[0]) * (1.f + 0x1p-20f);
+}
+__device__ __forceinline__ bool centroids_screen(const unsigned *cmax) {
+    return cmax[1] == 0u && cmax_norm(cmax) < kScreenMaxNorm;
+}
 
 // kSubT = 2: centroids in the tensor-core layout, d <= 256.  kSubT = 1: d <= 512,
 // A's hi half alone fills 256 columns, and the centroids' hi halves in a layout
@@ -93,7 +105,9 @@ struct PrefixMode {
         int64_t c0, nb;
         int ns, sstep;   // sample chunks first: chunks 0, sstep, 2 sstep, ...
     };
-    __device__ static int num_tiles(const Args &a) { return (int)ceil_div(a.nq, kRows) * a.nranges; }
+    __device__ static int num_tiles(const Args &a) {
+        return centroids_screen(a.cmax) ? (int)ceil_div(a.nq, kRows) * a.nranges : 0;
+    }
     __device__ static int *tile_counter(const Args &) { return nullptr; }
     __device__ static int d(const Args &a) { return a.d; }
     __device__ static int *status(const Args &a) { return a.status ? a.status : &g_prefix_status_sink; }
@@ -261,7 +275,7 @@ template <int kL, int KPL, int NV>
 __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const float *__restrict__ Q, int64_t nq, const float *__restrict__ C, int64_t nlist, int d,
     const float *__restrict__ list_s, const int2 *__restrict__ list_g,
-    const float2 *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax_bits,
+    const float2 *__restrict__ list_t, int nranges, int nprobe, const unsigned *__restrict__ cmax,
     const int *__restrict__ status, int32_t *__restrict__ order, float *__restrict__ cscores,
     int *__restrict__ limit) {
     constexpr float kS = 1.f / 65536.f;
@@ -271,7 +285,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     const unsigned below = (1u << lane) - 1u;
     const int64_t q = (int64_t)blockIdx.x * kFinalWarps + warp;
     if (q >= nq) return;
-    if (status && *status != 0) {
+    if ((status && *status != 0) || !centroids_screen(cmax)) {
         if (lane == 0) limit[q] = 0;
         return;
     }
@@ -430,15 +444,12 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     // the norms and the margin rounded upward (the bounds of k_rank_threshold:
     // the screen's, and one that covers fp32 sums with room)
     const float qn = __fsqrt_ru(qq) * (1.f + 0x1p-20f);
-    const float cn = __uint_as_float(*cmax_bits) * (1.f + 0x1p-20f);
+    const float cn = cmax_norm(cmax);
     const float rd = __fsqrt_ru((float)d);
     const float fp32 = (0x1p-20f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
     const float scr = (0x1p-10f + 0x1p-12f + (float)d * 0x1p-22f) * qn * cn + 0x1p-26f * rd * (qn + cn);
     const float margin = (scr + fp32) * (1.f + 0x1p-16f);
-    // scores past fp16's range (|256 x| above 65,504) are not screened soundly,
-    // and a NaN row is left out by every maximum
-    const bool sound = cmax_bits[1] == 0u && qn < 200.f && cn < 200.f;
-    const bool first = sound && cid[0] != INT32_MAX &&
+    const bool first = qn < kScreenMaxNorm && cid[0] != INT32_MAX &&
                        (un == 0u || s[0] > __fadd_ru(key_score(un), margin));
     const unsigned b = __ballot_sync(0xffffffffu, first);
     int R = b == 0xffffffffu ? 32 : __ffs(~b) - 1;   // the sorted entries up to the first that may not be
@@ -674,14 +685,13 @@ cudaError_t prepare_rank_prefix(int64_t nq, int64_t nlist, int nprobe, int W, in
 }
 
 template <int kL, int KPL>
-static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, const unsigned *cmax,
-                                int32_t *order, float *cscores, int *limit, cudaStream_t st) {
+static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, int32_t *order, float *cscores, int *limit, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(a.nq, kFinalWarps);
     auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 1>
              : a.d <= 256 ? k_prefix_final<kL, KPL, 2>
                           : k_prefix_final<kL, KPL, 4>;
     f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_g, a.list_t, a.nranges, nprobe,
-                                           cmax, a.status, order, cscores, limit);
+                                           a.cmax, a.status, order, cscores, limit);
 }
 
 // kernel launches of one prefix ranking of nq queries (and its contraction
@@ -730,7 +740,7 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);
-        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, wait_limit, tc_cent, P.nranges, P.range_len,
+        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, wait_limit, tc_cent, cmax, P.nranges, P.range_len,
                            list_s, list_g, list_t};
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, prefix_sub(d) * tcp::kM) * P.nranges, num_sms());
         if (mma_ms) {
@@ -746,8 +756,8 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
         int *lim = limit + q0 + b;
         const int kpl = (int)ceil_div(P.nranges * L, 32);
 #define SIEVE_PREFIX(K)                                                                       \
-    if (L == 16) launch_prefix_final<16, K>(a, C, nprobe, cmax, o, cs, lim, st);               \
-    else launch_prefix_final<32, K>(a, C, nprobe, cmax, o, cs, lim, st)
+    if (L == 16) launch_prefix_final<16, K>(a, C, nprobe, o, cs, lim, st);               \
+    else launch_prefix_final<32, K>(a, C, nprobe, o, cs, lim, st)
         if (kpl <= 1) { SIEVE_PREFIX(1); }
         else if (kpl <= 2) { SIEVE_PREFIX(2); }
         else if (kpl <= 4) { SIEVE_PREFIX(4); }

@@ -129,19 +129,45 @@ def test_prefix_host_path(dev):
         assert torch.equal(x.cpu(), y)
 
 
-def test_nan_centroid_is_ranked_as_by_the_full_order(dev):
+@pytest.mark.parametrize("d", [96, 320])
+@pytest.mark.parametrize("odd", ["nan centroid", "long centroid", "infinite centroid", "long centroids",
+                                 "nan query", "infinite query", "long query", "zero query"])
+def test_rows_that_cannot_be_screened_are_ranked_as_by_the_full_order(dev, d, odd):
+    """NaN, infinities and norms from 200 up leave the prefix empty: of every
+    query where a centroid has them, of the query alone where a query does."""
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 10_000, 96, 640, seed=4, tau=0.5)
-    C = ix.centroids.clone()
-    C[17, 3] = float("nan")
+    nlist, nq = 2_100, 700
+    ix, X = _index(sieve, dev, 10_000, d, nlist, seed=4, tau=0.5)
     ix = sieve.build_layout(ix.vectors, torch.repeat_interleave(
-        torch.arange(640, device=dev), ix.list_offsets.diff()).int(), 640, C)
-    Q = X[:5_000].to(dev)
-    qids = torch.full((5_000,), -1, dtype=torch.int64, device=dev)
+        torch.arange(nlist, device=dev), ix.list_offsets.diff()).int(), nlist, ix.centroids.clone())
+    C, Q = ix.centroids, X[:nq].to(dev)
+    if odd == "nan centroid":
+        C[17, 3] = float("nan")
+    elif odd == "long centroid":
+        C[17] *= 210.
+    elif odd == "infinite centroid":
+        C[2_099, 0] = float("inf")
+    elif odd == "long centroids":
+        C *= 300.
+    elif odd == "nan query":
+        Q[5, 7] = float("nan")
+    elif odd == "infinite query":
+        Q[699, 0] = -float("inf")
+    elif odd == "long query":
+        Q[5] *= 250.
+    else:
+        Q[5] = 0.
+    if ix.tc_centroids is not None:
+        ix = sieve.add_tc_layout(ix)
+    qids = torch.full((nq,), -1, dtype=torch.int64, device=dev)
     order = sieve.rank_partitions(ix, Q, 64)
     want = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, order=order, check=True)
-    got = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, check=True)
-    for x, y in zip(got, want):
+    got = sieve.search(ix, Q, 0.9, 10, 64, 8, query_ids=qids, stats=True)
+    if "centroid" in odd:
+        assert got[4]["extended"] == nq
+    else:
+        assert 1 <= got[4]["extended"] <= nq
+    for x, y in zip(got[:4], want):
         assert torch.equal(x, y)
 
 
