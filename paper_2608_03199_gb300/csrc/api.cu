@@ -653,7 +653,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         const bool bulk = a.tc_cent && rank_bulk_stages(a.d) > 0;
         int prefix_mma = 0, prefix_launches = 0;   // the prefix ranking, if it ran here, and its extensions
         if (prefix && with_rank)
-            prefix_launches = rank_prefix_launches(a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma);
+            prefix_launches = rank_prefix_launches(0, a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma);
         for (int i = 0; prefix && i < 2; ++i)
             if (c.ext_runs[i] > 0) {
                 int mma = 0;
@@ -1035,7 +1035,7 @@ sieve_status sieve_search_host(const sieve_index_view *ix, const float *Q_host, 
                                            static_cast<const unsigned char *>(ix->tc_centroids), st, nullptr,
                                            p->wait_limit));
             int mma = 0;
-            rank_launches += rank_prefix_launches(n, nq, ix->nlist, p->nprobe, p->W, ix->d, &mma);
+            rank_launches += rank_prefix_launches(q0, n, nq, ix->nlist, p->nprobe, p->W, ix->d, &mma);
             mma_launches += mma;
             continue;
         }

@@ -694,18 +694,20 @@ static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe,
                                            a.cmax, a.status, order, cscores, limit);
 }
 
-// kernel launches of one prefix ranking of nq queries (and its contraction
-// launches), for scratch sized for plan_nq
-int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma) {
+// kernel launches of the prefix ranking of nq queries from q0 on (and its
+// contraction launches), for scratch sized for plan_nq
+int rank_prefix_launches(int64_t q0, int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma) {
     const int L = rank_prefix_len(plan_nq, nlist, nprobe, W, d);
     const PrefixScratch S = prefix_scratch(plan_nq, nlist, nprobe, d, L);
     const int chunks = (int)ceil_div(nq, S.chunk);
     *mma = chunks;
-    return 2 * chunks + 1 + (prefix_sub(d) == 1 ? 1 : 0);
+    return 2 * chunks + (q0 > 0 ? 0 : prefix_sub(d) == 1 ? 2 : 1);
 }
 
 // The prefix of nq queries q0 .. q0 + nq - 1 of a batch of plan_nq (whose
-// scratch this is): order, cscores (nullable) and the scratch's limits.
+// scratch this is): order, cscores (nullable) and the scratch's limits.  The
+// largest norm and the wide rows' layout are made with the first part (q0 = 0)
+// and stay in the scratch for the others, which follow it on the same stream.
 cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
@@ -730,13 +732,15 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
             for (cudaEvent_t e : v) cudaEventDestroy(e);
         }
     } ev;
-    cudaError_t e = launch_cnorm_max(C, nlist, d, cmax, st);
+    cudaError_t e = q0 == 0 ? launch_cnorm_max(C, nlist, d, cmax, st) : cudaSuccess;
     if (e != cudaSuccess) return e;
     if (prefix_sub(d) == 1) {
-        const int64_t pieces = ceil_div(nlist, kTcRows) * ceil_div(d, 64) * kTcRows * 8;
-        k_prefix_fill<<<(unsigned)std::min<int64_t>(ceil_div(pieces, 256), 16 * num_sms()), 256, 0, st>>>(
-            C, nlist, d, (int)ceil_div(d, 64), w + S.fill);
         tc_cent = w + S.fill;
+        if (q0 == 0) {
+            const int64_t pieces = ceil_div(nlist, kTcRows) * ceil_div(d, 64) * kTcRows * 8;
+            k_prefix_fill<<<(unsigned)std::min<int64_t>(ceil_div(pieces, 256), 16 * num_sms()), 256, 0, st>>>(
+                C, nlist, d, (int)ceil_div(d, 64), w + S.fill);
+        }
     }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);

@@ -158,7 +158,7 @@ int rank_prefix_len(int64_t nq, int64_t nlist, int nprobe, int W, int d);
 size_t rank_prefix_scratch_bytes(int64_t nq, int64_t nlist, int nprobe, int W, int d);   // W = 0: any window
 int *rank_prefix_limit(void *scratch, int64_t nq, int64_t nlist, int nprobe, int W, int d, int **ext);
 cudaError_t prepare_rank_prefix(int64_t nq, int64_t nlist, int nprobe, int W, int d);
-int rank_prefix_launches(int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma);
+int rank_prefix_launches(int64_t q0, int64_t nq, int64_t plan_nq, int64_t nlist, int nprobe, int W, int d, int *mma);
 cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t plan_nq, const float *C,
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,

@@ -118,15 +118,34 @@ def test_which_ranking_runs(dev, nlist, nq, W, d, prefix):
     assert torch.equal(got[3], want[3]) and torch.equal(got[2], want[2])
 
 
-def test_prefix_host_path(dev):
+@pytest.mark.parametrize("d", [96, 320])
+def test_prefix_host_path(dev, d):
+    """Each upload chunk's prefix, with the largest norm and the wide rows'
+    layout made once for all of them."""
+    import ctypes
     import paper_2608_03199_gb300 as sieve
-    ix, X = _index(sieve, dev, 30_000, 96, 600, seed=9, tau=0.5)
-    Q = X[:25_000].contiguous()          # two upload chunks
-    ids = torch.arange(25_000)
-    a = sieve.search(ix, Q.to(dev), 0.9, 10, 100, 8, query_ids=ids.to(dev), check=True)
-    b = sieve.search_host(ix, Q.pin_memory(), 0.9, 10, 100, 8, query_ids_host=ids.pin_memory())
+    ix, X = _index(sieve, dev, 30_000, d, 600, seed=9, tau=0.2)
+    nq = 25_000                          # two upload chunks
+    Q = X[:nq].contiguous().pin_memory()
+    ids = torch.arange(nq).pin_memory()
+    a = sieve.search(ix, Q.to(dev), 0.9, 10, 100, 8, query_ids=ids.to(dev), stats=True)
+    b = sieve.search_host(ix, Q, 0.9, 10, 100, 8, query_ids_host=ids)
     for x, y in zip(a, b):
         assert torch.equal(x.cpu(), y)
+    v, p, st = ix.view(), sieve._params(0.9, 10, 100, 8, True, 0, 0), sieve.StatsC()
+    ws = torch.empty(sieve.workspace_size(ix, nq, 0.9, 10, 100, 8, host_io=True), dtype=torch.uint8, device=dev)
+    out = [torch.empty_like(y) for y in b]
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    rc = sieve.lib().sieve_search_host(ctypes.byref(v), ptr(Q), nq, ptr(ids), ctypes.byref(p), *map(ptr, out),
+                                       ctypes.byref(st), ptr(ws), ws.numel(), None)
+    assert rc == 0
+    for x, y in zip(out, b):
+        assert torch.equal(x, y)
+    host = dict(zip(sieve.KERNELS, st.kernel_launches))
+    device = a[4]["kernel_launches"]
+    # a second scan and a second final, and nothing else, for the second chunk
+    assert host["rank"] == device["rank"] + 2 and host["rank_mma"] == device["rank_mma"] + 1
+    assert st.extended == a[4]["extended"] > 0
 
 
 @pytest.mark.parametrize("d", [96, 320])
