@@ -567,10 +567,10 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(SearchArgs a) {
             // (listed as the next round issued, a round later, the ranks to the
             // prefix's end and the rest read their partitions in two rounds: 131K
             // queries x 8,192 x 256 that all go past it 8.5 -> 7.6 ms)
-            if (a.limit) {
+            const int s0 = a.W < a.nprobe ? a.W : a.nprobe;
+            if (a.limit && s > s0) {   // few: the others' limits are not read
                 const int lim = a.limit[q];
-                if (s > lim && lim >= (a.W < a.nprobe ? a.W : a.nprobe))
-                    a.ext[atomicAdd(&ctl->n_ext, 1)] = q;
+                if (s > lim && lim >= s0) a.ext[atomicAdd(&ctl->n_ext, 1)] = q;
             }
         }
     }
@@ -589,11 +589,14 @@ __global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
         more = 0;
     }
     c->more = more;
-    c->ext_n = more ? c->n_ext : 0;
+    const int ext = more ? c->n_ext : 0;
+    c->ext_n = ext;
     c->n_ext = 0;
-    c->tot_ext += (unsigned long long)c->ext_n;
-    c->ext_runs[0] += c->ext_n > 0;
-    c->ext_runs[1] += c->ext_n > kExtFirst;
+    if (ext > 0) {
+        c->tot_ext += (unsigned long long)ext;
+        c->ext_runs[0] += 1;
+        c->ext_runs[1] += ext > kExtFirst;
+    }
     c->n_items = 0;
     c->n_active = 0;
     c->n_tiles = 0;
@@ -604,7 +607,7 @@ __global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
     c->n_continue = 0;
     if (use_cond) {
         cudaGraphSetConditional(conds.more, more ? 1u : 0u);
-        if (a.limit) cudaGraphSetConditional(conds.ext, c->ext_n > 0 ? 1u : 0u);
+        if (a.limit) cudaGraphSetConditional(conds.ext, ext > 0 ? 1u : 0u);
     }
 }
 
