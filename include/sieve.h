@@ -289,7 +289,12 @@ sieve_status sieve_search_workspace_size(const sieve_index_view *ix, int64_t nq,
  *              query's id is neither a candidate nor a hit (self-join
  *              deduplication with queries drawn from the indexed rows)
  *   order      device [nq][nprobe] int32 (nullable): precomputed centroid
- *              ranks; NULL ranks inside the call (sieve_rank_partitions)
+ *              ranks; NULL ranks inside the call, in the order of
+ *              sieve_rank_partitions but for centroids whose scores lie
+ *              within the rounding of either (a few 1e-7 on unit vectors):
+ *              where the first ranks are found before the rest their scores
+ *              are fp32 sums, not three fp16 products, and two such
+ *              centroids may change places
  *   out_ids    device [nq][k] int64: result ids by (score desc, id asc),
  *              -1 past out_count
  *   out_scores device [nq][k] fp32: their similarities, -inf past out_count

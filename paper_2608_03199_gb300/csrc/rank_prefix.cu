@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
         for (int g = 0; g < kL; ++g) {
             const bool sel = raw[g] >= t_raw;   // past the centroids the score is -inf
             const unsigned b = __ballot_sync(0xffffffffu, sel);
-            if (sel) s_id[warp][n + __popc(b & below)] = min(s_c0[warp][g] + lane, (int)nlist - 1);
+            if (sel) s_id[warp][n + __popc(b & below)] = (int)min((unsigned)s_c0[warp][g] + lane, (unsigned)nlist - 1u);
             n += __popc(b);
         }
     } else {

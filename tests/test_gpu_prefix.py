@@ -300,3 +300,29 @@ def test_a_loose_threshold_ranks_whole(dev, nq, tau, prefix):
     if not prefix:
         for x, y in zip(got[:4], want):
             assert torch.equal(x, y)
+
+
+def test_several_passes_of_one_batch(dev):
+    """400,000 queries at W = 16 need more than the 1 GiB of lists: two passes,
+    the second from a whole number of waves of tiles on."""
+    import paper_2608_03199_gb300 as sieve
+    nq, nprobe, W = 400_000, 32, 16
+    ix, X = _index(sieve, dev, 20_000, 32, 2_100, seed=14)
+    rows = torch.randint(0, 20_000, (nq,), generator=torch.Generator().manual_seed(15))
+    Q, qids = X[rows].to(dev), rows.to(dev)
+    order = sieve.rank_partitions(ix, Q, nprobe)
+    kw = dict(query_ids=qids, stats=True)
+    want = sieve.search(ix, Q, 0.9, 10, nprobe, W, order=order, **kw)
+    got = sieve.search(ix, Q, 0.9, 10, nprobe, W, **kw)
+    st = got[4]
+    assert st["extended"] >= 0 and st["kernel_launches"]["rank_mma"] - 2 * (st["extended"] > 0) >= 2
+    bad = (got[3] != want[3]) | (got[2] != want[2]) | (got[0] != want[0]).any(1)
+    as_dict = lambda out: {k: x[bad].cpu().numpy() for k, x in zip(("ids", "scores", "count", "probes"), out)}
+    host = dict(X=X.numpy(), ids=np.arange(20_000), assign=ix.assign.numpy(), centroids=ix.centroids.cpu().numpy())
+    at = bad.nonzero()[:, 0].cpu().numpy()
+    print(f"{len(at)} of {nq} queries differ")
+    assert len(at) <= nq // 1000
+    if len(at):
+        rep = compare(as_dict(got), as_dict(want), host, Q[bad].cpu().numpy(), rows.numpy()[at], 0.9, 10, nprobe,
+                      order[bad].cpu().numpy())
+        assert len(rep["unexplained"]) == 0

@@ -109,3 +109,53 @@ def test_screen_slack_on_adversarial_rounding(dev):
           f"all pairs max {r.max():.3f}")
     assert r.max() < 1.0
     assert diag.max() > 0.5
+
+
+@pytest.mark.parametrize("d", [96, 256, 260, 384, 512])
+def test_prefix_order_under_adversarial_rounding(dev, d):
+    """The prefix ranking relies on the bound up to d = 512, where no screened
+    score can be read.  Queries whose every coordinate the screen rounds down by
+    nearly 2^-11, three centroids equal to each but for a few coordinates (the
+    first ranks; screened low by nearly 2^-10), and 24 whose coordinates are
+    exact in fp16 and whose scores lie between: the screen ranks these first.
+    Every rank that the search wrote must be the exact order's."""
+    rng = np.random.default_rng(d)
+    nq, near, nlist, nprobe = 64, 24, 2_304, 64
+    base = 2.0 ** rng.integers(-4, 0, (nq, d)) * rng.choice([-1.0, 1.0], (nq, d)) * (8.0 / d ** 0.5)
+    base = np.sign(base) * 2.0 ** np.round(np.log2(np.abs(base)))      # powers of two
+    q = base * (1.0 + 2.0**-11 * 0.999)
+    cent = [np.where(rng.random((nlist - nq * (3 + near), d)) < 0.5, 1.0, -1.0) * 2.0**-5]
+    for i in range(nq):
+        for j in range(3):
+            a = q[i].copy()
+            a[rng.choice(d, j + 1, replace=False)] *= 1.0 - 2.0**-9
+            cent.append(a[None])
+        for _ in range(near):
+            up = rng.random(d) < 0.3
+            cent.append((base[i] * np.where(up, 1.0 + 2.0**-10, 1.0))[None])
+    cent = np.concatenate(cent).astype(np.float32)[rng.permutation(nlist)]
+    q = q.astype(np.float32)
+    exact = q.astype(np.float64) @ cent.astype(np.float64).T
+    h = q.astype(np.float16).astype(np.float64) @ cent.astype(np.float16).astype(np.float64).T
+    assert (h.argmax(1) != exact.argmax(1)).mean() > 0.8   # the screen's first is not the first
+    C = torch.from_numpy(cent).to(dev)
+    index = sieve.build_layout(torch.zeros(nlist, d, device=dev),
+                               torch.arange(nlist, dtype=torch.int32, device=dev), nlist, C)
+    ws = sieve.Workspace()
+    args = (index, torch.from_numpy(q).to(dev), 0.9, 10, nprobe, 8)
+    sieve.search(*args, workspace=ws)
+    # the order is the workspace's second part, behind the control block's 256 bytes
+    order = ws.buf[256:256 + nq * nprobe * 4].view(torch.int32).view(nq, nprobe)
+    order.fill_(-1)
+    st = sieve.search(*args, workspace=ws, stats=True)[4]
+    got = order.cpu().numpy()
+    print(f"\nprefix under adversarial rounding, d = {d}: {st['extended']} of {nq} queries extended")
+    assert st["extended"] >= 0 and (got[:, :8] >= 0).all()
+    tol = 1e-6 * np.abs(exact).max()
+    for i in range(nq):
+        ids = got[i][got[i] >= 0]
+        e = exact[i, ids]
+        assert len(set(ids.tolist())) == len(ids)
+        assert (np.diff(e) <= tol).all()
+        rest = np.delete(exact[i], ids)
+        assert rest.max() <= e.min() + tol

@@ -61,7 +61,7 @@ def unit(v):
     return v / np.linalg.norm(v, axis=-1, keepdims=True)
 
 
-@pytest.mark.parametrize("d", [4, 32, 96, 256])
+@pytest.mark.parametrize("d", [4, 32, 96, 256, 260, 512])
 def test_bound_holds_on_random_unit_vectors(d):
     rng = np.random.default_rng(d)
     q = unit(rng.standard_normal((3000, d))).astype(np.float32)
@@ -70,7 +70,7 @@ def test_bound_holds_on_random_unit_vectors(d):
     assert worst_ratio(q, x) < 1.0
 
 
-@pytest.mark.parametrize("d", [64, 256])
+@pytest.mark.parametrize("d", [64, 256, 512])
 def test_bound_holds_on_other_norms(d):
     rng = np.random.default_rng(100 + d)
     q = (unit(rng.standard_normal((3000, d))) * rng.uniform(0.05, 20, (3000, 1))).astype(np.float32)
