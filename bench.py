@@ -164,7 +164,9 @@ _SCAN_SOURCES = ("common.cuh", "search.cuh", "scan_tc.cu", "tcgen05.cuh", "tc_bu
                  "tc_pipeline.cuh", "tc_layout.cu", "rq.cu")
 _RANK_SOURCES = ("common.cuh", "search.cuh", "rank_tc.cu", "tcgen05.cuh", "tc_bulk.cuh",
                  "tc_pipeline.cuh", "tc_layout.cu")
-KERNEL_SOURCES = {"k_scan_bulk": _SCAN_SOURCES, "k_scan_rq": _SCAN_SOURCES,
+_PREFIX_SOURCES = ("common.cuh", "search.cuh", "rank_prefix.cu", "rank_select.cuh", "tcgen05.cuh",
+                   "tc_bulk.cuh", "tc_pipeline.cuh", "tc_layout.cu")
+KERNEL_SOURCES = {"k_prefix_scan": _PREFIX_SOURCES, "k_scan_bulk": _SCAN_SOURCES, "k_scan_rq": _SCAN_SOURCES,
                   "k_scan_screen": _SCAN_SOURCES, "k_rank_bulk + k_rank_screen": _RANK_SOURCES}
 
 

@@ -284,6 +284,10 @@ def test_an_extension_takes_no_round_of_its_own(dev, lookahead, nq, d, nlist, W)
         assert got[4]["extended"] > 0
         assert got[4]["rounds"] == want[4]["rounds"]
         assert got[4]["items"] == want[4]["items"]
+        # rounds cut short by a cap defer queries, listed ones among them
+        cut = sieve.search(ix, Q, 0.9, 10, 64, W, loop=loop, max_items_per_round=nq + 7, **kw)
+        for x, y in zip(cut[:4], got[:4]):
+            assert torch.equal(x, y)
 
 
 @pytest.mark.parametrize("nq,tau,prefix", [(1_000, 0.85, True), (1_000, 0.84, False), (16_383, 0.84, False),
