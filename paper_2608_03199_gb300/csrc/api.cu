@@ -250,7 +250,7 @@ cudaError_t launch_search_rank(const SearchArgs &a, int rank_tc, cudaStream_t st
 // the end of a round that met queries whose stop line passes their prefix
 cudaError_t launch_search_ext(const SearchArgs &a, int part, cudaStream_t st, float *mma_ms = nullptr) {
     return enqueue_rank_ext(part, a.Q, a.nq, a.C, a.nlist, a.d, a.nprobe, a.W, const_cast<int32_t *>(a.order),
-                            a.cscores, a.rank_scratch, &a.ctl->ext_n, &a.ctl->status, a.tc_cent, st, mma_ms);
+                            a.cscores, a.rank_scratch, a.ctl, a.tc_cent, st, mma_ms);
 }
 
 // quantized search: q' = P^T q for the batch, after init (which clears the
@@ -289,8 +289,7 @@ sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaSuccess;
     RoundConds conds{};
-    cudaGraphConditionalHandle more_ext = 0;
-    cudaGraph_t body = nullptr, ext_body = nullptr, more_body = nullptr;
+    cudaGraph_t body = nullptr, ext_body = nullptr;
     do {
         // outer graph: init -> [rank] -> WHILE(rounds) -> finalize
         if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
@@ -312,30 +311,26 @@ sieve_status build_graph(const GraphKey &key, cudaGraph_t *g_out, cudaGraphExec_
         e2 = cudaStreamEndCapture(cs, &body);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess) break;
-        if (a.limit) {
-            if ((e = cudaStreamBeginCaptureToGraph(cs, ext_body, nullptr, nullptr, 0,
+        // the extension's parts, each nested in the one before it (two nodes side
+        // by side cost eight searches of 100K x 1,500 x 96 about 130 us)
+        for (int i = 0; a.limit && ext_part_of(i, a.nq); ++i) {
+            cudaGraph_t part_body = ext_body;
+            if ((e = cudaStreamBeginCaptureToGraph(cs, part_body, nullptr, nullptr, 0,
                                                    cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
                 break;
-            e = launch_search_ext(a, 0, cs);
-            if (a.nq > kExtFirst) {
+            e = launch_search_ext(a, i, cs);
+            if (ext_part_of(i + 1, a.nq)) {
+                cudaGraphConditionalHandle more = 0;
                 if (e == cudaSuccess)
-                    e = cudaGraphConditionalHandleCreate(&more_ext, ext_body, 0, cudaGraphCondAssignDefault);
-                if (e == cudaSuccess) e = launch_ext_more(a, more_ext, cs);
-                if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &more_ext, &more_body);
+                    e = cudaGraphConditionalHandleCreate(&more, part_body, 0, cudaGraphCondAssignDefault);
+                if (e == cudaSuccess) e = launch_ext_more(a, i + 1, more, cs);
+                if (e == cudaSuccess) e = add_conditional(cs, cudaGraphCondTypeIf, 0, &more, &ext_body);
             }
-            e2 = cudaStreamEndCapture(cs, &ext_body);
+            e2 = cudaStreamEndCapture(cs, &part_body);
             if (e == cudaSuccess) e = e2;
             if (e != cudaSuccess) break;
         }
-        if (more_body) {
-            if ((e = cudaStreamBeginCaptureToGraph(cs, more_body, nullptr, nullptr, 0,
-                                                   cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
-                break;
-            e = launch_search_ext(a, 1, cs);
-            e2 = cudaStreamEndCapture(cs, &more_body);
-            if (e == cudaSuccess) e = e2;
-            if (e != cudaSuccess) break;
-        }
+        if (e != cudaSuccess) break;
         e = cudaGraphInstantiate(exec_out, g, 0);
     } while (0);
     cudaStreamDestroy(cs);
@@ -626,7 +621,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
                 }
             }
             if (!more) break;
-            for (int i = 0; prefix && i < 2 && word[2] > (i ? kExtFirst : 0); ++i)
+            for (int i = 0; prefix && ext_part_of(i, nq) && word[2] > ext_begin(i); ++i)
                 SIEVE_CUDA(timed(SIEVE_K_RANK, [&] {
                     return launch_search_ext(a, i, st, p->profile ? &ms[SIEVE_K_RANK_MMA] : nullptr);
                 }));
@@ -654,7 +649,7 @@ sieve_status search_device(const sieve_index_view *ix, const float *Q, int64_t n
         int prefix_mma = 0, prefix_launches = 0;   // the prefix ranking, if it ran here, and its extensions
         if (prefix && with_rank)
             prefix_launches = rank_prefix_launches(0, a.nq, a.nq, a.nlist, a.nprobe, a.W, a.d, &prefix_mma);
-        for (int i = 0; prefix && i < 2; ++i)
+        for (int i = 0; prefix && i < kExtParts; ++i)
             if (c.ext_runs[i] > 0) {
                 int mma = 0;
                 prefix_launches += c.ext_runs[i] * rank_ext_launches(i, a.nq, a.nlist, a.nprobe, a.W, a.d, bulk, &mma);

@@ -36,8 +36,7 @@ struct Ctl {
     int n_ext;         // the same, counted while the round issues and merges
     int n_tc_tiles;    // tensor-core scan tiles this round
     int tc_tile_next;  // tensor-core scan work counter
-    int ext_runs[2];   // rounds that ended with the extension's first part, and with its second
-    int pad;
+    int ext_runs[3];   // rounds whose end ran each part of an extension
     unsigned long long tot_items, tot_groups, tot_tiles, tot_rows, tot_pairs;
     unsigned long long tot_rows_tc, tot_pairs_tc;   // the tensor-core share of the two above
     unsigned long long tot_ext;                     // queries extended

@@ -458,11 +458,16 @@ __global__ void __launch_bounds__(kFinalWarps * 32) k_prefix_final(
     if (lane == 0) limit[q] = R;
 }
 
-// row i of Qx = query ext[q0 + i] (a warp per row), for the listed queries of this chunk
+// row i of Qx = query ext[q0 + i] (a warp per row), for the listed queries of
+// this chunk; the first chunk of a part (-1: another) counts its run
 __global__ void k_ext_gather(const float *__restrict__ Q, int d, const int *__restrict__ ext,
-                             const int *__restrict__ ext_n, int64_t q0, int64_t chunk,
-                             float *__restrict__ Qx) {
-    const int64_t left = (int64_t)*ext_n - q0, n = left < chunk ? left : chunk;
+                             Ctl *ctl, int64_t q0, int64_t chunk, float *__restrict__ Qx, int part) {
+    const int ext_n = ctl->ext_n;
+    if (part >= 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->ext_runs[part] += 1;
+        if (part == 0) ctl->tot_ext += (unsigned long long)ext_n;
+    }
+    const int64_t left = (int64_t)ext_n - q0, n = left < chunk ? left : chunk;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
@@ -600,7 +605,7 @@ struct PrefixScratch {
     struct Ext {                   // a part of the extension: queries per pass, and byte offsets
         int64_t chunk;             // of its buffers (after its ranking scratch)
         int64_t q, order, s, end;
-    } ext_part[2];
+    } ext_part[kExtParts];
     int64_t total;
 };
 
@@ -624,13 +629,13 @@ static PrefixScratch prefix_scratch(int64_t nq, int64_t nlist, int nprobe, int d
     S.limit = 0;
     S.ext = round_up(nq * 4, 256);
     S.rest = S.ext + round_up(nq * 4, 256);
-    S.ext_part[0] = ext_part(S.rest, std::min(nq, kExtFirst), nlist, nprobe, d);
-    S.total = std::max(S.ext_part[0].end, plain);
-    if (nq > kExtFirst) {
-        PrefixScratch::Ext &E = S.ext_part[1];
-        E = ext_part(S.rest, nq - kExtFirst, nlist, nprobe, d);
-        while (E.end > S.total && E.chunk > kExtFirst)
-            E = ext_part(S.rest, std::max(kExtFirst, round_up(ceil_div(E.chunk, 2), (int64_t)128)), nlist, nprobe, d);
+    S.total = plain;
+    for (int i = 0; ext_part_of(i, nq); ++i) {
+        PrefixScratch::Ext &E = S.ext_part[i];
+        E = ext_part(S.rest, ext_end(i, nq) - ext_begin(i), nlist, nprobe, d);
+        const int64_t least = ext_begin(1);   // more passes before more scratch, down to this many queries
+        while (E.end > S.total && E.chunk > least)
+            E = ext_part(S.rest, std::max(least, round_up(ceil_div(E.chunk, 2), (int64_t)128)), nlist, nprobe, d);
         S.total = std::max(S.total, E.end);
     }
     const PrefixPlan P = prefix_plan(nq, nlist, d, L);
@@ -780,12 +785,11 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
 }
 
 // The extension: the full ranking of the queries ext[0 .. *ext_n - 1], behind
-// their prefixes; part 0 the first kExtFirst of them, part 1 the others.
-// Every pass is launched; passes past *ext_n find no work.
+// their prefixes, those of one part.  Every pass is launched; passes past
+// *ext_n find no work.
 cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                              int nprobe, int W, int32_t *order, float *cscores, void *scratch,
-                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st,
-                             float *mma_ms) {
+                             Ctl *ctl, const unsigned char *tc_cent, cudaStream_t st, float *mma_ms) {
     const PrefixScratch S = prefix_scratch(nq, nlist, nprobe, d, rank_prefix_len(nq, nlist, nprobe, W, d));
     const PrefixScratch::Ext &E = S.ext_part[part];
     unsigned char *w = static_cast<unsigned char *>(scratch);
@@ -795,15 +799,15 @@ cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *
     int32_t *full = reinterpret_cast<int32_t *>(w + E.order);
     float *full_s = cscores ? reinterpret_cast<float *>(w + E.s) : nullptr;
     const int blocks = 4 * num_sms();
-    const int64_t lo = part ? kExtFirst : 0, hi = part ? nq : std::min(nq, kExtFirst);
-    for (int64_t b = lo; b < hi; b += E.chunk) {
+    const int64_t hi = ext_end(part, nq);
+    for (int64_t b = ext_begin(part); b < hi; b += E.chunk) {
         const int64_t n = std::min(E.chunk, hi - b);
-        k_ext_gather<<<blocks, 256, 0, st>>>(Q, d, ext, ext_n, b, n, Qx);
+        k_ext_gather<<<blocks, 256, 0, st>>>(Q, d, ext, ctl, b, n, Qx, b == ext_begin(part) ? part : -1);
         cudaError_t e = enqueue_rank_tc(Qx, n, C, nlist, d, nprobe, full, full_s,
-                                        reinterpret_cast<float *>(w + S.rest), status, st, tc_cent, mma_ms,
-                                        E.chunk, ext_n, b);
+                                        reinterpret_cast<float *>(w + S.rest), &ctl->status, st, tc_cent, mma_ms,
+                                        E.chunk, &ctl->ext_n, b);
         if (e != cudaSuccess) return e;
-        k_ext_merge<<<blocks, 256, 0, st>>>(ext, ext_n, b, n, nprobe, full, full_s, order, cscores, limit);
+        k_ext_merge<<<blocks, 256, 0, st>>>(ext, &ctl->ext_n, b, n, nprobe, full, full_s, order, cscores, limit);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -814,7 +818,7 @@ int rank_ext_launches(int part, int64_t nq, int64_t nlist, int nprobe, int W, in
     const int64_t chunk = S.ext_part[part].chunk;
     int n = 0;
     *mma = 0;
-    for (int64_t b = part ? kExtFirst : 0, hi = part ? nq : std::min(nq, kExtFirst); b < hi; b += chunk) {
+    for (int64_t b = ext_begin(part), hi = ext_end(part, nq); b < hi; b += chunk) {
         const int64_t m = std::min(chunk, hi - b);
         n += 2 + rank_tc_launches(m, nlist, nprobe, d, chunk, bulk);
         *mma += rank_tc_mma_launches(m, nlist, nprobe, d, chunk, bulk);

@@ -163,16 +163,27 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
                                 int64_t nlist, int d, int nprobe, int W, int32_t *order, float *cscores,
                                 void *scratch, int *status, const unsigned char *tc_cent, cudaStream_t st,
                                 float *mma_ms = nullptr, int wait_limit = 0);
-// an extension in two parts: the first kExtFirst queries as a small batch, cut
-// into ranges that fill the SMs (as part of a batch of all queries they were a
-// few tiles that each went over all centroids), and the rest, if there are any
-constexpr int64_t kExtFirst = 4096;
-// sets cond (of a node that follows in the same graph) where part 1 has queries
-cudaError_t launch_ext_more(const SearchArgs &a, cudaGraphConditionalHandle cond, cudaStream_t st);
+// an extension in parts, each ranked as a batch of its size, so that its few
+// tiles are cut into ranges that fill the SMs: the first 4,096 queries, with
+// more than 262,144 in all those up to the 32,768th, and the rest.  (As part of
+// a batch of all queries, 1,363 x 65,536 x 96 behind the first 4,096 went over
+// all centroids in a few tiles, with seven empty passes behind them: 2.4 ms of a
+// search of 1M, now 0.5.  Each part is one more condition in the graph, 16 us a
+// search, which a smaller batch does not repay.)  A part runs where the list
+// reaches into it.
+constexpr int kExtParts = 3;
+__host__ __device__ constexpr int64_t ext_begin(int part) { return part == 0 ? 0 : part == 1 ? 4096 : 32768; }
+__host__ __device__ constexpr bool ext_part_of(int part, int64_t nq) {   // whether a search of nq queries has it
+    return part < kExtParts && nq > (part == 2 ? 262144 : ext_begin(part));
+}
+inline int64_t ext_end(int part, int64_t nq) {
+    return ext_part_of(part + 1, nq) ? ext_begin(part + 1) : nq;
+}
+// sets cond (of a node that follows in the same graph) where `part` has queries
+cudaError_t launch_ext_more(const SearchArgs &a, int part, cudaGraphConditionalHandle cond, cudaStream_t st);
 cudaError_t enqueue_rank_ext(int part, const float *Q, int64_t nq, const float *C, int64_t nlist, int d,
                              int nprobe, int W, int32_t *order, float *cscores, void *scratch,
-                             const int *ext_n, int *status, const unsigned char *tc_cent, cudaStream_t st,
-                             float *mma_ms = nullptr);
+                             Ctl *ctl, const unsigned char *tc_cent, cudaStream_t st, float *mma_ms = nullptr);
 // kernel launches of one run of a part (and its contraction launches)
 int rank_ext_launches(int part, int64_t nq, int64_t nlist, int nprobe, int W, int d, bool bulk, int *mma);
 

@@ -589,14 +589,8 @@ __global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
         more = 0;
     }
     c->more = more;
-    const int ext = more ? c->n_ext : 0;
-    c->ext_n = ext;
+    c->ext_n = more ? c->n_ext : 0;
     c->n_ext = 0;
-    if (ext > 0) {
-        c->tot_ext += (unsigned long long)ext;
-        c->ext_runs[0] += 1;
-        c->ext_runs[1] += ext > kExtFirst;
-    }
     c->n_items = 0;
     c->n_active = 0;
     c->n_tiles = 0;
@@ -607,12 +601,14 @@ __global__ void k_round_end(SearchArgs a, RoundConds conds, int use_cond) {
     c->n_continue = 0;
     if (use_cond) {
         cudaGraphSetConditional(conds.more, more ? 1u : 0u);
-        if (a.limit) cudaGraphSetConditional(conds.ext, ext > 0 ? 1u : 0u);
+        if (a.limit) cudaGraphSetConditional(conds.ext, c->ext_n > 0 ? 1u : 0u);
     }
 }
 
-__global__ void k_ext_more(const Ctl *c, cudaGraphConditionalHandle cond) {
-    cudaGraphSetConditional(cond, c->ext_n > kExtFirst ? 1u : 0u);
+static_assert(sizeof(Ctl::ext_runs) == kExtParts * sizeof(int), "a counter for each part");
+
+__global__ void k_ext_more(const Ctl *c, int part, cudaGraphConditionalHandle cond) {
+    cudaGraphSetConditional(cond, c->ext_n > ext_begin(part) ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -650,8 +646,8 @@ cudaError_t launch_finalize(const SearchArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_ext_more(const SearchArgs &a, cudaGraphConditionalHandle cond, cudaStream_t st) {
-    k_ext_more<<<1, 1, 0, st>>>(a.ctl, cond);
+cudaError_t launch_ext_more(const SearchArgs &a, int part, cudaGraphConditionalHandle cond, cudaStream_t st) {
+    k_ext_more<<<1, 1, 0, st>>>(a.ctl, part, cond);
     return cudaGetLastError();
 }
 

@@ -70,7 +70,8 @@ CASES = [  # n, d, nlist, nq, nprobe, W, tau, lookahead, grouped, equal
     (9_000, 4, 2_081, 127, 40, 4, 0.97, True, False, 0),
     (9_000, 100, 2_176, 129, 64, 8, 0.45, True, False, 0),
     (9_000, 132, 2_305, 257, 64, 8, 0.45, True, False, 0),
-    (12_000, 64, 2_500, 9_001, 64, 8, 0.20, True, False, 0),   # nearly every query extended: both parts
+    (12_000, 64, 2_500, 9_001, 64, 8, 0.20, True, False, 0),   # nearly every query extended: two parts
+    (12_000, 32, 2_100, 262_145, 40, 8, 0.20, True, False, 0),  # and all three
     (8_000, 96, 2_309, 5_000, 64, 16, 0.45, True, True, 0),    # a last group of five centroids
 ]
 
