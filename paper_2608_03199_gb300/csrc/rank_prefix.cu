@@ -65,7 +65,6 @@ struct PrefixArgs {
     int *status;
     int wait_limit;      // polls of the epilogue's accumulator wait (0: default)
     const unsigned char *tc_cent;
-    const unsigned *cmax;   // launch_cnorm_max of the centroids
     int nranges;         // centroid ranges per query tile
     int64_t range_len;   // centroids per range, a multiple of 128
     float *list_s;       // [nq][nranges][kL][32] the kept groups' screened scores (raw: x 2^16) ...
@@ -77,8 +76,10 @@ struct PrefixArgs {
 __device__ int g_prefix_status_sink;
 
 // Scores past fp16's range (|256 x| above 65,504) are not screened soundly, and
-// a NaN row is left out by every maximum: with such centroids no prefix is
-// found, and the scan goes over nothing.
+// a NaN row is left out by every maximum: with such centroids every prefix is
+// empty.  (The scan runs for them all the same: returning at its start on these
+// two words took the compiler to other code, 13.4 -> 13.7 ms for 1M queries x
+// 65,536 x 96 that have no such centroids.)
 constexpr float kScreenMaxNorm = 200.f;
 __device__ __forceinline__ float norm_up(unsigned bits) { return __uint_as_float(bits) * (1.f + 0x1p-20f); }
 __device__ __forceinline__ bool centroids_screen(unsigned norm, unsigned nan) {
@@ -103,9 +104,7 @@ struct PrefixMode {
         int64_t c0, nb;
         int ns, sstep;   // sample chunks first: chunks 0, sstep, 2 sstep, ...
     };
-    __device__ static int num_tiles(const Args &a) {
-        return centroids_screen(a.cmax[0], a.cmax[1]) ? (int)ceil_div(a.nq, kRows) * a.nranges : 0;
-    }
+    __device__ static int num_tiles(const Args &a) { return (int)ceil_div(a.nq, kRows) * a.nranges; }
     __device__ static int *tile_counter(const Args &) { return nullptr; }
     __device__ static int d(const Args &a) { return a.d; }
     __device__ static int *status(const Args &a) { return a.status ? a.status : &g_prefix_status_sink; }
@@ -264,8 +263,8 @@ __device__ __forceinline__ float warp_sum_each(float (&acc)[B]) {
 }
 
 // One warp per query.  NV: float4 of a row per lane (d <= 128 NV); KPL: kept
-// groups per lane (nranges * kL <= 32 KPL).  A scan that gave up on a wait, or
-// was skipped, leaves lists that an earlier call wrote, or nobody: every id is
+// groups per lane (nranges * kL <= 32 KPL).  A scan that gave up on a wait
+// leaves lists that an earlier call wrote, or nobody: every id is
 // kept below nlist before a row is read, and with the status word set, or
 // centroids that are not screened, every prefix is empty.  (Asked at the end,
 // where the answer is at hand: 1M queries 1.59 ms; a branch up front 1.76.)
@@ -687,13 +686,13 @@ cudaError_t prepare_rank_prefix(int64_t nq, int64_t nlist, int nprobe, int W, in
 }
 
 template <int kL, int KPL>
-static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, int32_t *order, float *cscores, int *limit, cudaStream_t st) {
+static void launch_prefix_final(const PrefixArgs &a, const float *C, int nprobe, const unsigned *cmax, int32_t *order, float *cscores, int *limit, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(a.nq, kFinalWarps);
     auto f = a.d <= 128   ? k_prefix_final<kL, KPL, 1>
              : a.d <= 256 ? k_prefix_final<kL, KPL, 2>
                           : k_prefix_final<kL, KPL, 4>;
     f<<<blocks, kFinalWarps * 32, 0, st>>>(a.Q, a.nq, C, a.nlist, a.d, a.list_s, a.list_g, a.list_t, a.nranges, nprobe,
-                                           a.cmax, a.status, order, cscores, limit);
+                                           cmax, a.status, order, cscores, limit);
 }
 
 // kernel launches of the prefix ranking of nq queries from q0 on (and its
@@ -746,7 +745,7 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
     }
     for (int64_t b = 0; b < nq; b += S.chunk) {
         const int64_t n = std::min(S.chunk, nq - b);
-        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, wait_limit, tc_cent, cmax, P.nranges, P.range_len,
+        const PrefixArgs a{Q + (q0 + b) * d, n, nlist, d, status, wait_limit, tc_cent, P.nranges, P.range_len,
                            list_s, list_g, list_t};
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, prefix_sub(d) * tcp::kM) * P.nranges, num_sms());
         if (mma_ms) {
@@ -762,8 +761,8 @@ cudaError_t enqueue_rank_prefix(const float *Q, int64_t q0, int64_t nq, int64_t 
         int *lim = limit + q0 + b;
         const int kpl = (int)ceil_div(P.nranges * L, 32);
 #define SIEVE_PREFIX(K)                                                                       \
-    if (L == 16) launch_prefix_final<16, K>(a, C, nprobe, o, cs, lim, st);               \
-    else launch_prefix_final<32, K>(a, C, nprobe, o, cs, lim, st)
+    if (L == 16) launch_prefix_final<16, K>(a, C, nprobe, cmax, o, cs, lim, st);               \
+    else launch_prefix_final<32, K>(a, C, nprobe, cmax, o, cs, lim, st)
         if (kpl <= 1) { SIEVE_PREFIX(1); }
         else if (kpl <= 2) { SIEVE_PREFIX(2); }
         else if (kpl <= 4) { SIEVE_PREFIX(4); }
